@@ -520,6 +520,7 @@ ec_status rle_job_desc(const ec_rle_job& j, bool compress, RleJobDesc* d)
     d->w = j.w;
     d->h = j.h;
     d->pitch = j.pitch;
+    d->winv = rle_winv(j.w);
     d->n_chunks = (uint32_t)((n + EC_RLE_CHUNK - 1) / EC_RLE_CHUNK);
     if (compress) {
         if (j.mode > 2) return EC_ERR_INVALID_ARG;
@@ -535,7 +536,9 @@ ec_status rle_job_desc(const ec_rle_job& j, bool compress, RleJobDesc* d)
         if (!j.src || (reinterpret_cast<uintptr_t>(j.src) & 3u)) return EC_ERR_INVALID_ARG;
         if (n > 0 && (reinterpret_cast<uintptr_t>(j.dst) & 3u)) return EC_ERR_INVALID_ARG;
         d->capacity = j.capacity;
-        d->vec = aligned16(j.dst) && j.w % 4 == 0 && j.pitch % 4 == 0;
+        // 16-byte stores: rows of whole 16-byte groups, or one contiguous run
+        // (whose last elements, where 4 does not divide it, are written singly)
+        d->vec = aligned16(j.dst) && ((j.w % 4 == 0 && j.pitch % 4 == 0) || j.pitch == j.w);
     }
     return EC_OK;
 }

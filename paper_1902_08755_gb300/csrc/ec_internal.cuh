@@ -164,9 +164,11 @@ struct RleJobDesc {
     uint32_t n_chunks;     // ceil(w*h / 4096)
     uint32_t first_unit;   // first global work unit of this job
     uint32_t vec;          // 16-byte element loads/stores allowed
-    uint32_t pad;
+    uint32_t winv;         // floor((2^32 - 1) / w): rows of elements without divisions (0 if w is 0)
 };
 static_assert(sizeof(RleJobDesc) == 64, "rle job layout");
+
+inline uint32_t rle_winv(int32_t w) { return w > 0 ? 0xFFFFFFFFu / (uint32_t)w : 0u; }
 
 // At most kRleJobsPerLaunch jobs travel in one launch's parameters; larger
 // batches are split into several launches.

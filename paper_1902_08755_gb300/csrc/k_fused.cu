@@ -210,7 +210,6 @@ k_fused_depth(const FusedStage* __restrict__ stages, const FusedUnit* __restrict
 {
     __shared__ __align__(16) uint8_t planes[8][kChunk];
     __shared__ __align__(16) uint32_t staged[2][kStageWords];
-    __shared__ uint8_t s_hdr[2][rlec::kHdrBytes];
     __shared__ uint32_t s_beg[2][5];
     __shared__ int s_mode[2];
     __shared__ int s_fail, s_over;
@@ -231,22 +230,19 @@ k_fused_depth(const FusedStage* __restrict__ stages, const FusedUnit* __restrict
     // header bytes are read within the streams' capacity, in parallel with
     // their sizes; the validation then uses the sizes
     const uint64_t csz = *u.csize, dsz = *u.dsize;
-    if (tid < rlec::kHdrBytes) s_hdr[0][tid] = rlec::header_byte(u.cs, (uint64_t)u.cap, nc, u.chunk, tid);
-    else if (tid >= 64 && tid < 64 + rlec::kHdrBytes)
-        s_hdr[1][tid - 64] = rlec::header_byte(u.ds, (uint64_t)u.cap, nc, u.chunk, tid - 64);
-    if (tid == 0) { s_fail = 0; s_over = 0; }
     // the run bitmaps (aliased with the planes) start empty
     uint32_t* bm = reinterpret_cast<uint32_t*>(&planes[0][0]);       // [8][128] run starts per plane
     for (int i = tid; i < 8 * 128; i += kFT) bm[i] = 0u;
-    __syncthreads();
-    if (tid == 0 || tid == 32) {
-        const int k = tid >> 5;
-        if (rlec::check_header(s_hdr[k], k ? dsz : csz, (uint32_t)u.w, (uint32_t)u.h, nc, u.chunk,
-                               s_beg[k], &s_mode[k]))
-            s_fail = 1;
+    // warps 0-3 check the colour stream, 4-7 the depth stream
+    const rlec::ChunkEnds E = warp < 4
+        ? rlec::check_chunk(u.cs, u.cap, csz, (uint32_t)u.w, (uint32_t)u.h, nc, u.chunk, false)
+        : rlec::check_chunk(u.ds, u.cap, dsz, (uint32_t)u.w, (uint32_t)u.h, nc, u.chunk, false);
+    if ((warp & 3) == 0) {
+        if (lane >= 8 && lane < 13) s_beg[warp >> 2][lane - 8] = E.v;
+        if (lane == 0) s_mode[warp >> 2] = E.mode;
     }
-    __syncthreads();
-    if (s_fail) {
+    if (tid == 0) { s_fail = 0; s_over = 0; }
+    if (__syncthreads_or(E.bad)) {
         if (tid == 0) set_status(status, EC_ERR_CORRUPT);
         return;
     }
@@ -337,12 +333,8 @@ k_fused_depth(const FusedStage* __restrict__ stages, const FusedUnit* __restrict
     // many runs: decode the planes into shared memory
     {
         const int k = warp >> 2, p = warp & 3;
-        const int b = (int)s_beg[k][p], e = (int)s_beg[k][p + 1];
-        const int w0 = k ? dw0 : cw0, nw = k ? dnw : cnw;
-        const int bad = nw <= kStageWords
-            ? rlec::decode_plane(rlec::SharedBytes{reinterpret_cast<const uint8_t*>(staged[k]), 4 * w0},
-                                 b, e, len, planes[warp], lane)
-            : rlec::decode_plane(rlec::GlobalBytes{k ? dpay : cpay}, b, e, len, planes[warp], lane);
+        const int bad = rlec::decode_plane_dense(rlec::GlobalWords{k ? dpay : cpay}, (int)s_beg[k][p],
+                                                 (int)s_beg[k][p + 1], len, planes[warp], lane);
         if (bad && lane == 0) s_fail = 1;
     }
     __syncthreads();

@@ -21,14 +21,12 @@
 //      entries; the dense chunks coded again, straight to their place.
 // Every wait (the copies into shared memory) is bounded (EC_ERR_TIMEOUT).
 //
-// Decompress: one CTA of four warps per chunk.  The header and the chunk's
-// end-table entries are fetched in one round trip and validated.  Warp p
-// decodes plane p in windows of 32 stream bytes: the jump from each byte to
-// the token after one starting there is composed by doubling, so lane t holds
-// the window's t-th token; a warp scan places the tokens, each is checked
-// against its stream and chunk bounds, lanes write the unaligned ends of their
-// repeat tokens and short aligned bodies, the warp a long body per store.  The four
-// planes are then transposed back into elements with byte permutes.
+// Decompress: one CTA of four warps per chunk.  Every warp fetches the header
+// and the chunk's end-table entries in one round trip and validates them.
+// Warp p walks plane p's tokens; each is checked against its stream and chunk bounds.  A
+// chunk of few runs is written from the runs' starts and bytes (16-byte stores
+// of constant groups); the planes of the others are decoded into shared memory
+// and transposed back into elements with byte permutes.
 #include "ec_internal.cuh"
 #include "rle_codec.cuh"
 
@@ -45,7 +43,6 @@ constexpr int kSpinLimit = 1 << 20;            // tries of a bounded mbarrier wa
 
 using rlec::swizzle;
 using rlec::transpose4;
-using rlec::bcast8;
 
 template <int N>
 __device__ __forceinline__ int find_job(const RleJobList<N>& J, uint32_t unit)
@@ -65,10 +62,19 @@ __device__ __forceinline__ void put_u32(uint8_t* p, uint32_t v)
 }
 
 
+// Row of element q: q / w from the reciprocal winv = floor((2^32 - 1) / w).
+// q winv / 2^32 lies in (q / w - 2 q / 2^32, q / w], and q < 2^27, so its floor
+// is the quotient or one less.
+__device__ __forceinline__ uint32_t row_of(const RleJobDesc& jb, uint32_t q)
+{
+    const uint32_t y = __umulhi(q, jb.winv);
+    return q - y * (uint32_t)jb.w >= (uint32_t)jb.w ? y + 1u : y;
+}
+
 // Element q of a job's image.
 __device__ __forceinline__ size_t elem_off(const RleJobDesc& jb, uint32_t q)
 {
-    const uint32_t y = q / (uint32_t)jb.w;
+    const uint32_t y = row_of(jb, q);
     return (size_t)y * jb.pitch + (q - y * (uint32_t)jb.w);
 }
 
@@ -236,13 +242,12 @@ __device__ __forceinline__ uint4 load_elems(const RleJobDesc& jb, uint32_t q0, i
     if (jb.vec) {
         size_t e = q0 + (uint32_t)q;
         if (jb.pitch != jb.w) {
-            const uint32_t y = (q0 + (uint32_t)q) / w;
-            e = (size_t)y * jb.pitch + (q0 + (uint32_t)q - y * w);
+            e = elem_off(jb, q0 + (uint32_t)q);
         }
         return __ldg(reinterpret_cast<const uint4*>(jb.src + e));
     }
     uint32_t v[4];
-    uint32_t y = (q0 + (uint32_t)q) / w, x = q0 + (uint32_t)q - y * w;
+    uint32_t y = row_of(jb, q0 + (uint32_t)q), x = q0 + (uint32_t)q - y * w;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         v[k] = q + k < len ? __ldg(jb.src + (size_t)y * jb.pitch + x) : 0u;
@@ -288,7 +293,7 @@ __device__ void issue_quarter(const RleJobDesc& jb, uint32_t unit, int qi, int s
     uint32_t* dst = W.buf[slot] + 4;
     const uint32_t w = (uint32_t)jb.w;
     if (!jb.vec) {
-        uint32_t y = (qs + (uint32_t)lane) / w, x = qs + (uint32_t)lane - y * w;
+        uint32_t y = row_of(jb, qs + (uint32_t)lane), x = qs + (uint32_t)lane - y * w;
         for (int i = lane; i < qlen; i += 32) {
             cp_async4(dst + i, jb.src + (size_t)y * jb.pitch + x);
             x += 32u;
@@ -305,7 +310,7 @@ __device__ void issue_quarter(const RleJobDesc& jb, uint32_t unit, int qi, int s
         if (lane == 0) bulk_load(dst, jb.src + qs, 4u * (uint32_t)qlen, &W.full[slot]);
         return;
     }
-    const uint32_t y0 = qs / w, y1 = (qs + (uint32_t)qlen - 1u) / w;
+    const uint32_t y0 = row_of(jb, qs), y1 = row_of(jb, qs + (uint32_t)qlen - 1u);
     for (uint32_t y = y0 + (uint32_t)lane; y <= y1; y += 32) {
         const uint32_t a = y == y0 ? qs - y0 * w : 0u;                   // first column of the segment
         const uint32_t b = min(w, qs + (uint32_t)qlen - y * w);          // its end column
@@ -1399,7 +1404,7 @@ __device__ void decode_mode0(const RleJobDesc& jb, const uint8_t* pay, uint32_t 
     const uint8_t* sb = sbuf - 4u * w0;                // stream byte i at sb[i]
     const uint32_t* sw = st - w0;                      // stream word j (bytes 4j .. 4j+3) at sw[j]
     uint32_t* dst = reinterpret_cast<uint32_t*>(jb.dst);
-    const bool pairs = jb.vec != 0u;                   // rows 16-byte aligned: a unit never straddles rows
+    const bool pairs = jb.vec != 0u;                   // a unit's elements are adjacent, 8-byte aligned
     const bool dense = jb.pitch == jb.w;
     const uint32_t nu = (uint32_t)len / 2u;
     for (;;) {
@@ -1431,11 +1436,7 @@ __device__ void decode_mode0(const RleJobDesc& jb, const uint8_t* pay, uint32_t 
                 const uint32_t lo = __funnelshift_r(a0, a1, sh), hi = __funnelshift_r(a1, a2, sh);
                 const uint32_t q = q0 + 2u * (o + k);
                 if (pairs) {
-                    size_t eo = q;
-                    if (!dense) {
-                        const uint32_t y = q / (uint32_t)jb.w;
-                        eo = (size_t)y * jb.pitch + (q - y * (uint32_t)jb.w);
-                    }
+                    const size_t eo = dense ? q : elem_off(jb, q);
                     __stcs(reinterpret_cast<uint2*>(dst + eo), make_uint2(lo, hi));
                 } else {
                     dst[elem_off(jb, q)] = lo;
@@ -1470,15 +1471,14 @@ __device__ void decode_mode0(const RleJobDesc& jb, const uint8_t* pay, uint32_t 
 // val: their run bytes [4][256]; work: shared scratch of kRunArea bytes
 // (bitmaps included).
 constexpr int kRunCap = 255;                        // runs per plane the run path takes
-constexpr int kRunArea = 2048 + 3 * 512;            // bitmaps, union, two prefix arrays
+constexpr int kRunArea = 2048 + 1024 + 64;          // bitmaps, union with its prefix, warp totals
 
-__device__ void fill_segments(const RleJobDesc& jb, uint32_t q0, int len, bool sw, const uint32_t* bm,
-                              const uint8_t* val, uint8_t* work, uint32_t* dstp)
+__device__ __forceinline__ void fill_segments(const RleJobDesc& jb, uint32_t q0, int len, bool sw, const uint32_t* bm,
+                                              const uint8_t* val, uint8_t* work, uint32_t* dstp)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint32_t* U = reinterpret_cast<uint32_t*>(work + 2048);      // [128] union of run starts
-    uint32_t* PU = U + 128;                                       // [128] segments before word i
-    uint32_t* wt = PU + 128;                                      // per-warp totals (scan)
+    uint2* UP = reinterpret_cast<uint2*>(work + 2048);           // [128] union of run starts, segments before it - 1
+    uint2* wt = UP + 128;                                         // per-warp totals (scan)
     uint32_t* SV = reinterpret_cast<uint32_t*>(work + kRunArea + 1024);   // segment elements
     // word tid of every bitmap; exclusive prefixes of their bit counts
     const uint32_t b0 = bm[tid], b1 = bm[128 + tid], b2 = bm[256 + tid], b3 = bm[384 + tid];
@@ -1491,12 +1491,15 @@ __device__ void fill_segments(const RleJobDesc& jb, uint32_t q0, int len, bool s
         const uint32_t yu = __shfl_up_sync(0xffffffffu, iu, o), yb = __shfl_up_sync(0xffffffffu, ib, o);
         if (lane >= o) { iu += yu; ib += yb; }
     }
-    if (lane == 31) { wt[2 * warp] = iu; wt[2 * warp + 1] = ib; }
+    if (lane == 31) wt[warp] = make_uint2(iu, ib);
     __syncthreads();
     uint32_t eu = iu - cu, eb = ib - cb;
-    for (int k = 0; k < warp; ++k) { eu += wt[2 * k]; eb += wt[2 * k + 1]; }
-    U[tid] = u;
-    PU[tid] = eu;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const uint2 t = wt[k];
+        if (k < warp) { eu += t.x; eb += t.y; }
+    }
+    UP[tid] = make_uint2(u, eu - 1u);
     // the element of every segment starting in word tid
     for (uint32_t m = u; m; m &= m - 1u) {
         const int b = __ffs(m) - 1;
@@ -1511,24 +1514,40 @@ __device__ void fill_segments(const RleJobDesc& jb, uint32_t q0, int len, bool s
         SV[eu + __popc(u & (le >> 1))] = e;
     }
     __syncthreads();
-    const uint32_t w = (uint32_t)jb.w;
     const bool dense = jb.pitch == jb.w;
-    for (int g = tid; 4 * g < len; g += kDT) {
-        const uint32_t uw = U[g >> 3];
-        const int bb = (g & 7) << 2;
-        const uint32_t k0 = PU[g >> 3] + __popc(uw & ((2u << bb) - 1u)) - 1u;
-        const uint32_t in = (uw >> (bb + 1)) & 7u;                // segments starting inside the group
-        const uint32_t k1 = k0 + (in & 1u), k2 = k1 + ((in >> 1) & 1u), k3 = k2 + (in >> 2);
+    const int bb = (tid & 7) << 2;               // a thread's groups start at one bit of their words
+    const uint32_t le = (2u << bb) - 1u;
+    auto group = [&](int i) {                    // elements [4 (tid + 128 i), + 4)
+        const uint2 up = UP[(tid >> 3) + 16 * i];
+        const uint32_t k0 = up.y + __popc(up.x & le);
+        const uint32_t in = (up.x >> (bb + 1)) & 7u;             // segments starting inside the group
         const uint32_t v0 = SV[k0];
-        const uint4 v = in ? make_uint4(v0, SV[k1], SV[k2], SV[k3]) : make_uint4(v0, v0, v0, v0);
+        uint4 v = make_uint4(v0, v0, v0, v0);
+        if (in) {
+            const uint32_t k1 = k0 + (in & 1u), k2 = k1 + ((in >> 1) & 1u), k3 = k2 + (in >> 2);
+            v.y = SV[k1]; v.z = SV[k2]; v.w = SV[k3];
+        }
+        return v;
+    };
+    if (jb.vec && len == kChunk) {               // whole chunks: every group is one 16-byte store
+        const uint32_t q = q0 + 4u * (uint32_t)tid;
+        if (dense) {
+            uint4* o = reinterpret_cast<uint4*>(dstp + q);
+#pragma unroll
+            for (int i = 0; i < kChunk / 4 / kDT; ++i) st_stream(o + kDT * i, group(i));
+        } else {
+#pragma unroll 2
+            for (int i = 0; i < kChunk / 4 / kDT; ++i)
+                st_stream(reinterpret_cast<uint4*>(dstp + elem_off(jb, q + 4u * kDT * i)), group(i));
+        }
+        return;
+    }
+    for (int i = 0; 4 * (tid + kDT * i) < len; ++i) {
+        const uint4 v = group(i);
+        const int g = tid + kDT * i;
         const uint32_t q = q0 + 4u * (uint32_t)g;
-        if (jb.vec) {
-            size_t e = q;
-            if (!dense) {
-                const uint32_t y = q / w;
-                e = (size_t)y * jb.pitch + (q - y * w);
-            }
-            st_stream(reinterpret_cast<uint4*>(dstp + e), v);
+        if (jb.vec && 4 * g + 4 <= len) {
+            st_stream(reinterpret_cast<uint4*>(dstp + (dense ? (size_t)q : elem_off(jb, q))), v);
         } else {
             const uint32_t vv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -1539,128 +1558,95 @@ __device__ void fill_segments(const RleJobDesc& jb, uint32_t q0, int len, bool s
 }
 
 template <int N>
-__global__ void __launch_bounds__(kDT)
+__global__ void __launch_bounds__(kDT, 12)
 k_rle_decompress(const __grid_constant__ RleJobList<N> J, uint32_t* status)
 {
     // the four decoded planes; a mode-0 chunk's stream (at most 8 * 2048 + 16
     // bytes) is staged here instead
     __shared__ __align__(16) uint8_t sbuf[4 * kChunk + 64];
     uint8_t (*planes)[kChunk] = reinterpret_cast<uint8_t (*)[kChunk]>(sbuf);
-    __shared__ uint32_t s_beg[5];
-    __shared__ int s_fail, s_over, s_mode;
-    __shared__ uint8_t s_hdr[rlec::kHdrBytes];
     __shared__ uint32_t s_tok[kTok0];                 // mode 0: listed tokens
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t unit = blockIdx.x;
-    // the run bitmaps start empty; nothing else uses sbuf before they are filled
-#pragma unroll
-    for (int i = 0; i < 4; ++i) reinterpret_cast<uint32_t*>(sbuf)[tid + kDT * i] = 0u;
-    if (tid == 0) s_over = 0;
     const RleJobDesc& jb = J.j[find_job(J, unit)];
     const uint8_t* src = reinterpret_cast<const uint8_t*>(jb.src);
     const uint64_t size = jb.capacity;
     const uint32_t nc = jb.n_chunks;
     const uint32_t c = unit - jb.first_unit;
-
-    // header (32 bytes) and this chunk's end-table entries 4c-1 .. 4c+3 (20 bytes),
-    // fetched in one round trip by 52 threads
-    if (tid < rlec::kHdrBytes) s_hdr[tid] = rlec::header_byte(src, size, nc, c, tid);
-    __syncthreads();
-    if (tid == 0) {
-        const int bad = rlec::check_header(s_hdr, size, (uint32_t)jb.w, (uint32_t)jb.h, nc, c, s_beg, &s_mode, true);
-        s_fail = bad;
-        if (bad) set_status(status, EC_ERR_CORRUPT);
+    const rlec::ChunkEnds E = rlec::check_chunk(src, size, size, (uint32_t)jb.w, (uint32_t)jb.h, nc, c, true);
+    if (E.bad) {
+        if (tid == 0) set_status(status, EC_ERR_CORRUPT);
+        return;
     }
-    __syncthreads();
-    if (s_fail || nc == 0) return;
+    if (nc == 0) return;
 
     const uint32_t n = (uint32_t)jb.w * (uint32_t)jb.h;
     const uint32_t q0 = c * (uint32_t)kChunk;
     const int len = (int)min((uint32_t)kChunk, n - q0);
-    if (s_mode == 0) {
-        decode_mode0(jb, src + 32 + 4ull * nc, s_beg[0], s_beg[1], q0, len, sbuf, s_tok, status);
+    if (E.mode == 0) {
+        decode_mode0(jb, src + 32 + 4ull * nc, (uint32_t)E.beg(5), (uint32_t)E.end(5), q0, len, sbuf, s_tok, status);
         return;
     }
     const uint8_t* payload = src + 32 + 16ull * nc;
     uint32_t* dstp = reinterpret_cast<uint32_t*>(jb.dst);
-    const uint32_t w = (uint32_t)jb.w;
-    const bool sw = s_mode == 2;
+    const bool sw = E.mode == 2;
+    const int beg = E.beg(warp), end = E.end(warp);
 
     // Runs first: warp p walks plane p's tokens, marking where each run starts
-    // (every repeat token, every literal byte) and keeping its byte.
-    {
+    // (every repeat token, every literal byte) and keeping its byte.  A token of
+    // k bytes starts at least k / 2 runs, so a stream of more than 2 kRunCap
+    // bytes has too many for this path, and its walk is not begun.
+    if (!E.any_longer(2u * (uint32_t)kRunCap)) {
         uint32_t* bm = reinterpret_cast<uint32_t*>(sbuf);          // [4][128] run starts per plane
         uint8_t* val = sbuf + kRunArea;                             // [4][256] run bytes per plane
+        reinterpret_cast<uint4*>(bm + 128 * warp)[lane] = make_uint4(0u, 0u, 0u, 0u);
+        __syncwarp();
         int nr = 0;
-        const int r = rlec::decode_plane_runs(rlec::GlobalBytes{payload}, (int)s_beg[warp], (int)s_beg[warp + 1],
-                                              len, bm + 128 * warp, val + 256 * warp, kRunCap, &nr, lane);
-        if (lane == 0 && r == 1) s_fail = 1;
-        if (lane == 0 && r == 2) s_over = 1;
-        __syncthreads();
-        if (s_fail) {
-            if (tid == 0) set_status(status, EC_ERR_CORRUPT);
+        const int r = rlec::decode_plane_runs(rlec::GlobalBytes{payload}, beg, end, len, bm + 128 * warp,
+                                              val + 256 * warp, kRunCap, &nr, lane);
+        if (!__syncthreads_or(r)) {
+            fill_segments(jb, q0, len, sw, bm, val, sbuf, dstp);
             return;
         }
-        if (!s_over) {
-            fill_segments(jb, q0, len, sw, bm, val, sbuf, dstp);
+        if (__syncthreads_or(r == 1)) {
+            if (tid == 0) set_status(status, EC_ERR_CORRUPT);
             return;
         }
     }
 
     // many runs: warp p decodes byte plane p into shared memory
-    if (rlec::decode_plane(rlec::GlobalBytes{payload}, (int)s_beg[warp], (int)s_beg[warp + 1], len, planes[warp],
-                           lane) &&
-        lane == 0)
-        s_fail = 1;
-    __syncthreads();
-    if (s_fail) {
+    if (__syncthreads_or(rlec::decode_plane_dense(rlec::GlobalWords{payload}, beg, end, len, planes[warp], lane))) {
         if (tid == 0) set_status(status, EC_ERR_CORRUPT);
         return;
     }
 
-    // transpose planes back into elements, 16 per thread; groups of four
-    // equal elements (each plane word one repeated byte) are un-swizzled once
-    if (jb.vec) {
-        const bool dense = jb.pitch == jb.w;
-        for (int g16 = tid; 16 * g16 < len; g16 += kDT) {
-            const uint4 A = *reinterpret_cast<const uint4*>(&planes[0][16 * g16]);
-            const uint4 B = *reinterpret_cast<const uint4*>(&planes[1][16 * g16]);
-            const uint4 C = *reinterpret_cast<const uint4*>(&planes[2][16 * g16]);
-            const uint4 D = *reinterpret_cast<const uint4*>(&planes[3][16 * g16]);
-            const uint32_t a4[4] = {A.x, A.y, A.z, A.w}, b4[4] = {B.x, B.y, B.z, B.w};
-            const uint32_t c4[4] = {C.x, C.y, C.z, C.w}, d4[4] = {D.x, D.y, D.z, D.w};
+    // transpose planes back into elements, 16 per thread; the swizzle is undone
+    // on the plane words, four elements at a time
+    const int whole = jb.vec ? len & ~3 : 0;                  // elements written by 16-byte groups
+    const bool dense = jb.pitch == jb.w;
+    for (int g16 = tid; 16 * g16 < whole; g16 += kDT) {
+        const uint4 A = *reinterpret_cast<const uint4*>(&planes[0][16 * g16]);
+        const uint4 B = *reinterpret_cast<const uint4*>(&planes[1][16 * g16]);
+        const uint4 C = *reinterpret_cast<const uint4*>(&planes[2][16 * g16]);
+        const uint4 D = *reinterpret_cast<const uint4*>(&planes[3][16 * g16]);
+        uint32_t a4[4] = {A.x, A.y, A.z, A.w}, b4[4] = {B.x, B.y, B.z, B.w};
+        uint32_t c4[4] = {C.x, C.y, C.z, C.w}, d4[4] = {D.x, D.y, D.z, D.w};
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int g = 4 * g16 + k;
-                if (4 * g >= len) break;
-                const uint32_t a = a4[k], bb = b4[k], c = c4[k], d = d4[k];
-                uint4 v;
-                if (a == bcast8(a) && bb == bcast8(bb) && c == bcast8(c) && d == bcast8(d)) {
-                    uint32_t e = __byte_perm(__byte_perm(a, bb, 0x0040), __byte_perm(c, d, 0x0040), 0x5410);
-                    if (sw) e = swizzle(e);
-                    v = make_uint4(e, e, e, e);
-                } else {
-                    v = transpose4(a, bb, c, d);              // planes -> elements
-                    if (sw) { v.x = swizzle(v.x); v.y = swizzle(v.y); v.z = swizzle(v.z); v.w = swizzle(v.w); }
-                }
-                const uint32_t q = q0 + 4u * g;
-                size_t e = q;
-                if (!dense) {
-                    const uint32_t y = q / w;
-                    e = (size_t)y * jb.pitch + (q - y * w);
-                }
-                st_stream(reinterpret_cast<uint4*>(dstp + e), v);
-            }
+        for (int k = 0; k < 4; ++k) {
+            const int g = 4 * g16 + k;
+            if (4 * g >= whole) break;
+            if (sw) rlec::swizzle_planes(a4[k], b4[k], c4[k], d4[k]);
+            const uint4 v = transpose4(a4[k], b4[k], c4[k], d4[k]);
+            const uint32_t q = q0 + 4u * g;
+            st_stream(reinterpret_cast<uint4*>(dstp + (dense ? (size_t)q : elem_off(jb, q))), v);
         }
-    } else {
-        for (int t = tid; t < len; t += kDT) {
-            uint32_t v = (uint32_t)planes[0][t] | ((uint32_t)planes[1][t] << 8) |
-                         ((uint32_t)planes[2][t] << 16) | ((uint32_t)planes[3][t] << 24);
-            if (sw) v = swizzle(v);
-            const uint32_t q = q0 + t, y = q / w, x = q - y * w;
-            dstp[(size_t)y * jb.pitch + x] = v;
-        }
+    }
+    for (int t = whole + tid; t < len; t += kDT) {
+        uint32_t v = (uint32_t)planes[0][t] | ((uint32_t)planes[1][t] << 8) |
+                     ((uint32_t)planes[2][t] << 16) | ((uint32_t)planes[3][t] << 24);
+        if (sw) v = swizzle(v);
+        dstp[elem_off(jb, q0 + t)] = v;
     }
 }
 

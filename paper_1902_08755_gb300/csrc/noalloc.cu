@@ -80,6 +80,7 @@ extern "C" ec_status ec_rle_compress_noalloc(const void* src, int32_t w, int32_t
     d.w = w;
     d.h = h;
     d.pitch = pitch;
+    d.winv = ec::rle_winv(w);
     d.mode = mode;
     d.n_chunks = (uint32_t)nchunks;
     d.first_unit = 0;
