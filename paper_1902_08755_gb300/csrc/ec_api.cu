@@ -165,7 +165,7 @@ ec_status ec_create(ec_ctx** out, int device)
     cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, device);
     if (cudaMalloc(&ctx->d_status, sizeof(uint32_t)) != cudaSuccess ||
         cudaMemset(ctx->d_status, 0, sizeof(uint32_t)) != cudaSuccess ||
-        ensure_scratch(ctx, rle_compress_scratch_bytes(1024, kRlePoolPerUnit)) != EC_OK) {
+        ensure_scratch(ctx, rle_compress_scratch_bytes(1024, rle_pool_bytes(1024))) != EC_OK) {
         ec_destroy(ctx);
         return EC_ERR_CUDA;
     }
@@ -530,8 +530,8 @@ ec_status rle_job_desc(const ec_rle_job& j, bool compress, RleJobDesc* d)
         d->mode = j.mode;
         d->d_size = j.d_size;
         // 16-byte reads: rows of whole 16-byte groups, or one contiguous run
-        // of a multiple of 4 elements
-        d->vec = aligned16(j.src) && ((j.w % 4 == 0 && j.pitch % 4 == 0) || (j.pitch == j.w && n % 4 == 0));
+        // (whose last elements, where 4 does not divide it, are read singly)
+        d->vec = aligned16(j.src) && ((j.w % 4 == 0 && j.pitch % 4 == 0) || j.pitch == j.w);
     } else {
         if (!j.src || (reinterpret_cast<uintptr_t>(j.src) & 3u)) return EC_ERR_INVALID_ARG;
         if (n > 0 && (reinterpret_cast<uintptr_t>(j.dst) & 3u)) return EC_ERR_INVALID_ARG;
@@ -573,7 +573,7 @@ static ec_status rle_batch(ec_ctx* ctx, const ec_rle_job* jobs, int32_t njobs, b
         }
         cudaError_t e;
         if (compress) {
-            const ec_status st = ensure_scratch(ctx, rle_compress_scratch_bytes(units, kRlePoolPerUnit));
+            const ec_status st = ensure_scratch(ctx, rle_compress_scratch_bytes(units, rle_pool_bytes(units)));
             if (st != EC_OK) return st;
             e = launch_rle_compress(&d[b], cnt, units, ctx->scratch, ctx->scratch_bytes, ctx->d_status,
                                     (cudaStream_t)s);

@@ -184,13 +184,21 @@ struct RleJobList {
 static_assert(sizeof(RleJobList<kRleJobsPerLaunch>) < 32764 - 256, "kernel parameter limit");
 
 // Scratch of a compress launch of `units` work units: a ticket, a counter and a
-// pool cursor, a 16-byte record and a 4-byte list entry per unit (modes 1, 2;
-// mode 0 uses 8 bytes per unit of them), then a pool for the coded chunks,
-// pool_per_unit bytes per unit.  A
-// chunk that finds the pool full is coded a second time when placed, so any
-// pool size gives the same stream.
-size_t rle_compress_scratch_bytes(uint32_t units, size_t pool_per_unit);
+// pool cursor, a 16-byte record and a 4-byte list entry per unit, then a pool
+// of pool_bytes for the coded chunks.  A chunk that finds the pool full is
+// coded a second time when placed, so any pool size gives the same stream.
+size_t rle_compress_scratch_bytes(uint32_t units, size_t pool_bytes);
+
+// The pool a launch is given: 512 bytes per unit, which few-run chunks stay
+// below on average, and 8 KB more per unit (half of a chunk's size) for chunks
+// of many tokens, up to 256 MB in all.
 constexpr size_t kRlePoolPerUnit = 512;
+constexpr size_t kRleDensePoolPerUnit = 8192, kRleDensePoolMax = 256u << 20;
+inline size_t rle_pool_bytes(uint32_t units)
+{
+    const size_t dense = kRleDensePoolPerUnit * units;
+    return kRlePoolPerUnit * units + (dense < kRleDensePoolMax ? dense : kRleDensePoolMax);
+}
 
 cudaError_t launch_rle_compress(const RleJobDesc* jobs, int n, uint32_t total_units,
                                 void* scratch, size_t scratch_bytes, uint32_t* status, cudaStream_t s);

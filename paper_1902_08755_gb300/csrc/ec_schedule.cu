@@ -574,8 +574,8 @@ ec_status ec_schedule_plan(ec_ctx* ctx, int32_t mode, int32_t algorithm, const e
         lr.fst_off = A.take(std::max<size_t>(ns, 1) * sizeof(FusedStage));
         lr.fun_off = A.take(std::max<size_t>(nu, 1) * sizeof(FusedUnit));
     }
-    const size_t scratch_bytes = ec::rle_compress_scratch_bytes((uint32_t)std::max<uint64_t>(max_units, 1),
-                                                                ec::kRlePoolPerUnit);
+    const uint32_t scratch_units = (uint32_t)std::max<uint64_t>(max_units, 1);
+    const size_t scratch_bytes = ec::rle_compress_scratch_bytes(scratch_units, ec::rle_pool_bytes(scratch_units));
     const size_t scratch_off = A.take(scratch_bytes);
 
     DeviceGuard g(ctx->device);

@@ -2,24 +2,25 @@
 // per-component RLE, bit-swizzle preconditioner, data decomposition).
 //
 // Compress: a pipeline of kernels with no waits between warps.
-//   1. Coding (persistent warps, a chunk of 4096 elements at a time from an
-//      atomic ticket): the chunk streams through shared memory and its change
-//      points are listed; a chunk with few of them (sparse) is coded at once
-//      from the list into a scratch pool, the others (dense) are listed.
+//   1. Coding, a chunk of 4096 elements at a time: the chunk's change points are
+//      listed; a chunk with few of them (sparse) is coded at once from the list
+//      into a scratch pool, the others (dense) are listed.
 //      Modes 1, 2: element change points, four byte planes (mode 2 swizzled;
 //      the swizzle permutes bits, so it commutes with the comparison); runs of
 //      three or more bytes become repeat tokens, maximal spans of shorter runs
 //      literal tokens.  Mode 0 (basic RLE): change points of 8-byte units,
 //      one stream; runs of two or more units repeat, single units literal.
-//   2. Sizing of the dense chunks from the image: all four planes classified
+//   2. The dense chunks, coded from the image: all four planes classified
 //      at once with byte-SIMD masks (a byte is part of a repeat iff one of the
-//      three windows of 3 around it is constant), warp max- and sum-scans over
-//      8 steps of 512 positions; in mode 0 a CTA per chunk with block scans.
+//      three windows of 3 around it is constant), max- and sum-scans over the
+//      CTA, and the streams to the pool where it has room; in mode 0 a CTA per
+//      chunk with block scans, which sizes them.
 //   3. A scan of each job's chunk sizes: the chunks' offsets, the header and
 //      the stream size.
 //   4. Placing: the pooled chunks copied to their place with their end-table
-//      entries; the dense chunks coded again, straight to their place.
-// Every wait (the copies into shared memory) is bounded (EC_ERR_TIMEOUT).
+//      entries; dense chunks that are not in the pool coded again, straight to
+//      their place.
+// Every wait (for copies into shared memory) is bounded (EC_ERR_TIMEOUT).
 //
 // Decompress: one CTA of four warps per chunk.  Every warp fetches the header
 // and the chunk's end-table entries in one round trip and validates them.
@@ -132,24 +133,21 @@ __device__ __forceinline__ void copy_out(uint8_t* __restrict__ o, const uint8_t*
     if (th) o[tail0 + t] = tb;
 }
 
-// ---- compressor: one warp per chunk ---------------------------------------
-// Every warp of the coding kernel works alone, chunk after chunk.  It streams
-// each chunk through a ring of two 2 KB quarter buffers in shared memory,
-// filled by asynchronous copies (bulk copies of row segments, or 4-byte copies
-// where rows are not 16-byte aligned) that complete on the buffer's mbarrier;
-// a buffer is refilled with the next quarter (of this chunk or the next) as
-// soon as it has been read.  Reading a chunk, the warp lists its change
-// points: the positions where the element differs from its predecessor, with
-// the element there.  A byte plane can change only where the element does, so
-// each plane's runs are the change points where that plane's byte differs
-// from the previous change point's, and every run's value is the byte at its
-// start: the sparse path codes the chunk's streams from the change list alone,
-// into the warp's stage, and leaves them in a scratch pool.  Chunks with more
-// change points than the list holds are dense: a recoding kernel sizes them
-// from the image.  A scan over each job's chunk sizes gives every chunk its
-// offset; a placing kernel copies the pooled chunks to their place and the
-// recoding kernel writes the dense ones there (coded again from the image,
-// partly from L2).  No kernel waits for another's warps.
+// ---- compressor --------------------------------------------------------------
+// The coding kernels list each chunk's change points.  A chunk of few of them
+// (sparse) is coded at once from the list, its streams left in a scratch pool;
+// the others (dense) are listed, and a recoding kernel codes them from the
+// image.  A scan over each job's chunk sizes gives every chunk its offset; the
+// placing kernels copy the pooled chunks to their place, and code those that
+// the pool had no room for again.  No kernel waits for another's warps.
+//
+// Four-plane modes: a CTA of four warps per chunk (k_rle_code).  Mode 0: every
+// warp of a persistent kernel works alone, chunk after chunk (k_rle_compress0):
+// it streams each chunk through a ring of two 2 KB quarter buffers in shared
+// memory, filled by asynchronous copies (bulk copies of row segments, or 4-byte
+// copies where rows are not 16-byte aligned) that complete on the buffer's
+// mbarrier; a buffer is refilled with the next quarter (of this chunk or the
+// next) as soon as it has been read.
 constexpr int kWPB = 2;                       // warps per CTA
 constexpr int kCap = 128;                     // change points the sparse path takes
 constexpr int kQ = 512;                       // elements per quarter buffer
@@ -161,6 +159,7 @@ constexpr int kSlots = 2;                     // quarter buffers per warp
 // 2 + L / 64 bytes, a literal span of k short runs to at most 3k bytes).
 constexpr int kStagePlane = 3 * kCap + kChunk / 64;
 constexpr uint32_t kRecode = 0xFFFFFFFFu;      // record: coded again when placed
+constexpr uint32_t kDense = 0x80000000u;       // record: a pooled dense chunk (offset / 16 in the low bits)
 
 // One warp's shared memory.  Quarter s of the warp's sequence of quarters
 // (4 per chunk) goes to buf[s % kSlots].
@@ -169,16 +168,17 @@ struct WarpRing {
     uint64_t full[kSlots];
     uint64_t pad[4 - kSlots];       // (keeps what follows 16-byte aligned)
     uint8_t stage[4 * kStagePlane]; // the chunk's plane streams (plane p at p * kStagePlane)
-    uint32_t ce[kCap];              // the chunk being read: element at each change point
-    uint16_t cq[kCap];              // (swizzled in mode 2) and its position
-    uint8_t rl[4][kCap];            // the planes' runs: index of the change point starting each
+    uint32_t ce[kCap];              // the chunk being read: first element of each change point's unit,
+    uint32_t ch[kCap];              // its second element
+    uint16_t cq[kCap];              // and its position
 };
 static_assert((kQ + 4) * 4 % 16 == 0 && sizeof(WarpRing) % 16 == 0, "16-byte aligned buffers");
 
-// A coded chunk, as the coding kernel leaves it for the placing kernels: its
-// four plane stream sizes, where its streams wait in the pool (kRecode: not
-// kept, coded again from the image when placed), and its offset inside the
-// stream's payload (written by the scan).
+// A coded chunk, as the coding kernels leave it for the placing kernels: its
+// four plane stream sizes, where its streams wait in the pool (a sparse chunk's
+// offset / 4, a dense chunk's offset / 16 with kDense, or kRecode: not kept,
+// coded again from the image when placed), and its offset inside the stream's
+// payload (written by the scan).
 struct ChunkRec {
     uint16_t T[4];
     uint32_t pool;
@@ -239,11 +239,8 @@ __device__ __forceinline__ uint4 load_elems(const RleJobDesc& jb, uint32_t q0, i
 {
     if (q >= len) return make_uint4(0u, 0u, 0u, 0u);
     const uint32_t w = (uint32_t)jb.w;
-    if (jb.vec) {
-        size_t e = q0 + (uint32_t)q;
-        if (jb.pitch != jb.w) {
-            e = elem_off(jb, q0 + (uint32_t)q);
-        }
+    if (jb.vec && q + 4 <= len) {
+        const size_t e = jb.pitch == jb.w ? q0 + (uint32_t)q : elem_off(jb, q0 + (uint32_t)q);
         return __ldg(reinterpret_cast<const uint4*>(jb.src + e));
     }
     uint32_t v[4];
@@ -292,7 +289,7 @@ __device__ void issue_quarter(const RleJobDesc& jb, uint32_t unit, int qi, int s
     }
     uint32_t* dst = W.buf[slot] + 4;
     const uint32_t w = (uint32_t)jb.w;
-    if (!jb.vec) {
+    if (!jb.vec || (qlen & 3)) {                       // (a contiguous image may end inside a 16-byte group)
         uint32_t y = row_of(jb, qs + (uint32_t)lane), x = qs + (uint32_t)lane - y * w;
         for (int i = lane; i < qlen; i += 32) {
             cp_async4(dst + i, jb.src + (size_t)y * jb.pitch + x);
@@ -318,276 +315,318 @@ __device__ void issue_quarter(const RleJobDesc& jb, uint32_t unit, int qi, int s
     }
 }
 
-// Append the change points among positions [kQ qi, kQ qi + kQ) of the chunk
-// to W.ce / W.cq (the quarter's elements in shared memory at `data`).  carry:
-// the element before the quarter (updated to the quarter's last).  Every lane
-// flags the changes among its four elements of each of the G groups of 128
-// positions; one warp scan of the four groups' per-lane counts, packed in the
-// bytes of a word (a group has at most 128 changes, so no byte carries into
-// the next), places every change point in position order at once.  Returns
-// false once the chunk has more than kCap change points.
-__device__ bool detect_quarter(const uint32_t* data, int len, int qi, WarpRing& W, int& m, uint32_t& carry)
+// ---- coding kernel of the four-plane modes: a CTA of four warps per chunk ----
+// The chunk is copied into shared memory (bulk copies, or 4-byte asynchronous
+// copies where rows are not 16-byte aligned); twelve CTAs are resident on an
+// SM, so the copies of most overlap the work of the others.  Lane l of warp k
+// holds positions [1024 k + 32 l, + 32) and flags those whose element differs
+// from its predecessor in the bits of one word.  One scan over the CTA lists
+// the change points of the whole chunk in order.  A byte plane can change only
+// where the element does, so each plane's runs are the change points where that
+// plane's byte differs from the previous change point's, and every run's value
+// is the byte at its start: warp p then codes plane p from the list alone.  A
+// chunk with more than kCap change points is dense and left to the recoding
+// kernel.
+//
+// Bound by instruction issue up to a few thousand chunks per launch, by HBM and
+// issue alike beyond (2280 warp instructions per chunk, issue 68% active, DRAM
+// 74%).  16 flat sources, colour and depth: 1920x1080 54 -> 34.5 us, 7680x4320
+// (1.87 GB) 357 -> 322 us, against persistent warps that each streamed a chunk
+// through two 2 KB buffers (2930 instructions per chunk, and a chunk's whole
+// latency on one warp: the pieces of a binary-swap stage took 34 us whatever
+// their number, 18 here).  Holding the chunk in registers (eight 16-byte groups
+// per lane, eight CTAs per SM) took 3220 instructions per chunk and 465 us.
+constexpr int kCT = 128;
+
+// Plane stream of a chunk of len elements from its m <= 32 change points, run
+// by run, where every run is at least 3 bytes (so all of it is repeat tokens).
+// Lane i holds change point i: byte v at position q (valid: i < m).  Returns
+// the bytes written, or 0 (nothing written) when a run is shorter.
+__device__ __forceinline__ uint32_t code_plane_few(bool valid, uint32_t v, int q, int len, uint8_t* out)
 {
     const int lane = threadIdx.x & 31;
-    constexpr int G = kQ / 128;
-    static_assert(G == 4, "four groups' counts in the bytes of one word");
-    uint4 vv[G];
-    uint32_t pv[G];
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-        vv[g] = *reinterpret_cast<const uint4*>(data + 128 * g + 4 * lane);
-        pv[g] = data[128 * g + 4 * lane - 1];             // g = lane = 0 reads the guard word
-    }
-    if (lane == 0) pv[0] = qi == 0 ? ~vv[0].x : carry;    // position 0 is always listed
-    carry = __shfl_sync(0xffffffffu, vv[G - 1].w, 31);   // (used only when the quarter is full)
-    const int qend = min(len - kQ * qi, kQ);              // positions of this quarter
-    uint32_t f[G], packed = 0u;
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-        const uint4 v = vv[g];
-        f[g] = (uint32_t)(v.x != pv[g]) | ((uint32_t)(v.y != v.x) << 1) | ((uint32_t)(v.z != v.y) << 2) |
-               ((uint32_t)(v.w != v.z) << 3);
-    }
-    if (qend < kQ) {                                      // the chunk's last quarter: positions past len
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const int q = 128 * g + 4 * lane;
-            if (q + 4 > qend) f[g] &= q >= qend ? 0u : (1u << (qend - q)) - 1u;
+    const uint32_t before = __shfl_up_sync(0xffffffffu, v, 1);
+    const bool keep = valid && (lane == 0 || v != before);          // starts a run
+    const uint32_t K = __ballot_sync(0xffffffffu, keep);
+    const uint32_t nm = lane == 31 ? 0u : K & ~((2u << lane) - 1u);
+    const int qn = __shfl_sync(0xffffffffu, q, nm ? __ffs(nm) - 1 : 0);
+    const int L = (nm ? qn : len) - q;
+    if (__any_sync(0xffffffffu, keep && L < 3)) return 0u;
+    const uint32_t cost = keep ? 2u * (uint32_t)((L + 127) >> 7) : 0u;
+    const uint32_t incl = (uint32_t)rlec::warp_incl_sum((int)cost, lane);
+    const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+    if (keep) {
+        uint8_t* o = out + (incl - cost);
+        for (int r = L; r > 0; r -= 128) {
+            o[0] = (uint8_t)(127 + min(r, 128));
+            o[1] = (uint8_t)v;
+            o += 2;
         }
     }
-#pragma unroll
-    for (int g = 0; g < G; ++g) packed |= (uint32_t)__popc(f[g]) << (8 * g);
-    uint32_t inc = packed;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += y;
-    }
-    const uint32_t tot = __shfl_sync(0xffffffffu, inc, 31), exc = inc - packed;
-    const int cnt = (int)((tot & 0xFFu) + ((tot >> 8) & 0xFFu) + ((tot >> 16) & 0xFFu) + (tot >> 24));
-    if (m + cnt > kCap) return false;
-    int base = m;
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-        if (f[g]) {
-            const uint4 v = vv[g];
-            const int qq = kQ * qi + 128 * g + 4 * lane;
-            int o = base + (int)((exc >> (8 * g)) & 0xFFu);
-            if (f[g] & 1u) { W.cq[o] = (uint16_t)qq; W.ce[o] = v.x; ++o; }
-            if (f[g] & 2u) { W.cq[o] = (uint16_t)(qq + 1); W.ce[o] = v.y; ++o; }
-            if (f[g] & 4u) { W.cq[o] = (uint16_t)(qq + 2); W.ce[o] = v.z; ++o; }
-            if (f[g] & 8u) { W.cq[o] = (uint16_t)(qq + 3); W.ce[o] = v.w; }
-        }
-        base += (int)((tot >> (8 * g)) & 0xFFu);
-    }
-    m += cnt;
-    return true;
+    return total;
 }
 
-// The change lists a sparse coder reads: element (swizzled in mode 2) and
-// position of each change point, in order; rl is its scratch.
-struct Lists {
-    uint32_t* ce;
-    uint16_t* cq;
-    uint8_t (*rl)[kCap];
-};
-
-// Sparse path, fast case: at most 32 change points and every run of every
-// plane at least 3 bytes long (so every run is repeat tokens).  Lane i holds
-// change point i; for each plane the lanes that start a run are found with
-// one ballot, each run's end is the next such lane's position (a shuffle) or
-// the chunk's end, and one scan over the four planes (16-bit halves) places
-// the tokens.  Returns false, writing nothing, when the case does not apply.
-__device__ bool code_sparse_fast(const Lists& W, int m, int len, uint32_t* T, uint8_t* stage)
+// Plane stream of a chunk of len elements from its m <= 128 change points
+// (positions cq of the elements el, the plane's byte at bit `shift`; swizzled on
+// reading when sw).  Lane l takes change points 4l .. 4l+3.  A run of three or
+// more bytes becomes repeat tokens; a shorter one belongs to a literal span (a
+// maximal sequence of short runs), whose start a warp max-scan finds.  A short
+// run at byte offset b of its span writes its bytes, the control byte of a
+// token that ends among them (127 for a full one), and, if the span ends with
+// it, the last token's control byte.  Returns the bytes written (at most
+// kStagePlane).
+__device__ __forceinline__ uint32_t code_plane_many(const uint32_t* el, const uint16_t* cq, int m, int shift, bool sw,
+                                                    int len, uint8_t* out)
 {
-    const int lane = threadIdx.x & 31;
-    if (m > 32) return false;
-    __syncwarp();                                     // the change list is complete
-    const bool valid = lane < m;
-    const uint32_t e = valid ? W.ce[lane] : 0u;
-    const int q = valid ? (int)W.cq[lane] : 0;
-    uint32_t diff = e ^ __shfl_up_sync(0xffffffffu, e, 1);
-    if (lane == 0) diff = 0xFFFFFFFFu;                // change point 0 starts a run in every plane
-    const uint32_t above = lane == 31 ? 0u : ~((2u << lane) - 1u);
-    uint32_t cost[4], K[4];
-    int L[4];
-    bool bad = false;
+    const int lane = threadIdx.x & 31, i0 = 4 * lane;
+    const uint32_t below = (1u << lane) - 1u, above = lane == 31 ? 0u : ~((2u << lane) - 1u);
+    uint32_t v[4];
+    int q[4], L[4];
+    uint32_t keep = 0u;                               // bit k: change point i0 + k starts a run of this plane
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        const bool keep = valid && ((diff >> (8 * p)) & 0xFFu) != 0u;
-        K[p] = __ballot_sync(0xffffffffu, keep);
-        const uint32_t nm = K[p] & above;
-        const int qn = __shfl_sync(0xffffffffu, q, nm ? __ffs(nm) - 1 : 0);
-        L[p] = keep ? (nm ? qn : len) - q : 0;
-        bad |= keep && L[p] < 3;
-        cost[p] = keep ? 2u * (uint32_t)((L[p] + 127) >> 7) : 0u;
+    for (int k = 0; k < 4; ++k) {
+        const bool ok = i0 + k < m;
+        q[k] = ok ? (int)cq[i0 + k] : len;
+        uint32_t e = ok ? el[q[k]] : 0u;
+        if (sw) e = swizzle(e);
+        v[k] = (e >> shift) & 0xFFu;
+        if (ok && k > 0 && v[k] != v[k - 1]) keep |= 1u << k;
     }
-    if (__any_sync(0xffffffffu, bad)) return false;
-    const uint32_t a = cost[0] | (cost[1] << 16), b = cost[2] | (cost[3] << 16);
-    uint32_t ia = a, ib = b;
+    const uint32_t vp = __shfl_up_sync(0xffffffffu, v[3], 1);
+    if (i0 < m && (lane == 0 || v[0] != vp)) keep |= 1u;
+    // where the next run starts: the lanes' first runs, then right to left
+    const uint32_t has = __ballot_sync(0xffffffffu, keep != 0u);
+    int first = len;
+#pragma unroll
+    for (int k = 3; k >= 0; --k)
+        if ((keep >> k) & 1u) first = q[k];
+    const int nl = (has & above) ? __ffs(has & above) - 1 : 0;
+    int next = __shfl_sync(0xffffffffu, first, nl);
+    if (!(has & above)) next = len;
+    uint32_t sh = 0u;                                 // bit k: a short run
+    uint32_t first_short = 0u, last_short = 0u;
+    bool any = false;
+#pragma unroll
+    for (int k = 3; k >= 0; --k) {
+        L[k] = 0;
+        if (!((keep >> k) & 1u)) continue;
+        L[k] = next - q[k];
+        next = q[k];
+        const uint32_t s = L[k] < 3 ? 1u : 0u;
+        sh |= s << k;
+        first_short = s;
+        if (!any) { last_short = s; any = true; }
+    }
+    const uint32_t ps = __shfl_sync(0xffffffffu, last_short, (has & below) ? 31 - __clz(has & below) : 0);
+    const uint32_t ns = __shfl_sync(0xffffffffu, first_short, nl);
+    const bool prev_short = (has & below) && ps, next_short = (has & above) && ns;
+    // the last span start up to each lane (position + 1; 0: none)
+    uint32_t start = 0u;
+    bool p = prev_short;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (!((keep >> k) & 1u)) continue;
+        const bool s = (sh >> k) & 1u;
+        if (s && !p) start = (uint32_t)q[k] + 1u;
+        p = s;
+    }
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t ya = __shfl_up_sync(0xffffffffu, ia, o), yb = __shfl_up_sync(0xffffffffu, ib, o);
-        if (lane >= o) { ia += ya; ib += yb; }
+        const uint32_t y = __shfl_up_sync(0xffffffffu, start, o);
+        if (lane >= o) start = max(start, y);
     }
-    const uint32_t ta = __shfl_sync(0xffffffffu, ia, 31), tb = __shfl_sync(0xffffffffu, ib, 31);
-    const uint32_t ea = ia - a, eb = ib - b;
-    const uint32_t ex[4] = {ea & 0xFFFFu, ea >> 16, eb & 0xFFFFu, eb >> 16};
-    T[0] = ta & 0xFFFFu; T[1] = ta >> 16; T[2] = tb & 0xFFFFu; T[3] = tb >> 16;
+    uint32_t span0 = __shfl_up_sync(0xffffffffu, start, 1);    // the span open at the lane's first run, if any
+    if (lane == 0) span0 = 0u;
+    uint32_t cost = 0u, sp = span0;
+    p = prev_short;
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        if (!((K[p] >> lane) & 1u) || ex[p] + cost[p] > (uint32_t)kStagePlane) continue;
-        uint8_t* ob = stage + p * kStagePlane + ex[p];
-        const uint8_t v = (uint8_t)(e >> (8 * p));
-        for (int rr = L[p]; rr > 0; rr -= 128) {
-            ob[0] = (uint8_t)(127 + min(rr, 128));
-            ob[1] = v;
-            ob += 2;
+    for (int k = 0; k < 4; ++k) {
+        if (!((keep >> k) & 1u)) continue;
+        const bool s = (sh >> k) & 1u;
+        if (s && !p) sp = (uint32_t)q[k] + 1u;
+        p = s;
+        if (!s) cost += 2u * (uint32_t)((L[k] + 127) >> 7);
+        else {
+            const uint32_t b = (uint32_t)q[k] + 1u - sp;
+            cost += (uint32_t)L[k] + (((b + (uint32_t)L[k] + 127u) >> 7) - ((b + 127u) >> 7));
         }
     }
-    return true;
+    const uint32_t incl = (uint32_t)rlec::warp_incl_sum((int)cost, lane);
+    const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+    uint32_t o = incl - cost;
+    sp = span0;
+    p = prev_short;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (!((keep >> k) & 1u)) continue;
+        const bool s = (sh >> k) & 1u;
+        if (s && !p) sp = (uint32_t)q[k] + 1u;
+        p = s;
+        if (!s) {
+            for (int r = L[k]; r > 0; r -= 128) {
+                out[o] = (uint8_t)(127 + min(r, 128));
+                out[o + 1] = (uint8_t)v[k];
+                o += 2;
+            }
+        } else {
+            const uint32_t b = (uint32_t)q[k] + 1u - sp;
+            const uint32_t so = o - b - ((b + 127u) >> 7);   // the span's first control byte
+            for (uint32_t x = b; x < b + (uint32_t)L[k]; ++x) {
+                out[so + x + (x >> 7) + 1u] = (uint8_t)v[k];
+                if ((x & 127u) == 127u) out[so + 129u * (x >> 7)] = 127u;
+            }
+            const uint32_t later = keep >> (k + 1);          // the lane's later runs
+            const bool more = later ? (sh >> (k + __ffs(later))) & 1u : next_short;
+            const uint32_t last = b + (uint32_t)L[k] - 1u;
+            if (!more) out[so + 129u * (last >> 7)] = (uint8_t)(last & 127u);
+            o += (uint32_t)L[k] + (((b + (uint32_t)L[k] + 127u) >> 7) - ((b + 127u) >> 7));
+        }
+    }
+    return total;
 }
 
-// Sparse path, the four planes together (their chains of shuffles and shared
-// memory accesses overlap).  Runs of plane p: change point i starts one iff
-// its plane-p byte differs from change point i-1's (point 0 always does);
-// rl[p][0, n_p) lists those change points.  Then the runs are coded 32 at a
-// time, a run per lane: a run of three or more bytes becomes repeat tokens; a
-// shorter one belongs to a literal span (a maximal sequence of short runs),
-// whose start a warp max-scan finds (four planes in the bytes of one word).
-// A short run at byte offset b of its span writes its bytes, the control
-// byte of a token that starts among them, and, if it holds a token's last
-// byte, that token's control byte (127 for a full token; the span's last run
-// knows the span's length).  Plane p's stream goes to stage + p * kStagePlane
-// (as far as it fits); its size to T[p].
-__device__ void code_sparse(const Lists& W, int m, int len, uint32_t* T, uint8_t* stage)
+template <int N>
+__global__ void __launch_bounds__(kCT, 12)
+k_rle_code(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, uint32_t* recode, uint8_t* pool, size_t pool_bytes,
+           uint32_t* ticket, uint32_t* status)
 {
-    const int lane = threadIdx.x & 31;
-    const uint32_t lt = (1u << lane) - 1u;
-    __syncwarp();                                     // the change list is complete
-    int n[4] = {0, 0, 0, 0};
-    uint32_t preve = 0u;
-    for (int r = 0; r < m; r += 32) {
-        const int i = r + lane;
-        const bool valid = i < m;
-        const uint32_t e = valid ? W.ce[i] : 0u;
-        uint32_t ep = __shfl_up_sync(0xffffffffu, e, 1);
-        if (lane == 0) ep = preve;
-        const uint32_t diff = e ^ ep;
-#pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            const bool keep = valid && (i == 0 || ((diff >> (8 * p)) & 0xFFu) != 0u);
-            const uint32_t K = __ballot_sync(0xffffffffu, keep);
-            if (keep) W.rl[p][n[p] + __popc(K & lt)] = (uint8_t)i;
-            n[p] += __popc(K);
+    __shared__ __align__(16) uint32_t raw[4 + kChunk];      // the chunk, after a guard
+    __shared__ __align__(16) uint8_t stage[4][kStagePlane];
+    __shared__ uint16_t cq[kCap];                            // the change points' positions
+    __shared__ uint64_t full;
+    __shared__ uint32_t s_cnt[4], s_T[4], s_po;
+    __shared__ int s_ji;
+    uint32_t* const el = raw + 4;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t unit = blockIdx.x;
+    if (warp == 0) {                                         // find the job, start the copies
+        if (lane == 0) {
+            mbar_init(&full, 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
-        preve = __shfl_sync(0xffffffffu, e, 31);
-    }
-    __syncwarp();
-    uint32_t carry[4] = {0u, 0u, 0u, 0u};
-    uint32_t sscarry = 0u;                            // byte p: 1 + the last span start of plane p so far
-    uint32_t prevshort = 0u;                          // bit p: the previous block's last run was short
-    const int nmax = max(max(n[0], n[1]), max(n[2], n[3]));
-    for (int r = 0; r < nmax; r += 32) {
-        const int i = r + lane;
-        int s[4], L[4];
-        uint32_t shm = 0u, nshm = 0u, stv = 0u;
-#pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            const uint8_t* R = W.rl[p];
-            const int np = n[p];
-            s[p] = 0;
-            L[p] = 0;
-            if (i < np) {
-                s[p] = (int)W.cq[R[i]];
-                L[p] = (i + 1 < np ? (int)W.cq[R[i + 1]] : len) - s[p];
-                if (L[p] < 3) shm |= 1u << p;
-            }
-        }
-        uint32_t prevm = __shfl_up_sync(0xffffffffu, shm, 1);
-        if (lane == 0) prevm = prevshort;
-        nshm = __shfl_down_sync(0xffffffffu, shm, 1);
-        if (lane == 31) {                             // the next block's first runs
-            nshm = 0u;
-#pragma unroll
-            for (int p = 0; p < 4; ++p) {
-                const uint8_t* R = W.rl[p];
-                const int np = n[p];
-                if (i + 1 < np) {
-                    const int ln = (i + 2 < np ? (int)W.cq[R[i + 2]] : len) - (int)W.cq[R[i + 1]];
-                    if (ln < 3) nshm |= 1u << p;
-                }
-            }
-        }
-#pragma unroll
-        for (int p = 0; p < 4; ++p)
-            if (((shm & ~prevm) >> p) & 1u) stv |= (uint32_t)(i + 1) << (8 * p);
-        uint32_t ss = stv;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, ss, o);
-            if (lane >= o) ss = __vmaxu4(ss, y);
-        }
-        ss = __vmaxu4(ss, sscarry);
-        sscarry = __shfl_sync(0xffffffffu, ss, 31);
-        prevshort = __shfl_sync(0xffffffffu, shm, 31);
-        uint32_t cost[4], B[4];
-#pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            cost[p] = 0u;
-            B[p] = 0u;
-            if (i >= n[p]) continue;
-            if (!((shm >> p) & 1u)) {
-                cost[p] = 2u * (uint32_t)((L[p] + 127) >> 7);
+        const int ji = find_job(J, unit);
+        const RleJobDesc& jb = J.j[ji];
+        const uint32_t q0 = (unit - jb.first_unit) * (uint32_t)kChunk, n = (uint32_t)jb.w * (uint32_t)jb.h;
+        const uint32_t w = (uint32_t)jb.w, len = n ? min((uint32_t)kChunk, n - q0) : 0u;
+        if (lane == 0) s_ji = ji;
+        if (len > 0 && jb.vec && !(len & 3u)) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive_tx(&full, 4u * len);
+            __syncwarp();
+            if (jb.pitch == jb.w) {
+                if (lane == 0) bulk_load(el, jb.src + q0, 4u * len, &full);
             } else {
-                const int ssi = (int)((ss >> (8 * p)) & 0xFFu) - 1;
-                const uint32_t b = (uint32_t)(s[p] - (int)W.cq[W.rl[p][ssi]]);   // offset in the span
-                B[p] = b;
-                cost[p] = (uint32_t)L[p] + (((b + (uint32_t)L[p] + 127u) >> 7) - ((b + 127u) >> 7));
-            }
-        }
-        // four scans at once: planes 0,1 and 2,3 in 16-bit halves
-        const uint32_t a = cost[0] | (cost[1] << 16), bb = cost[2] | (cost[3] << 16);
-        uint32_t ia = a, ib = bb;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t ya = __shfl_up_sync(0xffffffffu, ia, o), yb = __shfl_up_sync(0xffffffffu, ib, o);
-            if (lane >= o) { ia += ya; ib += yb; }
-        }
-        const uint32_t ta = __shfl_sync(0xffffffffu, ia, 31), tb = __shfl_sync(0xffffffffu, ib, 31);
-        const uint32_t ea = ia - a, eb = ib - bb;
-        const uint32_t ex[4] = {ea & 0xFFFFu, ea >> 16, eb & 0xFFFFu, eb >> 16};
-        const uint32_t tot[4] = {ta & 0xFFFFu, ta >> 16, tb & 0xFFFFu, tb >> 16};
-#pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            const uint32_t o = carry[p] + ex[p];
-            carry[p] += tot[p];
-            if (i >= n[p] || o + cost[p] > (uint32_t)kStagePlane) continue;   // (never exceeds: kStagePlane)
-            uint8_t* ob = stage + p * kStagePlane;
-            const uint8_t v = (uint8_t)(W.ce[W.rl[p][i]] >> (8 * p));
-            if (!((shm >> p) & 1u)) {
-                uint32_t q = o;
-                for (int rr = L[p]; rr > 0; rr -= 128) {
-                    ob[q] = (uint8_t)(127 + min(rr, 128));
-                    ob[q + 1] = v;
-                    q += 2;
-                }
-            } else {
-                const uint32_t b = B[p];
-                const uint32_t so = o - b - ((b + 127u) >> 7);   // the span's first control byte
-                for (uint32_t x = b; x < b + (uint32_t)L[p]; ++x) {
-                    ob[so + x + (x >> 7) + 1u] = v;
-                    if ((x & 127u) == 127u) ob[so + 129u * (x >> 7)] = 127u;
-                }
-                if (!((nshm >> p) & 1u)) {            // the span's last run: its last token
-                    const uint32_t last = b + (uint32_t)L[p] - 1u;
-                    ob[so + 129u * (last >> 7)] = (uint8_t)(last & 127u);
+                const uint32_t y0 = row_of(jb, q0), y1 = row_of(jb, q0 + len - 1u);
+                for (uint32_t y = y0 + (uint32_t)lane; y <= y1; y += 32) {
+                    const uint32_t a = y == y0 ? q0 - y0 * w : 0u;           // first column of the row's part
+                    const uint32_t b = min(w, q0 + len - y * w);             // its end column
+                    bulk_load(el + (y * w + a - q0), jb.src + (size_t)y * jb.pitch + a, 4u * (b - a), &full);
                 }
             }
         }
     }
+    __syncthreads();
+    const RleJobDesc& jb = J.j[s_ji];
+    if (jb.n_chunks == 0) return;                     // an empty image: its header is the scan's
+    const uint32_t q0 = (unit - jb.first_unit) * (uint32_t)kChunk;
+    const int len = (int)min((uint32_t)kChunk, (uint32_t)jb.w * (uint32_t)jb.h - q0);
+    if (jb.vec && !(len & 3)) {
+        mbar_wait(&full, 0u, status);
+    } else {                                          // (also a contiguous image that ends inside a 16-byte group)
+        const uint32_t w = (uint32_t)jb.w;
+        uint32_t y = row_of(jb, q0 + (uint32_t)tid), x = q0 + (uint32_t)tid - y * w;
+        for (int i = tid; i < len; i += kCT) {
+            cp_async4(el + i, jb.src + (size_t)y * jb.pitch + x);
+            x += (uint32_t)kCT;
+            if (w >= (uint32_t)kCT) {
+                if (x >= w) { x -= w; ++y; }
+            } else {
+                y = row_of(jb, q0 + (uint32_t)(i + kCT));
+                x = q0 + (uint32_t)(i + kCT) - y * w;
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+    }
+    // flags of the lane's 32 elements; its 16-byte groups are taken from the
+    // (lane mod 8)-th on, so that eight lanes' reads meet different banks
+    const int p0 = 1024 * warp + 32 * lane;
+    uint32_t F = 0u, pv = el[p0 + 4 * (lane & 7) - 1];
 #pragma unroll
-    for (int p = 0; p < 4; ++p) T[p] = carry[p];
+    for (int j = 0; j < 8; ++j) {
+        const int g = (j + lane) & 7;
+        const uint4 v = *reinterpret_cast<const uint4*>(el + p0 + 4 * g);
+        if (j > 0 && g == 0) pv = el[p0 - 1];
+        uint32_t f = v.x != pv ? 1u : 0u;
+        if (v.y != v.x) f |= 2u;
+        if (v.z != v.y) f |= 4u;
+        if (v.w != v.z) f |= 8u;
+        F |= f << (4 * g);
+        pv = v.w;
+    }
+    if (tid == 0) F |= 1u;                            // position 0 is always listed
+    if (len < kChunk) {
+        const int left = len - p0;
+        if (left < 32) F &= left <= 0 ? 0u : (1u << left) - 1u;
+    }
+    const int own = __popc(F), incl = rlec::warp_incl_sum(own, lane);
+    if (lane == 31) s_cnt[warp] = (uint32_t)incl;
+    __syncthreads();
+    const uint32_t n0 = s_cnt[0], n1 = s_cnt[1], n2 = s_cnt[2], n3 = s_cnt[3];
+    const int m = (int)(n0 + n1 + n2 + n3);
+    if (m > kCap) {                                   // dense: coded by the recoding kernel
+        if (tid == 0) {
+            rec[unit] = ChunkRec{{0, 0, 0, 0}, kRecode, 0u};
+            recode[atomicAdd(ticket + 1, 1u)] = unit;
+        }
+        return;
+    }
+    {
+        uint32_t o = (uint32_t)(incl - own) + (warp > 0 ? n0 : 0u) + (warp > 1 ? n1 : 0u) + (warp > 2 ? n2 : 0u);
+        for (; F; F &= F - 1u) cq[o++] = (uint16_t)(p0 + __ffs(F) - 1);
+    }
+    __syncthreads();
+    const bool sw = jb.mode == 2;
+    uint32_t T = 0u;
+    if (m <= 32) {
+        const int q = lane < m ? (int)cq[lane] : 0;
+        uint32_t e = el[q];
+        if (sw) e = swizzle(e);
+        T = code_plane_few(lane < m, (e >> (8 * warp)) & 0xFFu, q, len, stage[warp]);
+    }
+    if (T == 0u) T = code_plane_many(el, cq, m, 8 * warp, sw, len, stage[warp]);
+    if (lane == 0) s_T[warp] = T;
+    __syncthreads();
+    const uint32_t T0 = s_T[0], T1 = s_T[1], T2 = s_T[2], T3 = s_T[3], total = T0 + T1 + T2 + T3;
+    // The unit's own slot, or space behind the slots (+ 4: the copy to its place
+    // reads up to one word past a chunk's bytes).  The last 32-byte sector is
+    // filled up: a sector written in part would be fetched from memory when it
+    // is read.
+    const size_t slots = kRlePoolPerUnit * (size_t)J.total_units;
+    const uint32_t need = (total + 4u + 31u) & ~31u;
+    uint32_t po = kRecode;
+    if (need <= kRlePoolPerUnit && kRlePoolPerUnit * ((size_t)unit + 1) <= pool_bytes)
+        po = unit * (uint32_t)(kRlePoolPerUnit / 4);
+    if (po == kRecode) {
+        if (tid == 0) {
+            const unsigned long long a = slots + atomicAdd(reinterpret_cast<unsigned long long*>(ticket + 2),
+                                                           (unsigned long long)need);
+            s_po = a + need <= pool_bytes ? (uint32_t)(a >> 2) : kRecode;
+        }
+        __syncthreads();
+        po = s_po;
+    }
+    if (po != kRecode) {                              // the streams one after the other, then whole sectors
+        uint8_t* flat = reinterpret_cast<uint8_t*>(el) + (warp > 0 ? T0 : 0u) + (warp > 1 ? T1 : 0u) + (warp > 2 ? T2 : 0u);
+        for (uint32_t i = lane; i < T; i += 32) flat[i] = stage[warp][i];
+        __syncthreads();
+        uint4* o = reinterpret_cast<uint4*>(pool + 4 * (size_t)po);
+        for (uint32_t i = tid; 16u * i < need; i += kCT) o[i] = reinterpret_cast<const uint4*>(el)[i];
+    }
+    if (tid == 0) {
+        rec[unit] = ChunkRec{{(uint16_t)T0, (uint16_t)T1, (uint16_t)T2, (uint16_t)T3}, po, 0u};
+        if (po == kRecode) recode[atomicAdd(ticket + 1, 1u)] = unit;   // coded again when placed
+    }
 }
 
 // Four 16-bit lanes in two words (planes 0,1 | planes 2,3).
@@ -649,14 +688,6 @@ __device__ __forceinline__ uint32_t bit_range(int lo, int hi)
     return hi > lo ? ((1u << hi) - 1u) & ~((1u << lo) - 1u) : 0u;
 }
 
-// Elements [q, q + 4) of the chunk (q a multiple of 4), swizzled in mode 2.
-__device__ __forceinline__ uint4 load4(const RleJobDesc& jb, uint32_t q0, int len, int q, bool sw)
-{
-    uint4 v = load_elems(jb, q0, len, q);
-    if (sw) { v.x = swizzle(v.x); v.y = swizzle(v.y); v.z = swizzle(v.z); v.w = swizzle(v.w); }
-    return v;
-}
-
 // Dense path, a CTA of 8 warps per chunk: every position is classified with
 // byte-SIMD bit masks, all four planes at once.  Warp k takes positions
 // [512 k, 512 k + 512): lane l holds positions [P0, P0 + 16), P0 = 16 (32 k +
@@ -665,41 +696,39 @@ __device__ __forceinline__ uint4 load4(const RleJobDesc& jb, uint32_t q0, int le
 // byte lies in a repeat iff one of the three windows of 3 around it is
 // constant.  A max-scan of segment starts (warp scans, then the warps' totals
 // through shared memory) cuts tokens every 128 bytes of a segment, and a
-// sum-scan of output bytes (likewise) places them.  Without EMIT the plane
-// stream sizes are returned in T; with EMIT (T holding them) the streams are
-// written to out.  xw: 16 P4 of shared memory.
-template <bool EMIT>
-__device__ void dense_chunk(const RleJobDesc& jb, uint32_t q0, int len, bool sw, uint32_t* T, uint8_t* out, P4* xw)
+// sum-scan of output bytes (likewise) places them.  The four streams go to
+// `stage` back to back, their sizes to T.  The stage takes the scattered bytes:
+// a lane's literals are written in position order, one predicated store each,
+// so the lanes of a warp stay together whatever their tokens.  xw: 16 P4 of
+// shared memory.  The caller synchronises before it reads the stage.
+// Bound by instruction issue: the dense chunks of 8 shaded 1920x1080 sources
+// (colour and depth, 68 MB) take 99 us, and 12 us to be copied to their place;
+// sizing them (45 us) and coding them again to their place with scattered
+// byte stores (134 us) came before.
+__device__ __forceinline__ void dense_chunk(const RleJobDesc& jb, uint32_t q0, int len, bool sw, uint32_t* T,
+                                            uint8_t* stage, P4* xw)
 {
     const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
     const bool act = 512 * k < len;                          // (uniform in the warp)
-    uint32_t pbase[4] = {0u, 0u, 0u, 0u};
-    if (EMIT) {
-        pbase[1] = T[0];
-        pbase[2] = T[0] + T[1];
-        pbase[3] = T[0] + T[1] + T[2];
-    }
     const int P0 = 16 * (32 * k + lane);
     uint32_t REP[4] = {0u, 0u, 0u, 0u}, SEG[4] = {0u, 0u, 0u, 0u};
     uint4 bytes[4];
     uint32_t VALID = 0u;
     P4 mine = {0u, 0u};
+    // plane words of positions [q, q + 4) (word b = plane b)
+    auto load_planes = [&](int q) {
+        const uint4 g = load_elems(jb, q0, len, q);
+        uint4 t = transpose4(g.x, g.y, g.z, g.w);
+        if (sw) rlec::swizzle_planes(t.x, t.y, t.z, t.w);
+        return t;
+    };
     if (act) {
         uint4 t[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const uint4 g = load4(jb, q0, len, P0 + 4 * i, sw);
-            t[i] = transpose4(g.x, g.y, g.z, g.w);              // t[i] word b = plane b of 4 positions
-        }
+        for (int i = 0; i < 4; ++i) t[i] = load_planes(P0 + 4 * i);
         uint4 tn = make_uint4(0u, 0u, 0u, 0u), tp = make_uint4(0u, 0u, 0u, 0u);
-        if (lane == 31) {
-            const uint4 g = load4(jb, q0, len, P0 + 16, sw);
-            tn = transpose4(g.x, g.y, g.z, g.w);
-        }
-        if (lane == 0 && P0 > 0) {
-            const uint4 g = load4(jb, q0, len, P0 - 4, sw);
-            tp = transpose4(g.x, g.y, g.z, g.w);
-        }
+        if (lane == 31) tn = load_planes(P0 + 16);
+        if (lane == 0 && P0 > 0) tp = load_planes(P0 - 4);
         const uint32_t VQ = bit_range(4 - P0, len - P0 + 4);          // 0 <= q < len
         const uint32_t VEQ = bit_range(5 - P0, len - P0 + 4);         // 1 <= q < len
         const uint32_t HIGH = bit_range(len - P0 + 4, 24);            // q >= len
@@ -746,7 +775,7 @@ __device__ void dense_chunk(const RleJobDesc& jb, uint32_t q0, int len, bool sw,
     P4 before = smax;
     for (int j = 0; j < k; ++j) before = combine<true>(before, xw[j]);
     // piece starts (tokens hold <= 128 bytes) and output sizes
-    uint32_t PSV[4], PE[4], LIT[4], cost[4];
+    uint32_t PSV[4], PE[4], cost[4];
     int sbin[4];
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
@@ -764,8 +793,7 @@ __device__ void dense_chunk(const RleJobDesc& jb, uint32_t q0, int len, bool sw,
         const uint32_t next = ((SEG[b] >> 16) & 1u) | (((P0 + 16 - sb15) & 127) == 0 ? 1u : 0u);
         PSV[b] = PS & VALID;
         PE[b] = ((PS | (next << 16)) >> 1) & VALID;
-        LIT[b] = ~REP[b] & VALID;
-        cost[b] = __popc(LIT[b]) + __popc(PSV[b]) + __popc(PSV[b] & REP[b]);
+        cost[b] = __popc(~REP[b] & VALID) + __popc(PSV[b]) + __popc(PSV[b] & REP[b]);
     }
     P4 tsum = {0u, 0u}, ssum = {0u, 0u};
     if (act) ssum = warp_scan4<false>(P4{cost[0] | (cost[1] << 16), cost[2] | (cost[3] << 16)}, lane, &tsum);
@@ -778,42 +806,54 @@ __device__ void dense_chunk(const RleJobDesc& jb, uint32_t q0, int len, bool sw,
         if (j < k) off0 = combine<false>(off0, x);
         total = combine<false>(total, x);
     }
-    __syncthreads();                                         // xw is reused by the next chunk
 #pragma unroll
-    for (int b = 0; b < ((EMIT && act) ? 4 : 0); ++b) {
-        uint8_t* o = out + pbase[b];
-        const uint32_t off = lane16(off0, b);
-        const uint32_t lit = LIT[b], psv = PSV[b], psr = PSV[b] & REP[b], seg16 = SEG[b] & 0xFFFFu;
-        const uint4 v = bytes[b];
-        auto byte_at = [&](int i) -> uint8_t {
-            const uint32_t wd = i < 8 ? (i < 4 ? v.x : v.y) : (i < 12 ? v.z : v.w);
-            return (uint8_t)(wd >> (8 * (i & 3)));
-        };
-        auto inc_at = [&](int i) -> uint32_t {
-            const uint32_t le = (2u << i) - 1u;
-            return off + __popc(lit & le) + __popc(psv & le) + __popc(psr & le);
-        };
-        for (uint32_t m = lit; m; m &= m - 1u) {
-            const int i = __ffs(m) - 1;
-            o[inc_at(i) - 1] = byte_at(i);
-        }
-        for (uint32_t m = PE[b]; m; m &= m - 1u) {
-            const int i = __ffs(m) - 1;
-            const uint32_t inc = inc_at(i);
-            const uint32_t h = seg16 & ((2u << i) - 1u);
-            const int sbk = h ? P0 + 31 - __clz(h) : sbin[b];
-            const uint32_t jj = (uint32_t)(P0 + i - sbk) & 127u;
-            if ((REP[b] >> i) & 1u) {
-                o[inc - 2] = (uint8_t)(0x80u + jj);
-                o[inc - 1] = byte_at(i);
-            } else {
-                o[inc - 2 - jj] = (uint8_t)jj;
+    for (int b = 0; b < 4; ++b) T[b] = lane16(total, b);
+    uint8_t* plane = stage;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        if (act) {
+            uint8_t* const o = plane + lane16(off0, b);
+            const uint32_t lit = ~REP[b] & VALID, psv = PSV[b], rep = REP[b], seg16 = SEG[b] & 0xFFFFu;
+            const uint4 v = bytes[b];
+            // literal bytes in position order; a piece start leaves room for its
+            // control byte, a repeat's for its value too.  Warps without
+            // literals skip the pass, warps of literals only (noise) need no
+            // tests for them.
+            uint8_t* w = o;
+            if (__all_sync(0xffffffffu, lit == 0xFFFFu)) {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const uint32_t wd = i < 4 ? v.x : i < 8 ? v.y : i < 12 ? v.z : v.w;
+                    w += (psv >> i) & 1u;
+                    w[i] = (uint8_t)(wd >> (8 * (i & 3)));
+                }
+            } else if (__any_sync(0xffffffffu, lit != 0u)) {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const uint32_t wd = i < 4 ? v.x : i < 8 ? v.y : i < 12 ? v.z : v.w;
+                    if ((psv >> i) & 1u) w += 1 + ((rep >> i) & 1u);
+                    if ((lit >> i) & 1u) *w++ = (uint8_t)(wd >> (8 * (i & 3)));
+                }
+            }
+            // control bytes, at the pieces' ends
+            for (uint32_t m = PE[b]; m; m &= m - 1u) {
+                const int i = __ffs(m) - 1;
+                const uint32_t le = (2u << i) - 1u;
+                uint8_t* const e = o + __popc(lit & le) + __popc(psv & le) + __popc(psv & rep & le);   // past the piece
+                const uint32_t h = seg16 & le;
+                const int sbk = h ? P0 + 31 - __clz(h) : sbin[b];
+                const uint32_t jj = (uint32_t)(P0 + i - sbk) & 127u;
+                if ((rep >> i) & 1u) {
+                    const uint32_t wd = i < 8 ? (i < 4 ? v.x : v.y) : (i < 12 ? v.z : v.w);
+                    e[-2] = (uint8_t)(0x80u + jj);
+                    e[-1] = (uint8_t)(wd >> (8 * (i & 3)));
+                } else {
+                    *(e - 2 - jj) = (uint8_t)jj;
+                }
             }
         }
+        plane += T[b];
     }
-    if (!EMIT)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) T[b] = lane16(total, b);
 }
 
 // ---- basic RLE (mode 0) on the same pipeline --------------------------------
@@ -838,13 +878,15 @@ __device__ __forceinline__ void put8(uint8_t* p, uint32_t lo, uint32_t hi)
 }
 
 // Append the unit change points among units [kQ/2 qi, kQ/2 qi + kQ/2) of the
-// chunk (unit k = elements 2k, 2k + 1) to W.cq (the unit's index) and W.ce /
-// the second list `ch` (its two elements), as detect_quarter does for
-// elements: a lane's 16-byte group holds two units.  carry: the unit before
-// the quarter (updated to the quarter's last).  Returns false once the chunk
-// has more than kCap change points.
-__device__ bool detect_quarter0(const uint32_t* data, int len, int qi, WarpRing& W, uint32_t* ch, int& m,
-                                uint2& carry)
+// chunk (unit k = elements 2k, 2k + 1) to W.cq (the unit's index) and W.ce,
+// W.ch (its two elements); a lane's 16-byte group holds two units.  Every lane
+// flags the changes in its group of each of the quarter's four 128-element
+// groups; one warp scan of the four per-lane counts, packed in the bytes of a
+// word (a group has at most 64 changes, so no byte carries into the next),
+// places them all in order.  carry: the unit before the quarter (updated to the
+// quarter's last).  Returns false once the chunk has more than kCap change
+// points.
+__device__ bool detect_quarter0(const uint32_t* data, int len, int qi, WarpRing& W, int& m, uint2& carry)
 {
     const int lane = threadIdx.x & 31;
     constexpr int G = kQ / 128;
@@ -885,8 +927,8 @@ __device__ bool detect_quarter0(const uint32_t* data, int len, int qi, WarpRing&
             const uint4 v = vv[g];
             const int uu = kQ / 2 * qi + 64 * g + 2 * lane;
             int o = base + (int)((exc >> (8 * g)) & 0xFFu);
-            if (f[g] & 1u) { W.cq[o] = (uint16_t)uu; W.ce[o] = v.x; ch[o] = v.y; ++o; }
-            if (f[g] & 2u) { W.cq[o] = (uint16_t)(uu + 1); W.ce[o] = v.z; ch[o] = v.w; }
+            if (f[g] & 1u) { W.cq[o] = (uint16_t)uu; W.ce[o] = v.x; W.ch[o] = v.y; ++o; }
+            if (f[g] & 2u) { W.cq[o] = (uint16_t)(uu + 1); W.ce[o] = v.z; W.ch[o] = v.w; }
         }
         base += (int)((tot >> (8 * g)) & 0xFFu);
     }
@@ -1096,19 +1138,19 @@ __device__ uint32_t code0_block(const RleJobDesc& jb, uint32_t q0, int len, uint
     return body + ((len & 1) ? 4u : 0u);
 }
 
-// Coding kernel.  Per chunk a warp: takes its next ticket; reads the chunk's
-// eight quarters, refilling each slot as soon as it has been read (with the
-// next quarter of this chunk or of the next one); sizes the plane streams;
-// and leaves the chunk's record and, for a sparse chunk, its streams in the
+// Mode-0 coding kernel.  Per chunk a warp: takes its next ticket; reads the
+// chunk's eight quarters, refilling each slot as soon as it has been read (with
+// the next quarter of this chunk or of the next one); codes the stream; and
+// leaves the chunk's record and, for a sparse chunk, its stream in the
 // pool (space from the warp's slab, a fresh slab taken with one atomic on the
 // pool cursor when the chunk does not fit, or from the cursor chunk by chunk
 // when slab is 0; a chunk that finds the pool full is coded again when
 // placed, like a dense one; such chunks are listed for the recoding kernel).
-// No warp waits for another.  M0: basic RLE (mode 0), from unit change points.
-template <int N, bool M0>
+// No warp waits for another.
+template <int N>
 __global__ void __launch_bounds__(32 * kWPB, 16)
-k_rle_compress(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, uint32_t* recode, uint8_t* pool,
-               uint32_t pool_bytes, uint32_t slab, uint32_t* ticket, uint32_t* status)
+k_rle_compress0(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, uint32_t* recode, uint8_t* pool,
+                uint32_t pool_bytes, uint32_t slab, uint32_t* ticket, uint32_t* status)
 {
     extern __shared__ __align__(16) uint8_t smem[];
     WarpRing& W = reinterpret_cast<WarpRing*>(smem)[threadIdx.x >> 5];
@@ -1127,7 +1169,7 @@ k_rle_compress(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, uint32_t*
     int ji = cur < T ? find_job(J, cur) : 0;            // job of the current chunk
     if (cur < T)
         for (int q = 0; q < kSlots; ++q) issue_quarter(J.j[ji], cur, q, q, W);
-    for (uint32_t seq = 0; cur < T; ++seq) {
+    for (uint32_t qs = 0; cur < T;) {                   // qs: the warp's quarter sequence number
         uint32_t nxt = 0u;
         if (lane == 0) nxt = atomicAdd(ticket, 1u);
         nxt = __shfl_sync(0xffffffffu, nxt, 0);
@@ -1137,47 +1179,37 @@ k_rle_compress(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, uint32_t*
         const uint32_t q0 = nc ? (cur - jb.first_unit) * (uint32_t)kChunk : 0u;
         const int len = nc ? (int)min((uint32_t)kChunk, (uint32_t)jb.w * (uint32_t)jb.h - q0) : 0;
         int m = 0;
-        uint32_t carry = 0u;
-        uint2 carry2 = make_uint2(0u, 0u);
-        uint32_t* ch = reinterpret_cast<uint32_t*>(W.rl);    // mode 0: second element of each listed unit
+        uint2 carry = make_uint2(0u, 0u);
         bool fits = true;
-        for (int q = 0; q < kQPC; ++q) {
-            const uint32_t qs = (uint32_t)kQPC * seq + (uint32_t)q;   // the warp's quarter sequence number
+        // quarters [0, issued) of this chunk are in flight or read; once the chunk
+        // proves dense its remaining quarters are not fetched, and the slots go
+        // to the next chunk
+        int issued = kSlots;
+        for (int q = 0; q < issued; ++q, ++qs) {
             const int slot = (int)(qs % kSlots);
             mbar_wait(&W.full[slot], (qs / kSlots) & 1u, status);
-            if (fits && kQ * q < len)
-                fits = M0 ? detect_quarter0(W.buf[slot] + 4, len, q, W, ch, m, carry2)
-                          : detect_quarter(W.buf[slot] + 4, len, q, W, m, carry);
+            if (fits && kQ * q < len) fits = detect_quarter0(W.buf[slot] + 4, len, q, W, m, carry);
             // the quarter's values have all been consumed (compared, voted on) by
             // now, so its reads are complete before the refill below starts
             __syncwarp();
-            // refill the slot with quarter qs + kSlots: of this chunk or of the next
-            const int qn = q + kSlots;
-            if (qn < kQPC) issue_quarter(jb, cur, qn, slot, W);
-            else if (nxt < T) issue_quarter(J.j[jn], nxt, qn - kQPC, slot, W);
+            // refill the slot with the next quarter, of this chunk or of the next
+            if (fits && issued < kQPC) issue_quarter(jb, cur, issued++, slot, W);
+            else if (nxt < T) issue_quarter(J.j[jn], nxt, q + kSlots - issued, slot, W);
         }
         if (nc > 0) {
-            const bool sw = jb.mode == 2;
-            uint32_t Ts[4] = {0u, 0u, 0u, 0u};          // (a dense chunk is sized by the recoding kernels)
-            if (fits && M0) {
+            uint32_t total = 0u;                        // (a dense chunk is sized by the recoding kernel)
+            if (fits) {
                 __syncwarp();
-                Ts[0] = code_sparse0(W.ce, ch, W.cq, m, len / 2, W.stage);
+                total = code_sparse0(W.ce, W.ch, W.cq, m, len / 2, W.stage);
                 if (len & 1) {                            // the odd last element follows the tokens
-                    if (lane == 0) put_u32(W.stage + Ts[0], __ldg(jb.src + elem_off(jb, q0 + (uint32_t)len - 1u)));
-                    Ts[0] += 4u;
+                    if (lane == 0) put_u32(W.stage + total, __ldg(jb.src + elem_off(jb, q0 + (uint32_t)len - 1u)));
+                    total += 4u;
                 }
-            } else if (fits) {
-                __syncwarp();
-                if (sw)
-                    for (int i = lane; i < m; i += 32) W.ce[i] = swizzle(W.ce[i]);
-                const Lists L{W.ce, W.cq, W.rl};
-                if (!code_sparse_fast(L, m, len, Ts, W.stage)) code_sparse(L, m, len, Ts, W.stage);
             }
-            const uint32_t total = Ts[0] + Ts[1] + Ts[2] + Ts[3];
             uint32_t po = kRecode;
             if (fits && lane == 0) {
                 // (+ 4: the copy-out reads up to one word past a chunk's bytes)
-                const uint32_t need = (total + 3u) & ~3u;
+                const uint32_t need = (total + 15u) & ~15u;
                 if (slab == 0u) {                         // small pools: space per chunk
                     const unsigned long long a = atomicAdd(cursor, (unsigned long long)need);
                     if (a + total + 4u <= pool_bytes) po = (uint32_t)a;
@@ -1194,18 +1226,12 @@ k_rle_compress(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, uint32_t*
             }
             po = __shfl_sync(0xffffffffu, po, 0);
             __syncwarp();
-            if (po != kRecode) {                      // the four streams, back to back
-                const uint32_t e1 = Ts[0], e2 = e1 + Ts[1], e3 = e2 + Ts[2];
-                for (uint32_t i = lane; i < total; i += 32) {
-                    const int p = (i >= e1) + (i >= e2) + (i >= e3);
-                    const uint32_t b = p == 0 ? 0u : p == 1 ? e1 : p == 2 ? e2 : e3;
-                    pool[po + i] = W.stage[p * kStagePlane + (i - b)];
-                }
-            }
+            if (po != kRecode)
+                for (uint32_t i = lane; i < total; i += 32) pool[po + i] = W.stage[i];
             if (lane == 0) {
                 ChunkRec r;
-                r.T[0] = (uint16_t)Ts[0]; r.T[1] = (uint16_t)Ts[1]; r.T[2] = (uint16_t)Ts[2]; r.T[3] = (uint16_t)Ts[3];
-                r.pool = po;
+                r.T[0] = (uint16_t)total; r.T[1] = r.T[2] = r.T[3] = 0;
+                r.pool = po == kRecode ? kRecode : po >> 2;
                 r.off = 0u;
                 rec[cur] = r;
                 if (po == kRecode) recode[atomicAdd(ticket + 1, 1u)] = cur;   // coded again when placed
@@ -1264,7 +1290,7 @@ k_rle_scan(const __grid_constant__ RleJobList<N> J, ChunkRec* rec)
 // Placing kernel: kPlaceLanes lanes (a quarter-warp) per chunk copy its
 // streams from the pool to their place and write its end-table entries (four;
 // one in mode 0), so a warp's four chunks have their loads in flight together.
-// Chunks to be coded again are left to the recoding kernel.
+// Listed chunks (dense, or to be coded again) are left to the recoding kernel.
 constexpr int kPlaceLanes = 8;
 template <int N>
 __global__ void __launch_bounds__(128)
@@ -1277,54 +1303,84 @@ k_rle_place(const __grid_constant__ RleJobList<N> J, const ChunkRec* rec, const 
     const RleJobDesc& jb = J.j[find_job(J, unit)];
     const uint32_t nc = jb.n_chunks;
     if (nc == 0) return;                              // header written by the scan
-    if (r.pool == kRecode) return;
+    if (r.pool & kDense) return;                      // (kRecode too: the recoding kernel's)
+    const uint8_t* from = pool + 4ull * r.pool;
     const uint32_t c = unit - jb.first_unit;
     const uint32_t T0 = r.T[0], T1 = r.T[1], T2 = r.T[2], T3 = r.T[3];
     const uint32_t total = T0 + T1 + T2 + T3;
     uint8_t* dst = reinterpret_cast<uint8_t*>(jb.dst);
     if (jb.mode == 0) {                               // one stream, one end-table entry
-        copy_out(dst + 32 + 4ull * nc + r.off, pool + r.pool, total, lane, kPlaceLanes);
+        copy_out(dst + 32 + 4ull * nc + r.off, from, total, lane, kPlaceLanes);
         if (lane == 0) put_u32(dst + 32 + 4ull * c, r.off + total);
         return;
     }
-    copy_out(dst + 32 + 16ull * nc + r.off, pool + r.pool, total, lane, kPlaceLanes);
+    copy_out(dst + 32 + 16ull * nc + r.off, from, total, lane, kPlaceLanes);
     const uint32_t mine = lane == 0 ? T0 : lane == 1 ? T0 + T1 : lane == 2 ? T0 + T1 + T2 : total;
     if (lane < 4) put_u32(dst + 32 + 16ull * c + 4u * lane, r.off + mine);
 }
 
 // Recoding kernels: the listed chunks (dense, or sparse ones that found the
-// pool full) are coded from the image, a CTA of 8 warps per listed chunk over
-// a persistent grid.  Before the scan (EMIT false) the dense ones are sized,
-// their sizes written to their records; after it (EMIT true) every listed
-// chunk is written straight to its place with its four end-table entries.
-template <int N, bool EMIT>
-__global__ void __launch_bounds__(256)
-k_rle_recode(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, const uint32_t* recode, const uint32_t* count)
+// pool full), a CTA of 8 warps per listed chunk over a persistent grid.  Before
+// the scan (PLACE false) the dense ones are coded from the image into the
+// stage; their sizes go to their records and, where the pool has room, their
+// streams to the pool with 16-byte stores.  After it (PLACE true) the pooled
+// ones are copied to their place, the others coded (again) from the image and
+// copied from the stage; both write the four end-table entries.
+constexpr int kDenseStage = 4 * (kChunk + kChunk / 128) + 64;   // all literals, copy_out's read-ahead, whole sectors
+
+template <int N, bool PLACE>
+__global__ void __launch_bounds__(256, 4)
+k_rle_recode(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, const uint32_t* recode, uint32_t* ticket,
+             uint8_t* pool, size_t pool_bytes)
 {
     __shared__ P4 xw[16];
-    const uint32_t n = *count;
+    __shared__ __align__(16) uint8_t stage[kDenseStage];
+    __shared__ uint32_t s_pool;
+    const uint32_t n = ticket[1];
+    const int tid = threadIdx.x;
     for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) {
         const uint32_t unit = recode[i];
         const RleJobDesc& jb = J.j[find_job(J, unit)];
         const uint32_t nc = jb.n_chunks, c = unit - jb.first_unit;
         const ChunkRec r = rec[unit];
         uint32_t T[4] = {r.T[0], r.T[1], r.T[2], r.T[3]};
-        const uint32_t total = T[0] + T[1] + T[2] + T[3];
-        uint8_t* dst = reinterpret_cast<uint8_t*>(jb.dst);
         const uint32_t q0 = c * (uint32_t)kChunk;
         const int len = (int)min((uint32_t)kChunk, (uint32_t)jb.w * (uint32_t)jb.h - q0);
-        if (!EMIT) {
-            if (total != 0u) continue;                    // sized already (a sparse chunk)
-            dense_chunk<false>(jb, q0, len, jb.mode == 2, T, nullptr, xw);
-            if (threadIdx.x == 0)
-#pragma unroll
-                for (int p = 0; p < 4; ++p) rec[unit].T[p] = (uint16_t)T[p];
-            continue;
+        if (!PLACE) {
+            if (T[0] != 0u) continue;                         // sized already (a sparse chunk)
+            dense_chunk(jb, q0, len, jb.mode == 2, T, stage, xw);
+            const uint32_t total = T[0] + T[1] + T[2] + T[3];
+            if (tid == 0) {
+                const uint32_t need = (total + 4u + 31u) & ~31u;
+                const unsigned long long a = kRlePoolPerUnit * (unsigned long long)J.total_units +
+                    atomicAdd(reinterpret_cast<unsigned long long*>(ticket + 2), (unsigned long long)need);
+                s_pool = a + need <= pool_bytes ? kDense | (uint32_t)(a >> 4) : kRecode;
+                ChunkRec o;
+                o.T[0] = (uint16_t)T[0]; o.T[1] = (uint16_t)T[1]; o.T[2] = (uint16_t)T[2]; o.T[3] = (uint16_t)T[3];
+                o.pool = s_pool;
+                o.off = 0u;
+                rec[unit] = o;
+            }
+            __syncthreads();                                  // the stage is complete
+            if (s_pool != kRecode) {
+                uint4* to = reinterpret_cast<uint4*>(pool + ((size_t)(s_pool & ~kDense) << 4));
+                for (uint32_t j = tid; 32u * (j >> 1) < total + 4u; j += 256u)   // (whole 32-byte sectors)
+                    to[j] = reinterpret_cast<const uint4*>(stage)[j];
+            }
+        } else {
+            uint8_t* dst = reinterpret_cast<uint8_t*>(jb.dst);
+            const uint8_t* from = pool + ((size_t)(r.pool & ~kDense) << 4);
+            if (r.pool == kRecode) {
+                dense_chunk(jb, q0, len, jb.mode == 2, T, stage, xw);
+                __syncthreads();
+                from = stage;
+            }
+            const uint32_t total = T[0] + T[1] + T[2] + T[3];
+            copy_out(dst + 32 + 16ull * nc + r.off, from, total, tid, 256);
+            const uint32_t mine = tid == 0 ? T[0] : tid == 1 ? T[0] + T[1] : tid == 2 ? T[0] + T[1] + T[2] : total;
+            if (tid < 4) put_u32(dst + 32 + 16ull * c + 4u * tid, r.off + mine);
         }
-        dense_chunk<true>(jb, q0, len, jb.mode == 2, T, dst + 32 + 16ull * nc + r.off, xw);
-        const uint32_t t = threadIdx.x;
-        const uint32_t mine = t == 0 ? T[0] : t == 1 ? T[0] + T[1] : t == 2 ? T[0] + T[1] + T[2] : total;
-        if (t < 4) put_u32(dst + 32 + 16ull * c + 4u * t, r.off + mine);
+        __syncthreads();                                      // stage and xw are reused
     }
 }
 
@@ -1665,8 +1721,8 @@ RleJobList<N> make_jobs(const RleJobDesc* jobs, int n, uint32_t total)
 
 namespace {
 
-// Persistent grid: as many coding CTAs as fit on the device at once.
-template <int N, bool M0>
+// Mode 0's persistent grid: as many coding CTAs as fit on the device at once.
+template <int N>
 cudaError_t compress_grid(int* grid)
 {
     constexpr int kMaxDev = 64;
@@ -1675,15 +1731,15 @@ cudaError_t compress_grid(int* grid)
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < kMaxDev && (*grid = cache[dev].load(std::memory_order_relaxed)) > 0) return cudaSuccess;
-    e = cudaFuncSetAttribute(k_rle_compress<N, M0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCompressSmem);
+    e = cudaFuncSetAttribute(k_rle_compress0<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCompressSmem);
     if (e != cudaSuccess) return e;
     // the persistent grid is sized for the largest shared-memory carveout:
     // ask for it, so that every CTA of the grid is resident at once
-    e = cudaFuncSetAttribute(k_rle_compress<N, M0>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    e = cudaFuncSetAttribute(k_rle_compress0<N>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     int per_sm = 0, sms = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rle_compress<N, M0>, 32 * kWPB, kCompressSmem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rle_compress0<N>, 32 * kWPB, kCompressSmem);
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
@@ -1692,54 +1748,58 @@ cudaError_t compress_grid(int* grid)
     return cudaSuccess;
 }
 
-// Code (persistent warps), size the dense chunks, scan the sizes (a CTA per
-// job), place (a warp per chunk), write the dense chunks.  M0: basic RLE.
+// Code (a CTA per chunk; in mode 0 persistent warps), code or size the dense
+// chunks, scan the sizes (a CTA per job), place (a quarter-warp per chunk), place
+// or write the dense chunks.  M0: basic RLE.
 template <int N, bool M0>
 cudaError_t compress_n(const RleJobDesc* jobs, int n, uint32_t total_units, void* scratch, size_t scratch_bytes,
                        uint32_t* status, cudaStream_t s)
 {
-    int grid = 0;
-    cudaError_t e = compress_grid<N, M0>(&grid);
-    if (e != cudaSuccess) return e;
-    grid = (int)std::min<uint32_t>((uint32_t)grid, (total_units + kWPB - 1) / kWPB);
-    uint32_t* ticket = reinterpret_cast<uint32_t*>(scratch);     // [0] ticket, [1] chunks to recode
+    cudaError_t e;
+    uint32_t* ticket = reinterpret_cast<uint32_t*>(scratch);     // [0] ticket, [1] chunks to recode, [2, 3] pool cursor
     ChunkRec* rec = reinterpret_cast<ChunkRec*>(reinterpret_cast<char*>(scratch) + 16);
     uint32_t* recode = reinterpret_cast<uint32_t*>(rec + total_units);
-    uint8_t* pool = reinterpret_cast<uint8_t*>(recode + ((total_units + 3u) & ~3u));
-    const size_t used = rle_compress_scratch_bytes(total_units, 0);
-    const uint32_t pool_bytes = (uint32_t)std::min<size_t>(scratch_bytes - used, 0xFFFFFFF0u);
-    // pool space is taken in slabs of up to 16 KB per warp where the pool
-    // has room for eight slabs per warp of the grid (their unused tails are
-    // then at most an eighth of it), else chunk by chunk
-    uint32_t slab = std::min<uint32_t>(pool_bytes / (8u * (uint32_t)grid * kWPB), 16384u) & ~255u;
-    if (slab < 4u * kStagePlane) slab = 0u;
+    const size_t used = rle_compress_scratch_bytes(total_units, 0), pool_bytes = scratch_bytes - used;
+    uint8_t* pool = reinterpret_cast<uint8_t*>(scratch) + used;
     const RleJobList<N> J = make_jobs<N>(jobs, n, total_units);
     int sms = 0;
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     const int rgrid = std::max(1, sms) * 4;
-    k_rle_compress<N, M0><<<grid, 32 * kWPB, kCompressSmem, s>>>(J, rec, recode, pool, pool_bytes, slab, ticket,
-                                                                 status);
+    if (M0) {
+        int grid = 0;
+        if ((e = compress_grid<N>(&grid)) != cudaSuccess) return e;
+        grid = (int)std::min<uint32_t>((uint32_t)grid, (total_units + kWPB - 1) / kWPB);
+        // pool space is taken in slabs of up to 16 KB per warp where the pool
+        // has room for eight slabs per warp of the grid (their unused tails are
+        // then at most an eighth of it), else chunk by chunk
+        const uint32_t pb = (uint32_t)std::min<size_t>(pool_bytes, 0xFFFFFFF0u);
+        uint32_t slab = std::min<uint32_t>(pb / (8u * (uint32_t)grid * kWPB), 16384u) & ~255u;
+        if (slab < 4u * kStagePlane) slab = 0u;
+        k_rle_compress0<N><<<grid, 32 * kWPB, kCompressSmem, s>>>(J, rec, recode, pool, pb, slab, ticket, status);
+    } else {
+        k_rle_code<N><<<total_units, kCT, 0, s>>>(J, rec, recode, pool, pool_bytes, ticket, status);
+    }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (M0) k_rle0_recode<N, false><<<rgrid, kT, 0, s>>>(J, rec, recode, ticket + 1);
-    else k_rle_recode<N, false><<<rgrid, 256, 0, s>>>(J, rec, recode, ticket + 1);
+    else k_rle_recode<N, false><<<rgrid, 256, 0, s>>>(J, rec, recode, ticket, pool, pool_bytes);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_rle_scan<N><<<n, 1024, 0, s>>>(J, rec);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_rle_place<N><<<(total_units + 128 / kPlaceLanes - 1) / (128 / kPlaceLanes), 128, 0, s>>>(J, rec, pool);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (M0) k_rle0_recode<N, true><<<rgrid, kT, 0, s>>>(J, rec, recode, ticket + 1);
-    else k_rle_recode<N, true><<<rgrid, 256, 0, s>>>(J, rec, recode, ticket + 1);
+    else k_rle_recode<N, true><<<rgrid, 256, 0, s>>>(J, rec, recode, ticket, pool, pool_bytes);
     return cudaGetLastError();
 }
 
 }  // namespace
 
-size_t rle_compress_scratch_bytes(uint32_t units, size_t pool_per_unit)
+size_t rle_compress_scratch_bytes(uint32_t units, size_t pool_bytes)
 {
     const size_t u = std::max<uint32_t>(units, 1);
-    return 16 + sizeof(ChunkRec) * u + 4 * ((u + 3) & ~(size_t)3) + pool_per_unit * u;
+    return ((16 + sizeof(ChunkRec) * u + 4 * u + 127) & ~(size_t)127) + pool_bytes;   // the pool starts at a 128-byte line
 }
 
 cudaError_t launch_rle_compress(const RleJobDesc* jobs, int n, uint32_t total_units,

@@ -85,3 +85,69 @@ def test_malformed_streams_of_many_tokens(seed):
     assert st == oracle.rle_decompress_status(bytes(buf), w, h)
     if st == 0:
         assert np.array_equal(np_of(out), oracle.rle_decompress(bytes(buf), w, h))
+
+
+def _mixed(kind, w, h, seed):
+    """Rows that take each path of the compressor: flat, a few runs, runs of one
+    to three bytes in a plane, more change points than a list holds, noise."""
+    r = np.random.default_rng(seed)
+    img = np.zeros((h, w), np.uint32)
+    flat = img.reshape(-1)
+    n = flat.size
+    if kind == "edges":                              # changes at every edge of groups, warps and chunks
+        for q in [0, 1, 3, 4, 127, 128, 511, 512, 1023, 1024, 1025, 2047, 2048, 3071, 3072, 4094, 4095, 4096, 4097, n - 1]:
+            if q < n:
+                flat[q:] ^= np.uint32(r.integers(1, 1 << 32))
+    elif kind in ("cap", "over"):                    # exactly as many change points as a list holds, and one more
+        for c0 in range(0, n, CHUNK):
+            q = np.sort(r.choice(np.arange(1, min(CHUNK, n - c0)), min(127 + (kind == "over"), n - c0 - 1), replace=False))
+            for p in q:
+                flat[c0 + p:] ^= np.uint32(1 << int(r.integers(0, 32)))
+    elif kind == "short":                            # runs of 1 to 3 in single planes
+        q = 0
+        while q < n:
+            m = int(r.integers(1, 60) if r.random() < 0.6 else r.integers(1, 4))
+            flat[q:] ^= np.uint32(int(r.integers(1, 256)) << (8 * int(r.integers(0, 4))))
+            q += m
+    else:                                            # "noise": every byte differs
+        flat[:] = r.integers(0, 1 << 32, size=n, dtype=np.uint64).astype(np.uint32)
+    return img
+
+
+@pytest.mark.parametrize("mode", [1, 2])
+@pytest.mark.parametrize("w,h", [(4096, 3), (1000, 9), (997, 13), (8193, 1), (3, 1), (130, 70)])
+@pytest.mark.parametrize("kind", ["edges", "cap", "over", "short", "noise"])
+def test_compressor_paths_match_the_oracle(kind, w, h, mode):
+    require_gpu()
+    img = _mixed(kind, w, h, [w, h, mode])
+    want = oracle.rle_compress(img, mode)
+    wide = torch.full((h, w + 3), 77, dtype=torch.int32, device="cuda")
+    wide[:, :w] = torch.from_numpy(img.view(np.int32)).cuda()
+    for src in (wide[:, :w].contiguous(), wide[:, :w]):              # one run, and rows of another pitch
+        buf, size = ec.rle_compress(src.view(torch.uint32), mode)
+        ec.default_context().check_status()
+        assert buf[:int(size.item())].cpu().numpy().tobytes() == want
+
+
+@pytest.mark.parametrize("kind", ["noise", "cap"])
+@pytest.mark.parametrize("mode", [1, 2])
+def test_compressor_with_a_full_pool(kind, mode):
+    """The allocation-free entry point's pool holds 512 bytes per chunk of its
+    largest image: with every chunk larger, the chunks that find it full are
+    coded again when placed."""
+    from paper_1902_08755_gb300 import _abi as A
+    require_gpu()
+    rows = _mixed(kind, 4096, 16, [1, mode])
+    img = np.tile(rows, (ec.EC_RLE_CHUNK * 2 // 16, 1)) if kind == "noise" else np.tile(rows, (512, 1))
+    img = img[:A.EC_RLE_NOALLOC_MAX_CHUNKS]
+    h, w = img.shape
+    src = torch.from_numpy(img.view(np.int32)).cuda()
+    dst = torch.empty(ec.rle_max_size(w, h), dtype=torch.uint8, device="cuda")
+    size, st = torch.zeros(1, dtype=torch.uint64, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    A.check(A.load().ec_rle_compress_noalloc(src.data_ptr(), w, h, w, mode, dst.data_ptr(), dst.numel(), size.data_ptr(),
+                                             st.data_ptr(), torch.cuda.current_stream().cuda_stream), "noalloc")
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    want = oracle.rle_compress(img, mode)
+    assert int(size.item()) == len(want)
+    assert dst[:len(want)].cpu().numpy().tobytes() == want
