@@ -135,6 +135,7 @@ SIGNATURES = {
 }
 
 _lib = None
+_marshal = None
 _lock = threading.Lock()
 
 
@@ -164,6 +165,16 @@ def load(build_if_missing: bool = True):
             f.argtypes = args
         _lib = L
         return _lib
+
+
+def marshal():
+    """The native argument marshalling (csrc/marshal.cpp), built with libec.so."""
+    global _marshal
+    if _marshal is None:
+        load()
+        from . import _marshal as m
+        _marshal = m
+    return _marshal
 
 
 def check(code: int, what: str):

@@ -14,6 +14,7 @@ Tensor layouts (pitch = row stride in pixels, taken from the tensor's stride):
 from __future__ import annotations
 
 import ctypes as C
+import math
 from dataclasses import dataclass
 from typing import List, Optional, Sequence, Tuple
 
@@ -31,7 +32,7 @@ def _lib():
 
 def _stream_handle(stream) -> Optional[int]:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -131,7 +132,24 @@ def _image_struct(im: Image, dev: int, need_depth: bool) -> ec_image:
     return ec_image(_rect(pvp), _rect(roi), pitch, fmt, im.color.data_ptr(), dptr)
 
 
+_NO_DEPTH, _DEPTH, _ANY_DEPTH = 0, 1, 2          # what _images asks of the depth buffers
+
+
+def _images(images: Sequence[Image], dev: int, need: int):
+    """The ec_image array of a list of images.  Plain ones are read by the native
+    marshalling; where one is not, each is checked here, which accepts the rarer
+    forms and reports what is wrong."""
+    arr = (ec_image * max(1, len(images)))()
+    if not A.marshal().images(images, dev, need, C.addressof(arr)):
+        for i, im in enumerate(images):
+            arr[i] = _image_struct(im, dev, need == _DEPTH or (need == _ANY_DEPTH and im.depth is not None))
+    return arr
+
+
 def _target(color: torch.Tensor, depth: Optional[torch.Tensor], pvp, dev: int) -> ec_target:
+    tgt = ec_target()
+    if A.marshal().target(color, depth, pvp, dev, C.addressof(tgt)):
+        return tgt
     fmt, pitch, w, h = pixel_layout(color)
     _on_device(color, dev, "output colour")
     pvp = tuple(pvp) if pvp is not None else (0, 0, w, h)
@@ -150,7 +168,7 @@ def _dense(t: Optional[torch.Tensor], shape, dtype, dev: int, what: str) -> Opti
     if t is None:
         return None
     _on_device(t, dev, what)
-    if t.dtype != dtype or not t.is_contiguous() or t.numel() < int(torch.tensor(shape).prod()):
+    if t.dtype != dtype or not t.is_contiguous() or t.numel() < math.prod(shape):
         raise ValueError(f"{what} must be a contiguous {dtype} tensor of shape {shape}")
     return t.data_ptr()
 
@@ -162,7 +180,7 @@ def composite_depth(images: Sequence[Image], out_color: torch.Tensor,
     """ec_composite_depth: per-pixel depth-test merge.  Returns the merged ROI."""
     ctx = ctx or default_context(out_color.device.index)
     dev = ctx.device
-    arr = (ec_image * max(1, len(images)))(*[_image_struct(im, dev, True) for im in images])
+    arr = _images(images, dev, _DEPTH)
     tgt = _target(out_color, out_depth, out_pvp, dev)
     wp = _dense(winner, (tgt.pvp.h, tgt.pvp.w), torch.int16, dev, "winner")
     roi = ec_rect()
@@ -174,7 +192,9 @@ def composite_depth(images: Sequence[Image], out_color: torch.Tensor,
 def _order(order, n):
     if order is None:
         return None
-    o = (C.c_int32 * max(1, n))(*[int(v) for v in order])
+    o = (C.c_int32 * max(1, n))()
+    if not A.marshal().order(order, n, C.addressof(o)):
+        o = (C.c_int32 * max(1, n))(*[int(v) for v in order])
     if len(order) != n:
         raise ValueError("order needs one entry per layer")
     return o
@@ -186,7 +206,7 @@ def composite_alpha(layers: Sequence[Image], out: torch.Tensor, order=None,
     """ec_composite_alpha: front-to-back premultiplied 'over'.  Returns the merged ROI."""
     ctx = ctx or default_context(out.device.index)
     dev = ctx.device
-    arr = (ec_image * max(1, len(layers)))(*[_image_struct(im, dev, False) for im in layers])
+    arr = _images(layers, dev, _NO_DEPTH)
     tgt = _target(out, None, out_pvp, dev)
     tp = _dense(t_final, (tgt.pvp.h, tgt.pvp.w), torch.float32, dev, "t_final")
     roi = ec_rect()
@@ -203,13 +223,22 @@ def composite_alpha_backward(layers: Sequence[Image], out_pvp: Rect, grad_out: t
     ctx = ctx or default_context(grad_out.device.index)
     dev = ctx.device
     n = len(layers)
-    arr = (ec_image * max(1, n))(*[_image_struct(im, dev, False) for im in layers])
+    arr = _images(layers, dev, _NO_DEPTH)
     gp = _dense(grad_out, (out_pvp[3], out_pvp[2], 4), torch.float32, dev, "grad_out")
-    gfmt = _grad_format(grads, layers, dev)
-    ptrs = (C.c_void_p * max(1, n))(*[g.data_ptr() for g in grads])
+    gfmt, ptrs = _gradients(grads, layers, dev)
     check(_lib().ec_composite_alpha_backward(ctx.h, arr, _order(order, n), n, _rect(out_pvp), gp,
                                              ptrs, gfmt, _stream_handle(stream)),
           "ec_composite_alpha_backward")
+
+
+def _gradients(grads, layers, dev):
+    """(format, pointer array) of one gradient buffer per layer."""
+    ptrs = (C.c_void_p * max(1, len(layers)))()
+    fmt = A.marshal().gradients(grads, layers, dev, C.addressof(ptrs))
+    if fmt is False:
+        fmt = _grad_format(grads, layers, dev)
+        ptrs = (C.c_void_p * max(1, len(layers)))(*[g.data_ptr() for g in grads])
+    return fmt, ptrs
 
 
 def _grad_format(grads, layers, dev) -> int:
@@ -235,12 +264,11 @@ def composite_alpha_fwd_bwd(layers: Sequence[Image], out: torch.Tensor, w: torch
     ctx = ctx or default_context(out.device.index)
     dev = ctx.device
     n = len(layers)
-    arr = (ec_image * max(1, n))(*[_image_struct(im, dev, False) for im in layers])
+    arr = _images(layers, dev, _NO_DEPTH)
     tgt = _target(out, None, out_pvp, dev)
     tp = _dense(t_final, (tgt.pvp.h, tgt.pvp.w), torch.float32, dev, "t_final")
     wp = _dense(w, (tgt.pvp.h, tgt.pvp.w, 4), torch.float32, dev, "w")
-    gfmt = _grad_format(grads, layers, dev)
-    ptrs = (C.c_void_p * max(1, n))(*[g.data_ptr() for g in grads])
+    gfmt, ptrs = _gradients(grads, layers, dev)
     roi = ec_rect()
     check(_lib().ec_composite_alpha_fwd_bwd(ctx.h, arr, _order(order, n), n, C.byref(tgt), tp, wp,
                                             ptrs, gfmt, C.byref(roi), _stream_handle(stream)),
@@ -254,7 +282,7 @@ def assemble_tiles(images: Sequence[Image], out: torch.Tensor, out_pvp: Optional
     ctx = ctx or default_context(out.device.index)
     dev = ctx.device
     n = len(images)
-    arr = (ec_image * max(1, n))(*[_image_struct(im, dev, False) for im in images])
+    arr = _images(images, dev, _NO_DEPTH)
     tgt = _target(out, None, out_pvp, dev)
     check(_lib().ec_assemble_tiles(ctx.h, arr, n, C.byref(tgt), _stream_handle(stream)), "ec_assemble_tiles")
 
@@ -265,7 +293,7 @@ def average(images: Sequence[Image], out: torch.Tensor, out_pvp: Optional[Rect] 
     ctx = ctx or default_context(out.device.index)
     dev = ctx.device
     n = len(images)
-    arr = (ec_image * max(1, n))(*[_image_struct(im, dev, False) for im in images])
+    arr = _images(images, dev, _NO_DEPTH)
     tgt = _target(out, None, out_pvp, dev)
     check(_lib().ec_average(ctx.h, arr, n, C.byref(tgt), _stream_handle(stream)), "ec_average")
 
@@ -302,29 +330,14 @@ def detect_roi(images: Sequence[Image], tile: int = 64, occupancy: bool = True,
     dev = (ctx.device if ctx else (images[0].color.device.index if n else torch.cuda.current_device()))
     ctx = ctx or default_context(dev)
     dev = ctx.device
-    structs = []
-    for im in images:
-        fmt, pitch, w, h = pixel_layout(im.color)
-        _on_device(im.color, dev, "colour")
-        pvp = tuple(im.pvp) if im.pvp is not None else (0, 0, w, h)
-        roi = tuple(im.roi) if im.roi is not None else pvp
-        if pvp[2] > w or pvp[3] > h:
-            raise ValueError("pvp larger than the colour tensor")
-        dptr = None
-        if im.depth is not None:
-            _on_device(im.depth, dev, "depth")
-            dd = im.depth
-            if dd.dtype != torch.float32 or dd.dim() != 2 or dd.stride(1) != 1 or dd.stride(0) != pitch \
-                    or dd.shape[0] < pvp[3] or dd.shape[1] < pvp[2]:
-                raise ValueError("depth must be float32 [h][pitch] with the colour's pitch")
-            dptr = dd.data_ptr()
-        structs.append(ec_image(_rect(pvp), _rect(roi), pitch, fmt, im.color.data_ptr(), dptr))
-    arr = (ec_image * max(1, n))(*structs)
-    rois = torch.zeros((max(n, 1), 4), dtype=torch.int32, device=f"cuda:{dev}")[:n]
+    arr = _images(images, dev, _ANY_DEPTH)
+    # every image's rectangle is written by the call
+    device = torch.device("cuda", dev)
+    rois = torch.empty((n, 4), dtype=torch.int32, device=device)
     grids, occ = None, None
     if occupancy:
-        grids = [torch.empty((-(-s.pvp.h // tile), -(-s.pvp.w // tile)), dtype=torch.uint8, device=f"cuda:{dev}")
-                 for s in structs]
+        grids = [torch.empty((-(-arr[i].pvp.h // tile), -(-arr[i].pvp.w // tile)), dtype=torch.uint8, device=device)
+                 for i in range(n)]
         occ = (C.c_void_p * max(1, n))(*[g.data_ptr() if g.numel() else None for g in grids])
     check(_lib().ec_detect_roi(ctx.h, arr, n, int(tile), occ, rois.data_ptr() if n else None,
                                _stream_handle(stream)), "ec_detect_roi")
@@ -568,7 +581,7 @@ class Batch:
         arr = (A.ec_job * max(1, len(jobs)))()
         for k, jb in enumerate(jobs):
             depth = jb.mode == "depth"
-            imgs = (ec_image * max(1, len(jb.images)))(*[_image_struct(im, dev, depth) for im in jb.images])
+            imgs = _images(jb.images, dev, _DEPTH if depth else _NO_DEPTH)
             order = None if depth else _order(jb.order, len(jb.images))
             tgt = _target(jb.out_color, jb.out_depth if depth else None, jb.out_pvp, dev)
             wp = _dense(jb.winner, (tgt.pvp.h, tgt.pvp.w), torch.int16, dev, "winner") if depth else None
@@ -654,7 +667,7 @@ class Schedule:
         depth = mode == "depth"
         if not depth and mode != "alpha":
             raise ValueError("mode must be 'depth' or 'alpha'")
-        imgs = (ec_image * max(1, len(images)))(*[_image_struct(im, dev, depth) for im in images])
+        imgs = _images(images, dev, _DEPTH if depth else _NO_DEPTH)
         o = None if depth else _order(order, len(images))
         tgt = _target(out_color, out_depth if depth else None, out_pvp, dev)
         self._keep = [imgs, o, list(images), out_color, out_depth]

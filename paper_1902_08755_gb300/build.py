@@ -1,14 +1,16 @@
-"""Build libec.so (the CUDA library behind include/ec.h) in-tree with nvcc.
+"""Build libec.so (the CUDA library behind include/ec.h) in-tree with nvcc, and
+the binding's argument marshalling (_marshal.so) with the host compiler.
 
 Every translation unit is compiled for sm_103a only, in parallel, then linked
 into paper_1902_08755_gb300/libec.so.  No cmake; a rebuild happens when a
-source or header is newer than the library.
+source or header is newer than the libraries.
 """
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -16,6 +18,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libec.so")
+MARSHAL = os.path.join(HERE, "_marshal.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2", "--expt-relaxed-constexpr",
          "-I", os.path.join(ROOT, "include")]
@@ -32,10 +35,26 @@ def sources():
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(MARSHAL):
         return True
     deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
-    return os.path.getmtime(LIB) < max(os.path.getmtime(p) for p in deps)
+    deps.append(os.path.join(CSRC, "marshal.cpp"))
+    return min(os.path.getmtime(LIB), os.path.getmtime(MARSHAL)) < max(os.path.getmtime(p) for p in deps)
+
+
+def _build_marshal() -> None:
+    import torch
+    troot = os.path.dirname(torch.__file__)
+    tmp = MARSHAL + f".tmp{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", sysconfig.get_paths()["include"], "-I", os.path.join(troot, "include"),
+           os.path.join(CSRC, "marshal.cpp"), "-o", tmp,
+           "-L", os.path.join(troot, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed for marshal.cpp:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, MARSHAL)
 
 
 def build(force: bool = False, verbose: bool = False, extra=()) -> str:
@@ -54,8 +73,10 @@ def build(force: bool = False, verbose: bool = False, extra=()) -> str:
             print(r.stdout, r.stderr)
         return obj
 
-    with ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 1)) as ex:
+    with ThreadPoolExecutor(max_workers=min(12, os.cpu_count() or 1)) as ex:
+        marshal = ex.submit(_build_marshal)
         objs = list(ex.map(compile_one, sources()))
+        marshal.result()
     tmp = LIB + f".tmp{os.getpid()}"
     cmd = [nvcc, *ARCH, "-shared", "-o", tmp, *objs, "-lcudart"]
     r = subprocess.run(cmd, capture_output=True, text=True)
