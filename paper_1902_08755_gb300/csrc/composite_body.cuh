@@ -47,8 +47,9 @@ template <> struct ColorT<16> { using T = float4; };
 __device__ __forceinline__ void zero(uint32_t& c) { c = 0u; }
 __device__ __forceinline__ void zero(float4& c) { c = make_float4(0.f, 0.f, 0.f, 0.f); }
 
-// 4 consecutive pixels of one source: 16-byte loads (vec) or per-pixel loads.
-template <int CB>
+// The pixels x + j STEP, j = 0..3, of one source: 16-byte loads (vec, STEP 1) or
+// per-pixel loads.
+template <int CB, int STEP>
 __device__ __forceinline__ void load4(const SrcDesc& s, int x, int y, float (&d)[4],
                                       typename ColorT<CB>::T (&c)[4])
 {
@@ -56,7 +57,7 @@ __device__ __forceinline__ void load4(const SrcDesc& s, int x, int y, float (&d)
     const size_t e = (size_t)(y - s.oy) * (size_t)s.pitch + (size_t)(x - s.ox);
     const float* dp = s.depth + e;
     const C* cp = reinterpret_cast<const C*>(s.color) + e;
-    if (s.vec) {
+    if (STEP == 1 && s.vec) {
         const float4 d4 = ld_stream(reinterpret_cast<const float4*>(dp));
         d[0] = d4.x; d[1] = d4.y; d[2] = d4.z; d[3] = d4.w;
         if constexpr (CB == 4) {
@@ -69,11 +70,11 @@ __device__ __forceinline__ void load4(const SrcDesc& s, int x, int y, float (&d)
     } else {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int xj = x + j;
+            const int xj = x + j * STEP;
             if (xj >= s.x0 && xj < s.x1) {
-                d[j] = __ldcs(dp + j);
-                if constexpr (CB == 4) c[j] = __ldcs(reinterpret_cast<const unsigned int*>(cp + j));
-                else c[j] = __ldcs(cp + j);
+                d[j] = __ldcs(dp + j * STEP);
+                if constexpr (CB == 4) c[j] = __ldcs(reinterpret_cast<const unsigned int*>(cp + j * STEP));
+                else c[j] = __ldcs(cp + j * STEP);
             } else {
                 d[j] = 1.0f;
                 zero(c[j]);
@@ -82,9 +83,13 @@ __device__ __forceinline__ void load4(const SrcDesc& s, int x, int y, float (&d)
     }
 }
 
-// Depth merge of the 4 pixels x..x+3 of row y (output-relative coordinates),
-// U inputs' loads in flight per thread.
-template <int CB, class At, int U = 4>
+// Depth merge of the 4 pixels x + j STEP of row y (output-relative coordinates),
+// U inputs' loads in flight per thread.  STEP 1: a lane's pixels are adjacent
+// and inputs whose rows allow it are read 16 bytes at a time.  STEP 32: a
+// warp's lanes own adjacent pixels, for calls with inputs that must be read
+// pixel by pixel: every load of the warp then covers 128 contiguous bytes, where
+// adjacent pixels per lane would spread it over 512 (four times the sectors).
+template <int CB, int STEP, class At, int U = 4>
 __device__ __forceinline__ void depth_px4(At at, const int16_t* act, int nact, int x, int y,
                                           const DstDesc& D)
 {
@@ -106,8 +111,8 @@ __device__ __forceinline__ void depth_px4(At at, const int16_t* act, int nact, i
             live[u] = false;
             if (idx[u] >= 0) {
                 const SrcDesc& s = at(a + u, idx[u]);
-                live[u] = y >= s.y0 && y < s.y1 && x + 4 > s.x0 && x < s.x1;
-                if (live[u]) load4<CB>(s, x, y, d[u], c[u]);
+                live[u] = y >= s.y0 && y < s.y1 && x + 3 * STEP >= s.x0 && x < s.x1;
+                if (live[u]) load4<CB, STEP>(s, x, y, d[u], c[u]);
             }
         }
 #pragma unroll
@@ -116,7 +121,7 @@ __device__ __forceinline__ void depth_px4(At at, const int16_t* act, int nact, i
             const SrcDesc& s = at(a + u, idx[u]);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const int xj = x + j;
+                const int xj = x + j * STEP;
                 // strict '<': ties keep the earlier (lower-index) winner or the
                 // background; NaN never compares less
                 if (xj >= s.x0 && xj < s.x1 && d[u][j] < bd[j]) {
@@ -130,7 +135,7 @@ __device__ __forceinline__ void depth_px4(At at, const int16_t* act, int nact, i
 
     const size_t o = (size_t)y * (size_t)D.pitch + (size_t)x;
     C* oc = reinterpret_cast<C*>(D.color) + o;
-    if (D.vec && x + 4 <= D.W) {
+    if (STEP == 1 && D.vec && x + 4 <= D.W) {
         if constexpr (CB == 4) st_stream(reinterpret_cast<uint4*>(oc), make_uint4(bc[0], bc[1], bc[2], bc[3]));
         else {
 #pragma unroll
@@ -140,9 +145,9 @@ __device__ __forceinline__ void depth_px4(At at, const int16_t* act, int nact, i
     } else {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            if (x + j < D.W) {
-                oc[j] = bc[j];
-                if (D.depth) D.depth[o + j] = bd[j];
+            if (x + j * STEP < D.W) {
+                oc[j * STEP] = bc[j];
+                if (D.depth) D.depth[o + j * STEP] = bd[j];
             }
         }
     }
@@ -150,7 +155,7 @@ __device__ __forceinline__ void depth_px4(At at, const int16_t* act, int nact, i
         int16_t* w = D.winner + (size_t)y * D.W + x;
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-            if (x + j < D.W) w[j] = (int16_t)bi[j];
+            if (x + j * STEP < D.W) w[j * STEP] = (int16_t)bi[j];
     }
 }
 
@@ -194,6 +199,12 @@ __device__ __forceinline__ uint4 load_raw(const SrcDesc& s, int x, int y)
             const int xj = x + j;
             if (xj >= s.x0 && xj < s.x1) {
                 const unsigned short* h = reinterpret_cast<const unsigned short*>(p + j);
+                if ((reinterpret_cast<uintptr_t>(p) & 7u) == 0) {      // whole pixels
+                    const uint2 v = __ldcs(p + j);
+                    w[2 * j] = v.x;
+                    w[2 * j + 1] = v.y;
+                    continue;
+                }
                 w[2 * j] = (uint32_t)__ldcs(h) | ((uint32_t)__ldcs(h + 1) << 16);
                 w[2 * j + 1] = (uint32_t)__ldcs(h + 2) | ((uint32_t)__ldcs(h + 3) << 16);
             }
@@ -272,6 +283,9 @@ __device__ __forceinline__ void alpha_px(At at, const int16_t* act, int nact, in
         const uint2 h0 = float4_to_half4(acc[0]), h1 = float4_to_half4(acc[1]);
         if (D.vec && x + 2 <= D.W) {
             st_stream(reinterpret_cast<uint4*>(op), make_uint4(h0.x, h0.y, h1.x, h1.y));
+        } else if ((reinterpret_cast<uintptr_t>(op) & 7u) == 0) {      // whole pixels
+            op[0] = h0;
+            if (x + 1 < D.W) op[1] = h1;
         } else {
             unsigned short* hp = reinterpret_cast<unsigned short*>(op);
             hp[0] = (unsigned short)h0.x; hp[1] = (unsigned short)(h0.x >> 16);

@@ -97,8 +97,10 @@ k_assemble_tiles(const __grid_constant__ SrcList<N> L, const __grid_constant__ D
     uint32_t fast = 0;                                   // passes already written
     if (MASK && PX * BPP == 16 && D.vec && full == (1u << PX) - 1u) {
         // groups that one source covers whole (the usual case): every such
-        // pass's 16-byte load is issued before any store
-        const uint4* fp[kTPasses];
+        // pass's loads (one of 16 bytes, or the group's pixels where a source's
+        // rows start at another alignment) are issued before any store
+        const uint8_t* fp[kTPasses];
+        uint32_t wide = 0;                               // passes read with one load
 #pragma unroll
         for (int pass = 0; pass < kTPasses; ++pass) {
             fp[pass] = nullptr;
@@ -110,18 +112,28 @@ k_assemble_tiles(const __grid_constant__ SrcList<N> L, const __grid_constant__ D
                 const SrcDesc& s = L.s[i];
                 const uint32_t m = covered<PX>(s, x, y, D.W);
                 if (!m) continue;
-                if (m == full && s.vec) {
+                if (m == full) {
                     const size_t e = (size_t)(y - s.oy) * (size_t)s.pitch + (size_t)(x - s.ox);
-                    fp[pass] = reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(s.color) + e * BPP);
+                    fp[pass] = reinterpret_cast<const uint8_t*>(s.color) + e * BPP;
                     fast |= 1u << pass;
+                    if (s.vec) wide |= 1u << pass;
                 }
                 break;
             }
         }
         uint4 v[kTPasses];
 #pragma unroll
-        for (int pass = 0; pass < kTPasses; ++pass)
-            if ((fast >> pass) & 1u) v[pass] = __ldcs(fp[pass]);
+        for (int pass = 0; pass < kTPasses; ++pass) {
+            if ((wide >> pass) & 1u) {
+                v[pass] = __ldcs(reinterpret_cast<const uint4*>(fp[pass]));
+            } else if ((fast >> pass) & 1u) {
+                uint32_t w[PX][WPP];
+#pragma unroll
+                for (int j = 0; j < PX; ++j) load_px<BPP>(fp[pass] + j * BPP, w[j]);
+                const uint32_t* f = &w[0][0];
+                v[pass] = make_uint4(f[0], f[1], f[2], f[3]);
+            }
+        }
 #pragma unroll
         for (int pass = 0; pass < kTPasses; ++pass) {
             if (!((fast >> pass) & 1u)) continue;

@@ -26,7 +26,8 @@ constexpr int kRows = kThreads / 32;   // one warp per tile row
 constexpr int kDThreads = 128;
 constexpr int kDRows = kDThreads / 32;
 
-template <int N, int CB>
+// STEP 32: a lane's pixels lie 32 apart (see depth_px4).
+template <int N, int CB, int STEP>
 __global__ void __launch_bounds__(kDThreads)
 k_depth(const __grid_constant__ SrcList<N> L, const __grid_constant__ DstDesc D)
 {
@@ -39,9 +40,9 @@ k_depth(const __grid_constant__ SrcList<N> L, const __grid_constant__ DstDesc D)
     const int tx0 = blockIdx.x * kTW, ty0 = blockIdx.y * kDRows;
     build_active(at, L.n, tx0, ty0, min(tx0 + kTW, D.W), min(ty0 + kDRows, D.H), act, &nact_s);
     __syncthreads();
-    const int x = tx0 + lane * 4, y = ty0 + row;
+    const int x = tx0 + lane * (STEP == 1 ? 4 : 1), y = ty0 + row;
     if (x >= D.W || y >= D.H) return;
-    depth_px4<CB>(at, act, nact_s, x, y, D);
+    depth_px4<CB, STEP>(at, act, nact_s, x, y, D);
 }
 
 template <int N, bool F16>
@@ -91,8 +92,11 @@ cudaError_t depth_n(const SrcDesc* src, int n, int cb, const DstDesc& D, cudaStr
 {
     const dim3 grid(ceil_div(D.W, 128), ceil_div(D.H, kDRows));
     const SrcList<N> L = make_list<N>(src, n);
-    if (cb == 4) k_depth<N, 4><<<grid, kDThreads, 0, s>>>(L, D);
-    else k_depth<N, 16><<<grid, kDThreads, 0, s>>>(L, D);
+    bool vec = true;
+    for (int i = 0; i < n; ++i) vec = vec && (src[i].vec || src[i].x0 >= src[i].x1);
+    if (cb != 4) k_depth<N, 16, 1><<<grid, kDThreads, 0, s>>>(L, D);
+    else if (vec) k_depth<N, 4, 1><<<grid, kDThreads, 0, s>>>(L, D);
+    else k_depth<N, 4, 32><<<grid, kDThreads, 0, s>>>(L, D);
     return cudaGetLastError();
 }
 
