@@ -89,6 +89,42 @@ __device__ __forceinline__ float4 ld_stream(const float4* p) { return __ldcs(p);
 __device__ __forceinline__ void st_stream(uint4* p, uint4 v) { __stcs(p, v); }
 __device__ __forceinline__ void st_stream(float4* p, float4 v) { __stcs(p, v); }
 
+// Chained launches (programmatic dependent launch).  A kernel launched with
+// launch_chained is put on the SMs as soon as the last CTAs of the kernel before
+// it on the stream end, without waiting for that kernel's memory flush and the
+// launch's own latency: about 1.7 us less per launch (4 x 640x480 merges back
+// to back 6.2 -> 3.0 us, a compress, decompress and merge of 16 1920x1080
+// sources, nine launches, 117 -> 105 us).  Every thread calls chain_wait before
+// it touches memory that other kernels write: it returns once all earlier
+// kernels of the stream are complete and their writes visible.  Every CTA of a
+// chained kernel calls it, so that its completion implies its predecessors'.
+// chain_next lets the next chained kernel be put on the SMs once all of this
+// kernel's CTAs have started.  Only the kernels of a batch call it, which share
+// the device by intent: elsewhere the CTAs put there early took the room of
+// the running kernel's (16 7680x4320 sources 993 -> 1105 us).
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class T> struct SameType { using type = T; };
+
+template <class... P>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                           const typename SameType<P>::type&... args)
+{
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = at;
+    c.numAttrs = 1;
+    void* pargs[] = {const_cast<void*>(static_cast<const void*>(&args))...};
+    return cudaLaunchKernelExC(&c, reinterpret_cast<const void*>(kernel), pargs);
+}
+
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
 // Per-layer descriptor of the backward passes (64 bytes), in compositing

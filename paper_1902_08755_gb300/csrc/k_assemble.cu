@@ -83,6 +83,7 @@ k_assemble_tiles(const __grid_constant__ SrcList<N> L, const __grid_constant__ D
     __shared__ int nact_s;
     const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
     const int tx0 = blockIdx.x * TW, ty0 = blockIdx.y * (kARows * kTPasses);
+    chain_wait();
     uint64_t amask = 0;
     if (MASK) {
         amask = M.col[blockIdx.x] & M.row[blockIdx.y];
@@ -214,6 +215,7 @@ k_average(const __grid_constant__ SrcList<N> L, const __grid_constant__ DstDesc 
     const int tx1 = min(tx0 + 32 * PX, D.W), ty1 = min(ty0 + kARows * kAPasses, D.H);
     build_active(at, L.n, tx0, ty0, tx1, ty1, act, &nact_s);
     __syncthreads();
+    chain_wait();
     const int nact = nact_s;
     // every active source covers the whole tile with 16-byte rows: no per-pixel masks
     bool cov = true;
@@ -353,6 +355,7 @@ k_assemble_pixels(const __grid_constant__ PixList<N> P, const __grid_constant__ 
     constexpr int PX = Grp<BPP>::PX, WPP = BPP / 4;
     const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
     const int x = blockIdx.x * (32 * PX) + lane * PX;
+    chain_wait();
     if (x >= D.W) return;
     const int i00 = x / P.nx, rx00 = x - i00 * P.nx;    // one division; then step the residue
     // kAPasses rows per thread, every load issued before any store
@@ -408,18 +411,12 @@ SrcList<N> make_src_list(const SrcDesc* src, int n)
     return L;
 }
 
-template <int N, int BPP, bool MASK>
-void tiles_launch(const SrcList<N>& L, const DstDesc& D, const TileMasks& M, dim3 grid, cudaStream_t s)
-{
-    k_assemble_tiles<N, BPP, MASK><<<grid, kAT, 0, s>>>(L, D, M);
-}
-
 template <int N, bool MASK>
-void tiles_bpp(const SrcList<N>& L, int bpp, const DstDesc& D, const TileMasks& M, dim3 grid, cudaStream_t s)
+cudaError_t tiles_bpp(const SrcList<N>& L, int bpp, const DstDesc& D, const TileMasks& M, dim3 grid, cudaStream_t s)
 {
-    if (bpp == 4) tiles_launch<N, 4, MASK>(L, D, M, grid, s);
-    else if (bpp == 8) tiles_launch<N, 8, MASK>(L, D, M, grid, s);
-    else tiles_launch<N, 16, MASK>(L, D, M, grid, s);
+    if (bpp == 4) return launch_chained(k_assemble_tiles<N, 4, MASK>, grid, kAT, 0, s, L, D, M);
+    if (bpp == 8) return launch_chained(k_assemble_tiles<N, 8, MASK>, grid, kAT, 0, s, L, D, M);
+    return launch_chained(k_assemble_tiles<N, 16, MASK>, grid, kAT, 0, s, L, D, M);
 }
 
 template <int N>
@@ -440,11 +437,9 @@ cudaError_t tiles_n(const SrcDesc* src, int n, int bpp, const DstDesc& D, cudaSt
             for (int c = x0 / tw; c < ceil_div(x1, tw); ++c) M.col[c] |= 1ull << i;
             for (int r = y0 / th; r < ceil_div(y1, th); ++r) M.row[r] |= 1ull << i;
         }
-        tiles_bpp<N, true>(L, bpp, D, M, grid, s);
-    } else {
-        tiles_bpp<N, false>(L, bpp, D, M, grid, s);
+        return tiles_bpp<N, true>(L, bpp, D, M, grid, s);
     }
-    return cudaGetLastError();
+    return tiles_bpp<N, false>(L, bpp, D, M, grid, s);
 }
 
 template <int N>
@@ -453,10 +448,9 @@ cudaError_t average_n(const SrcDesc* src, int n, int fmt, const DstDesc& D, cuda
     const SrcList<N> L = make_src_list<N>(src, n);
     const int px = fmt == 0 ? 4 : fmt == 1 ? 1 : 2;
     const dim3 grid(ceil_div(D.W, 32 * px), ceil_div(D.H, kARows * kAPasses));
-    if (fmt == 0) k_average<N, 0><<<grid, kAT, 0, s>>>(L, D);
-    else if (fmt == 1) k_average<N, 1><<<grid, kAT, 0, s>>>(L, D);
-    else k_average<N, 2><<<grid, kAT, 0, s>>>(L, D);
-    return cudaGetLastError();
+    if (fmt == 0) return launch_chained(k_average<N, 0>, grid, kAT, 0, s, L, D);
+    if (fmt == 1) return launch_chained(k_average<N, 1>, grid, kAT, 0, s, L, D);
+    return launch_chained(k_average<N, 2>, grid, kAT, 0, s, L, D);
 }
 
 template <int N>
@@ -472,10 +466,9 @@ cudaError_t pixels_n(const PixSrc* src, const int16_t* owner, int n, int nx, int
     for (int i = 0; i < nx * ny; ++i) P.owner[i] = owner[i];
     const int px = 16 / bpp;
     const dim3 grid(ceil_div(D.W, 32 * px), ceil_div(D.H, kARows * kAPasses));
-    if (bpp == 4) k_assemble_pixels<N, 4><<<grid, kAT, 0, s>>>(P, D);
-    else if (bpp == 8) k_assemble_pixels<N, 8><<<grid, kAT, 0, s>>>(P, D);
-    else k_assemble_pixels<N, 16><<<grid, kAT, 0, s>>>(P, D);
-    return cudaGetLastError();
+    if (bpp == 4) return launch_chained(k_assemble_pixels<N, 4>, grid, kAT, 0, s, P, D);
+    if (bpp == 8) return launch_chained(k_assemble_pixels<N, 8>, grid, kAT, 0, s, P, D);
+    return launch_chained(k_assemble_pixels<N, 16>, grid, kAT, 0, s, P, D);
 }
 
 }  // namespace

@@ -520,6 +520,7 @@ k_alpha_bwd(const __grid_constant__ BwdList<N> L, const __grid_constant__ DstDes
             }
         }
     };
+    chain_wait();
     if (fast) {
         if constexpr (F16) rows_fast16();
         else for (int y = ty0; y < ty1; ++y) row_fast(y);
@@ -560,6 +561,7 @@ k_depth_bwd(const __grid_constant__ BwdList<N> L, int W, int H, const int16_t* _
     __syncthreads();
     const int nact = nact_s;
     const int x = tx0 + lane * 4, y = ty0 + row;
+    chain_wait();
     if (x >= W || y >= H) return;
     int win[4];
     float4 gv[4];
@@ -642,8 +644,7 @@ cudaError_t alpha_bwd_n(const BwdDesc* d, int n, const DstDesc& D, const float4*
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     const int rows = alpha_bwd_rows(n, D.W, D.H, tw, ns, smem, sms);
     const dim3 grid(ceil_div(D.W, tw), ceil_div(D.H, rows));
-    kern<<<grid, 32 * ns, smem, s>>>(make_bwd<N>(d, n), D, g, cap, rows);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, 32 * ns, smem, s, make_bwd<N>(d, n), D, g, cap, rows);
 }
 
 // One pixel per lane and eight layers per warp, FP32 and FP16 alike (two FP16
@@ -690,10 +691,9 @@ cudaError_t launch_depth_bwd(const BwdDesc* d, int n, int W, int H, const int16_
     if (W <= 0 || H <= 0 || n <= 0) return cudaSuccess;
     const dim3 grid(ceil_div(W, 128), ceil_div(H, 8));
     const float4* g4 = reinterpret_cast<const float4*>(g);
-    if (n <= 16) k_depth_bwd<16><<<grid, 256, 0, s>>>(make_bwd<16>(d, n), W, H, winner, g4);
-    else if (n <= 64) k_depth_bwd<64><<<grid, 256, 0, s>>>(make_bwd<64>(d, n), W, H, winner, g4);
-    else k_depth_bwd<kMaxBwdLayers><<<grid, 256, 0, s>>>(make_bwd<kMaxBwdLayers>(d, n), W, H, winner, g4);
-    return cudaGetLastError();
+    if (n <= 16) return launch_chained(k_depth_bwd<16>, grid, 256, 0, s, make_bwd<16>(d, n), W, H, winner, g4);
+    if (n <= 64) return launch_chained(k_depth_bwd<64>, grid, 256, 0, s, make_bwd<64>(d, n), W, H, winner, g4);
+    return launch_chained(k_depth_bwd<kMaxBwdLayers>, grid, 256, 0, s, make_bwd<kMaxBwdLayers>(d, n), W, H, winner, g4);
 }
 
 }  // namespace ec

@@ -40,6 +40,7 @@ k_depth(const __grid_constant__ SrcList<N> L, const __grid_constant__ DstDesc D)
     const int tx0 = blockIdx.x * kTW, ty0 = blockIdx.y * kDRows;
     build_active(at, L.n, tx0, ty0, min(tx0 + kTW, D.W), min(ty0 + kDRows, D.H), act, &nact_s);
     __syncthreads();
+    chain_wait();
     const int x = tx0 + lane * (STEP == 1 ? 4 : 1), y = ty0 + row;
     if (x >= D.W || y >= D.H) return;
     depth_px4<CB, STEP>(at, act, nact_s, x, y, D);
@@ -60,6 +61,7 @@ k_alpha_fwd(const __grid_constant__ SrcList<N> L, const __grid_constant__ DstDes
     const int tx1 = min(tx0 + kTW, D.W), ty1 = min(ty0 + kRows, D.H);
     build_active(at, L.n, tx0, ty0, tx1, ty1, act, &nact_s);
     __syncthreads();
+    chain_wait();
     const int nact = nact_s;
     // FP16 tiles that every active layer covers skip the range tests (FP32
     // keeps one path: its second path would cost more registers than it saves)
@@ -94,10 +96,9 @@ cudaError_t depth_n(const SrcDesc* src, int n, int cb, const DstDesc& D, cudaStr
     const SrcList<N> L = make_list<N>(src, n);
     bool vec = true;
     for (int i = 0; i < n; ++i) vec = vec && (src[i].vec || src[i].x0 >= src[i].x1);
-    if (cb != 4) k_depth<N, 16, 1><<<grid, kDThreads, 0, s>>>(L, D);
-    else if (vec) k_depth<N, 4, 1><<<grid, kDThreads, 0, s>>>(L, D);
-    else k_depth<N, 4, 32><<<grid, kDThreads, 0, s>>>(L, D);
-    return cudaGetLastError();
+    if (cb != 4) return launch_chained(k_depth<N, 16, 1>, grid, kDThreads, 0, s, L, D);
+    if (vec) return launch_chained(k_depth<N, 4, 1>, grid, kDThreads, 0, s, L, D);
+    return launch_chained(k_depth<N, 4, 32>, grid, kDThreads, 0, s, L, D);
 }
 
 template <int N>
@@ -106,12 +107,11 @@ cudaError_t alpha_n(const SrcDesc* src, int n, bool f16, const DstDesc& D, cudaS
     const SrcList<N> L = make_list<N>(src, n);
     if (f16) {
         const dim3 grid(ceil_div(D.W, 64), ceil_div(D.H, kRows));
-        k_alpha_fwd<N, true><<<grid, kThreads, 0, s>>>(L, D);
+        return launch_chained(k_alpha_fwd<N, true>, grid, kThreads, 0, s, L, D);
     } else {
         const dim3 grid(ceil_div(D.W, 32), ceil_div(D.H, kRows));
-        k_alpha_fwd<N, false><<<grid, kThreads, 0, s>>>(L, D);
+        return launch_chained(k_alpha_fwd<N, false>, grid, kThreads, 0, s, L, D);
     }
-    return cudaGetLastError();
 }
 
 }  // namespace

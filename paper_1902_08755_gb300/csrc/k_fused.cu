@@ -215,8 +215,10 @@ k_fused_depth(const FusedStage* __restrict__ stages, const FusedUnit* __restrict
     __shared__ int s_fail, s_over;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // (the plan's own arrays: written when it was made)
     const FusedUnit u = units[blockIdx.x];
     const FusedStage S = stages[u.stage];
+    chain_wait();
 
     if (u.cs == nullptr) {                    // fill: rows [chunk, chunk + nrows) of the rectangle
         compose<false>(S, u, (int)u.chunk, u.nrows, 0, 0, planes, false, false);
@@ -351,8 +353,7 @@ cudaError_t launch_fused_depth(const FusedStage* stages, const FusedUnit* units,
                                uint32_t* status, cudaStream_t s)
 {
     if (n_units <= 0) return cudaSuccess;
-    k_fused_depth<<<n_units, kFT, 0, s>>>(stages, units, status);
-    return cudaGetLastError();
+    return launch_chained(k_fused_depth, n_units, kFT, 0, s, stages, units, status);
 }
 
 }  // namespace ec

@@ -509,6 +509,7 @@ k_rle_code(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, uint32_t* rec
         const uint32_t q0 = (unit - jb.first_unit) * (uint32_t)kChunk, n = (uint32_t)jb.w * (uint32_t)jb.h;
         const uint32_t w = (uint32_t)jb.w, len = n ? min((uint32_t)kChunk, n - q0) : 0u;
         if (lane == 0) s_ji = ji;
+        chain_wait();
         if (len > 0 && jb.vec && !(len & 3u)) {
             __syncwarp();
             if (lane == 0) mbar_arrive_tx(&full, 4u * len);
@@ -525,6 +526,7 @@ k_rle_code(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, uint32_t* rec
             }
         }
     }
+    chain_wait();
     __syncthreads();
     const RleJobDesc& jb = J.j[s_ji];
     if (jb.n_chunks == 0) return;                     // an empty image: its header is the scan's
@@ -793,7 +795,7 @@ __device__ __forceinline__ void dense_chunk(const RleJobDesc& jb, uint32_t q0, i
         const uint32_t next = ((SEG[b] >> 16) & 1u) | (((P0 + 16 - sb15) & 127) == 0 ? 1u : 0u);
         PSV[b] = PS & VALID;
         PE[b] = ((PS | (next << 16)) >> 1) & VALID;
-        cost[b] = __popc(~REP[b] & VALID) + __popc(PSV[b]) + __popc(PSV[b] & REP[b]);
+        cost[b] = __popc((~REP[b] & VALID) | (PSV[b] & REP[b])) + __popc(PSV[b]);
     }
     P4 tsum = {0u, 0u}, ssum = {0u, 0u};
     if (act) ssum = warp_scan4<false>(P4{cost[0] | (cost[1] << 16), cost[2] | (cost[3] << 16)}, lane, &tsum);
@@ -839,7 +841,7 @@ __device__ __forceinline__ void dense_chunk(const RleJobDesc& jb, uint32_t q0, i
             for (uint32_t m = PE[b]; m; m &= m - 1u) {
                 const int i = __ffs(m) - 1;
                 const uint32_t le = (2u << i) - 1u;
-                uint8_t* const e = o + __popc(lit & le) + __popc(psv & le) + __popc(psv & rep & le);   // past the piece
+                uint8_t* const e = o + __popc((lit | (psv & rep)) & le) + __popc(psv & le);   // past the piece
                 const uint32_t h = seg16 & le;
                 const int sbk = h ? P0 + 31 - __clz(h) : sbin[b];
                 const uint32_t jj = (uint32_t)(P0 + i - sbk) & 127u;
@@ -1156,6 +1158,7 @@ k_rle_compress0(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, uint32_t
     WarpRing& W = reinterpret_cast<WarpRing*>(smem)[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     const uint32_t T = J.total_units;
+    chain_wait();
     unsigned long long* cursor = reinterpret_cast<unsigned long long*>(ticket + 2);   // pool bytes taken
     if (lane == 0) {
         for (int q = 0; q < kSlots; ++q) mbar_init(&W.full[q], 1);
@@ -1243,6 +1246,13 @@ k_rle_compress0(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, uint32_t
     }
 }
 
+// The counters of a launch: ticket, chunks to recode, pool cursor.
+__global__ void k_rle_begin(uint4* counters)
+{
+    chain_wait();
+    if (threadIdx.x == 0) *counters = make_uint4(0u, 0u, 0u, 0u);
+}
+
 // Scan kernel: one CTA per job.  The exclusive prefix of the job's chunk sizes
 // gives every chunk its offset in the payload (written to its record); the
 // job's header and stream size are written here too.
@@ -1253,6 +1263,7 @@ k_rle_scan(const __grid_constant__ RleJobList<N> J, ChunkRec* rec)
     __shared__ uint32_t wsum[32];
     const RleJobDesc& jb = J.j[blockIdx.x];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    chain_wait();
     uint8_t* dst = reinterpret_cast<uint8_t*>(jb.dst);
     const uint32_t nc = jb.n_chunks;
     if (nc == 0) {                                    // empty image: header only
@@ -1287,17 +1298,15 @@ k_rle_scan(const __grid_constant__ RleJobList<N> J, ChunkRec* rec)
     }
 }
 
-// Placing kernel: kPlaceLanes lanes (a quarter-warp) per chunk copy its
-// streams from the pool to their place and write its end-table entries (four;
-// one in mode 0), so a warp's four chunks have their loads in flight together.
-// Listed chunks (dense, or to be coded again) are left to the recoding kernel.
+// Placing: kPlaceLanes lanes (a quarter-warp) per chunk copy its streams from
+// the pool to their place and write its end-table entries (four; one in mode
+// 0), so a warp's four chunks have their loads in flight together.  Listed
+// chunks (dense, or to be coded again) are left to the recoding kernel.
 constexpr int kPlaceLanes = 8;
 template <int N>
-__global__ void __launch_bounds__(128)
-k_rle_place(const __grid_constant__ RleJobList<N> J, const ChunkRec* rec, const uint8_t* pool)
+__device__ __forceinline__ void place_chunk(const RleJobList<N>& J, const ChunkRec* rec, const uint8_t* pool,
+                                            uint32_t unit, int lane)
 {
-    const int lane = (int)threadIdx.x % kPlaceLanes;
-    const uint32_t unit = blockIdx.x * (128u / kPlaceLanes) + threadIdx.x / kPlaceLanes;
     if (unit >= J.total_units) return;
     const ChunkRec r = rec[unit];                     // (in flight during the job search)
     const RleJobDesc& jb = J.j[find_job(J, unit)];
@@ -1319,26 +1328,42 @@ k_rle_place(const __grid_constant__ RleJobList<N> J, const ChunkRec* rec, const 
     if (lane < 4) put_u32(dst + 32 + 16ull * c + 4u * lane, r.off + mine);
 }
 
+// Mode 0's placing kernel.
+template <int N>
+__global__ void __launch_bounds__(128, 8)
+k_rle_place(const __grid_constant__ RleJobList<N> J, const ChunkRec* rec, const uint8_t* pool)
+{
+    chain_wait();
+    place_chunk(J, rec, pool, blockIdx.x * (128u / kPlaceLanes) + threadIdx.x / kPlaceLanes,
+                (int)threadIdx.x % kPlaceLanes);
+}
+
 // Recoding kernels: the listed chunks (dense, or sparse ones that found the
 // pool full), a CTA of 8 warps per listed chunk over a persistent grid.  Before
 // the scan (PLACE false) the dense ones are coded from the image into the
 // stage; their sizes go to their records and, where the pool has room, their
 // streams to the pool with 16-byte stores.  After it (PLACE true) the pooled
 // ones are copied to their place, the others coded (again) from the image and
-// copied from the stage; both write the four end-table entries.
+// copied from the stage; both write the four end-table entries.  That launch
+// also places the sparse chunks, with the CTAs behind the first `grid`.
 constexpr int kDenseStage = 4 * (kChunk + kChunk / 128) + 64;   // all literals, copy_out's read-ahead, whole sectors
 
 template <int N, bool PLACE>
 __global__ void __launch_bounds__(256, 4)
 k_rle_recode(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, const uint32_t* recode, uint32_t* ticket,
-             uint8_t* pool, size_t pool_bytes)
+             uint8_t* pool, size_t pool_bytes, uint32_t grid)
 {
     __shared__ P4 xw[16];
     __shared__ __align__(16) uint8_t stage[kDenseStage];
     __shared__ uint32_t s_pool;
-    const uint32_t n = ticket[1];
+    chain_wait();
     const int tid = threadIdx.x;
-    for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) {
+    if (PLACE && blockIdx.x >= grid) {
+        place_chunk(J, rec, pool, (blockIdx.x - grid) * (256u / kPlaceLanes) + (uint32_t)tid / kPlaceLanes, tid % kPlaceLanes);
+        return;
+    }
+    const uint32_t n = ticket[1];
+    for (uint32_t i = blockIdx.x; i < n; i += grid) {
         const uint32_t unit = recode[i];
         const RleJobDesc& jb = J.j[find_job(J, unit)];
         const uint32_t nc = jb.n_chunks, c = unit - jb.first_unit;
@@ -1396,6 +1421,7 @@ k_rle0_recode(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, const uint
     __shared__ __align__(16) uint8_t stage[kStage0];
     __shared__ uint32_t wt[kT / 32];
     const int tid = threadIdx.x;
+    chain_wait();
     const uint32_t n = *count;
     for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) {
         const uint32_t unit = recode[i];
@@ -1630,6 +1656,7 @@ k_rle_decompress(const __grid_constant__ RleJobList<N> J, uint32_t* status)
     const uint64_t size = jb.capacity;
     const uint32_t nc = jb.n_chunks;
     const uint32_t c = unit - jb.first_unit;
+    chain_wait();
     const rlec::ChunkEnds E = rlec::check_chunk(src, size, size, (uint32_t)jb.w, (uint32_t)jb.h, nc, c, true);
     if (E.bad) {
         if (tid == 0) set_status(status, EC_ERR_CORRUPT);
@@ -1777,21 +1804,25 @@ cudaError_t compress_n(const RleJobDesc* jobs, int n, uint32_t total_units, void
         const uint32_t pb = (uint32_t)std::min<size_t>(pool_bytes, 0xFFFFFFF0u);
         uint32_t slab = std::min<uint32_t>(pb / (8u * (uint32_t)grid * kWPB), 16384u) & ~255u;
         if (slab < 4u * kStagePlane) slab = 0u;
-        k_rle_compress0<N><<<grid, 32 * kWPB, kCompressSmem, s>>>(J, rec, recode, pool, pb, slab, ticket, status);
+        e = launch_chained(k_rle_compress0<N>, grid, 32 * kWPB, kCompressSmem, s, J, rec, recode, pool, pb, slab, ticket,
+                           status);
+        if (e != cudaSuccess) return e;
+        if ((e = launch_chained(k_rle0_recode<N, false>, rgrid, kT, 0, s, J, rec, recode, ticket + 1)) != cudaSuccess) return e;
     } else {
-        k_rle_code<N><<<total_units, kCT, 0, s>>>(J, rec, recode, pool, pool_bytes, ticket, status);
+        e = launch_chained(k_rle_code<N>, total_units, kCT, 0, s, J, rec, recode, pool, pool_bytes, ticket, status);
+        if (e != cudaSuccess) return e;
+        e = launch_chained(k_rle_recode<N, false>, rgrid, 256, 0, s, J, rec, recode, ticket, pool, pool_bytes, (uint32_t)rgrid);
+        if (e != cudaSuccess) return e;
     }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (M0) k_rle0_recode<N, false><<<rgrid, kT, 0, s>>>(J, rec, recode, ticket + 1);
-    else k_rle_recode<N, false><<<rgrid, 256, 0, s>>>(J, rec, recode, ticket, pool, pool_bytes);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_rle_scan<N><<<n, 1024, 0, s>>>(J, rec);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_rle_place<N><<<(total_units + 128 / kPlaceLanes - 1) / (128 / kPlaceLanes), 128, 0, s>>>(J, rec, pool);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (M0) k_rle0_recode<N, true><<<rgrid, kT, 0, s>>>(J, rec, recode, ticket + 1);
-    else k_rle_recode<N, true><<<rgrid, 256, 0, s>>>(J, rec, recode, ticket, pool, pool_bytes);
-    return cudaGetLastError();
+    if ((e = launch_chained(k_rle_scan<N>, n, 1024, 0, s, J, rec)) != cudaSuccess) return e;
+    if (M0) {
+        e = launch_chained(k_rle_place<N>, (total_units + 128 / kPlaceLanes - 1) / (128 / kPlaceLanes), 128, 0, s, J, rec, pool);
+        if (e != cudaSuccess) return e;
+        return launch_chained(k_rle0_recode<N, true>, rgrid, kT, 0, s, J, rec, recode, ticket + 1);
+    }
+    const uint32_t place = (total_units + 256 / kPlaceLanes - 1) / (256 / kPlaceLanes);
+    return launch_chained(k_rle_recode<N, true>, (uint32_t)rgrid + place, 256, 0, s, J, rec, recode, ticket, pool, pool_bytes,
+                          (uint32_t)rgrid);
 }
 
 }  // namespace
@@ -1807,7 +1838,8 @@ cudaError_t launch_rle_compress(const RleJobDesc* jobs, int n, uint32_t total_un
 {
     if (n <= 0 || total_units == 0) return cudaSuccess;
     if (scratch_bytes < rle_compress_scratch_bytes(total_units, 0)) return cudaErrorInvalidValue;
-    const cudaError_t e = cudaMemsetAsync(scratch, 0, 16, s);   // ticket, recode count, pool cursor
+    // (a memset between the kernels would end the chain)
+    const cudaError_t e = launch_chained(k_rle_begin, 1, 32, 0, s, reinterpret_cast<uint4*>(scratch));
     if (e != cudaSuccess) return e;
     if (jobs[0].mode == 0) {                      // (one launch codes one mode family)
         if (n <= 8) return compress_n<8, true>(jobs, n, total_units, scratch, scratch_bytes, status, s);
@@ -1829,10 +1861,10 @@ cudaError_t launch_rle_decompress(const RleJobDesc* jobs, int n, uint32_t total_
                                   uint32_t* status, cudaStream_t s)
 {
     if (n <= 0 || total_units == 0) return cudaSuccess;
-    if (n <= 8) k_rle_decompress<8><<<total_units, kDT, 0, s>>>(make_jobs<8>(jobs, n, total_units), status);
-    else if (n <= 64) k_rle_decompress<64><<<total_units, kDT, 0, s>>>(make_jobs<64>(jobs, n, total_units), status);
-    else k_rle_decompress<kRleJobsPerLaunch><<<total_units, kDT, 0, s>>>(make_jobs<kRleJobsPerLaunch>(jobs, n, total_units), status);
-    return cudaGetLastError();
+    if (n <= 8) return launch_chained(k_rle_decompress<8>, total_units, kDT, 0, s, make_jobs<8>(jobs, n, total_units), status);
+    if (n <= 64) return launch_chained(k_rle_decompress<64>, total_units, kDT, 0, s, make_jobs<64>(jobs, n, total_units), status);
+    return launch_chained(k_rle_decompress<kRleJobsPerLaunch>, total_units, kDT, 0, s,
+                          make_jobs<kRleJobsPerLaunch>(jobs, n, total_units), status);
 }
 
 }  // namespace ec

@@ -147,6 +147,7 @@ k_detect_roi(const __grid_constant__ RoiList<N> L, uint32_t* acc)
     __syncthreads();
     const int img = find_image(L, blk);
     const RoiDesc& d = L.d[img];
+    chain_wait();
     const uint32_t bi = blk - d.first_block;
     const int bx = (int)(bi % (uint32_t)d.bw), by = (int)(bi / (uint32_t)d.bw);
     const int px0 = bx * kRoiBlkW, py0 = by * kRoiBlkH;
@@ -195,6 +196,7 @@ struct RoiOrigins {
 __global__ void k_roi_finalize(const __grid_constant__ RoiOrigins O, uint32_t* acc, ec_rect* out)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    chain_wait();
     if (i >= O.n) return;
     const uint4 a = reinterpret_cast<const uint4*>(acc)[i];
     ec_rect r{0, 0, 0, 0};
@@ -224,8 +226,7 @@ cudaError_t scan_kind(RoiDesc* d, const int* kinds, const uint32_t* nblocks, int
     }
     L.blocks = blocks;
     if (blocks == 0) return cudaSuccess;
-    k_detect_roi<kRoiPerLaunch, KIND><<<blocks, kRT, 0, s>>>(L, acc);
-    return cudaGetLastError();
+    return launch_chained(k_detect_roi<kRoiPerLaunch, KIND>, blocks, kRT, 0, s, L, acc);
 }
 
 }  // namespace
@@ -243,8 +244,7 @@ cudaError_t launch_detect_roi(RoiDesc* d, const int* kinds, const uint32_t* nblo
     O.n = n;
     O.pad = 0;
     for (int i = 0; i < n; ++i) O.o[i] = make_int2(d[i].ox, d[i].oy);
-    k_roi_finalize<<<(n + 127) / 128, 128, 0, s>>>(O, scratch, out);
-    return cudaGetLastError();
+    return launch_chained(k_roi_finalize, (n + 127) / 128, 128, 0, s, O, scratch, out);
 }
 
 }  // namespace ec

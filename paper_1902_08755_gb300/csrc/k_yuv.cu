@@ -149,6 +149,7 @@ k_yuv_encode(const __grid_constant__ YuvJobList<N> J)
     constexpr int kNP = kEncNP;
     int bp, by;
     const YuvJob& jb = tile_job<kNP>(J, blockIdx.x, bp, by);
+    chain_wait();
     const uint32_t* __restrict__ src = jb.src;
     uint32_t* __restrict__ dst = jb.dst;
     const int w = jb.w, h = jb.h, pitch = jb.pitch, dpitch = jb.dpitch, vec = jb.vec;
@@ -249,6 +250,7 @@ k_yuv_decode(const __grid_constant__ YuvJobList<N> J)
     constexpr int kNP = kDecNP;
     int bp, by;
     const YuvJob& jb = tile_job<kNP>(J, blockIdx.x, bp, by);
+    chain_wait();
     const uint32_t* __restrict__ src = jb.src;
     uint32_t* __restrict__ dst = jb.dst;
     const int w = jb.w, h = jb.h, pitch = jb.pitch, spitch = jb.dpitch, vec = jb.vec;
@@ -303,9 +305,8 @@ cudaError_t launch_n(const YuvJob* jobs, int n, uint32_t tiles, cudaStream_t s)
     YuvJobList<N> J;
     J.n = n;
     for (int i = 0; i < n; ++i) J.j[i] = jobs[i];
-    if (ENC) k_yuv_encode<N><<<tiles, dim3(kYX, kYY), 0, s>>>(J);
-    else k_yuv_decode<N><<<tiles, dim3(kYX, kYY), 0, s>>>(J);
-    return cudaGetLastError();
+    if (ENC) return launch_chained(k_yuv_encode<N>, tiles, dim3(kYX, kYY), 0, s, J);
+    return launch_chained(k_yuv_decode<N>, tiles, dim3(kYX, kYY), 0, s, J);
 }
 
 }  // namespace
