@@ -187,13 +187,13 @@ ec_status ec_composite_depth_backward(ec_ctx* ctx, const int16_t* winner,
                                       ec_stream_t s);
 
 /* --------------------------------------------------------- batched compositing
- * Many independent composites in one persistent launch.  Thesis 4.2.4 (tile
+ * Many independent composites in a few persistent launches.  Thesis 4.2.4 (tile
  * compounds): fixed-size work packages wait in a queue and are pulled until it
  * is empty, which balances uneven work.  A plan cuts every job's destination
  * into tiles (work items), sorts them by estimated cost (largest first),
- * uploads all descriptors once and captures one launch -- a queue-head reset
- * and a grid of resident CTAs that pull items with an atomic counter -- in a
- * CUDA graph; ec_batch_run replays that graph.  Results are bit-identical to
+ * uploads all descriptors once and captures the launches -- a reset of the
+ * queue heads and, per kind of item, a grid of resident CTAs that pull items
+ * with an atomic counter -- in a CUDA graph; ec_batch_run replays that graph.  Results are bit-identical to
  * calling ec_composite_depth / ec_composite_alpha per job, whatever the tile
  * shapes. */
 enum { EC_JOB_DEPTH = 0, EC_JOB_ALPHA = 1 };

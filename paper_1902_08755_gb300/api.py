@@ -567,7 +567,7 @@ class Job:
 
 
 class Batch:
-    """ec_batch: many composites in one persistent, graph-captured launch.
+    """ec_batch: many composites in a few persistent, graph-captured launches.
 
     ``config=None`` autotunes the tile shapes on the jobs themselves (running
     them, so the destinations are written during construction).  The tensors

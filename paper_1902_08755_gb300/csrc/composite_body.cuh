@@ -83,6 +83,38 @@ __device__ __forceinline__ void load4(const SrcDesc& s, int x, int y, float (&d)
     }
 }
 
+// Write the merged pixels x + j STEP of row y: depth, colour, winner.
+template <int CB, int STEP>
+__device__ __forceinline__ void store_depth4(const DstDesc& D, int x, int y, const float (&bd)[4],
+                                             const typename ColorT<CB>::T (&bc)[4], const int (&bi)[4])
+{
+    using C = typename ColorT<CB>::T;
+    const size_t o = (size_t)y * (size_t)D.pitch + (size_t)x;
+    C* oc = reinterpret_cast<C*>(D.color) + o;
+    if (STEP == 1 && D.vec && x + 4 <= D.W) {
+        if constexpr (CB == 4) st_stream(reinterpret_cast<uint4*>(oc), make_uint4(bc[0], bc[1], bc[2], bc[3]));
+        else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) st_stream(oc + j, bc[j]);
+        }
+        if (D.depth) st_stream(reinterpret_cast<float4*>(D.depth + o), make_float4(bd[0], bd[1], bd[2], bd[3]));
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (x + j * STEP < D.W) {
+                oc[j * STEP] = bc[j];
+                if (D.depth) D.depth[o + j * STEP] = bd[j];
+            }
+        }
+    }
+    if (D.winner) {
+        int16_t* w = D.winner + (size_t)y * D.W + x;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (x + j * STEP < D.W) w[j * STEP] = (int16_t)bi[j];
+    }
+}
+
 // Depth merge of the 4 pixels x + j STEP of row y (output-relative coordinates),
 // U inputs' loads in flight per thread.  STEP 1: a lane's pixels are adjacent
 // and inputs whose rows allow it are read 16 bytes at a time.  STEP 32: a
@@ -133,30 +165,7 @@ __device__ __forceinline__ void depth_px4(At at, const int16_t* act, int nact, i
         }
     }
 
-    const size_t o = (size_t)y * (size_t)D.pitch + (size_t)x;
-    C* oc = reinterpret_cast<C*>(D.color) + o;
-    if (STEP == 1 && D.vec && x + 4 <= D.W) {
-        if constexpr (CB == 4) st_stream(reinterpret_cast<uint4*>(oc), make_uint4(bc[0], bc[1], bc[2], bc[3]));
-        else {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) st_stream(oc + j, bc[j]);
-        }
-        if (D.depth) st_stream(reinterpret_cast<float4*>(D.depth + o), make_float4(bd[0], bd[1], bd[2], bd[3]));
-    } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            if (x + j * STEP < D.W) {
-                oc[j * STEP] = bc[j];
-                if (D.depth) D.depth[o + j * STEP] = bd[j];
-            }
-        }
-    }
-    if (D.winner) {
-        int16_t* w = D.winner + (size_t)y * D.W + x;
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (x + j * STEP < D.W) w[j * STEP] = (int16_t)bi[j];
-    }
+    store_depth4<CB, STEP>(D, x, y, bd, bc, bi);
 }
 
 // ----------------------------------------------------------------- alpha ---
@@ -225,6 +234,54 @@ __device__ __forceinline__ float4 pixel_of(const uint4& v, int j)
     }
 }
 
+// C += T c (premultiplied, all four channels); T *= (1 - a)
+__device__ __forceinline__ void over(const float4& c, float4& acc, float& T)
+{
+    acc.x = fmaf(T, c.x, acc.x);
+    acc.y = fmaf(T, c.y, acc.y);
+    acc.z = fmaf(T, c.z, acc.z);
+    acc.w = fmaf(T, c.w, acc.w);
+    T = fmaf(-T, c.w, T);
+}
+
+// Write the blended pixels x, x + 1 (FP16) of row y and what is left of their
+// transmittance.
+template <bool F16>
+__device__ __forceinline__ void store_alpha(const DstDesc& D, int x, int y, const float4 (&acc)[F16 ? 2 : 1],
+                                            const float (&T)[F16 ? 2 : 1])
+{
+    constexpr int PX = F16 ? 2 : 1;
+    const size_t o = (size_t)y * (size_t)D.pitch + (size_t)x;
+    if constexpr (!F16) {
+        float4* op = reinterpret_cast<float4*>(D.color) + o;
+        if (D.vec) st_stream(op, acc[0]);
+        else { float* f = reinterpret_cast<float*>(op); f[0] = acc[0].x; f[1] = acc[0].y; f[2] = acc[0].z; f[3] = acc[0].w; }
+    } else {
+        uint2* op = reinterpret_cast<uint2*>(D.color) + o;
+        const uint2 h0 = float4_to_half4(acc[0]), h1 = float4_to_half4(acc[1]);
+        if (D.vec && x + 2 <= D.W) {
+            st_stream(reinterpret_cast<uint4*>(op), make_uint4(h0.x, h0.y, h1.x, h1.y));
+        } else if ((reinterpret_cast<uintptr_t>(op) & 7u) == 0) {      // whole pixels
+            op[0] = h0;
+            if (x + 1 < D.W) op[1] = h1;
+        } else {
+            unsigned short* hp = reinterpret_cast<unsigned short*>(op);
+            hp[0] = (unsigned short)h0.x; hp[1] = (unsigned short)(h0.x >> 16);
+            hp[2] = (unsigned short)h0.y; hp[3] = (unsigned short)(h0.y >> 16);
+            if (x + 1 < D.W) {
+                hp[4] = (unsigned short)h1.x; hp[5] = (unsigned short)(h1.x >> 16);
+                hp[6] = (unsigned short)h1.y; hp[7] = (unsigned short)(h1.y >> 16);
+            }
+        }
+    }
+    if (D.tfinal) {
+        float* t = D.tfinal + (size_t)y * D.W + x;
+#pragma unroll
+        for (int j = 0; j < PX; ++j)
+            if (x + j < D.W) t[j] = T[j];
+    }
+}
+
 // Front-to-back "over" of the active layers at the thread's PX pixels, U
 // layers' loads in flight per thread.  full (uniform over the CTA): every
 // active layer's ROI covers the CTA's whole tile, so the per-layer and
@@ -263,45 +320,12 @@ __device__ __forceinline__ void alpha_px(At at, const int16_t* act, int nact, in
                 const int xj = x + j;
                 if (!full && (xj < s.x0 || xj >= s.x1)) continue;   // transparent outside the ROI
                 const float4 c = pixel_of<F16>(raw[u], j);
-                // C += T c (premultiplied, all four channels); T *= (1 - a)
-                acc[j].x = fmaf(T[j], c.x, acc[j].x);
-                acc[j].y = fmaf(T[j], c.y, acc[j].y);
-                acc[j].z = fmaf(T[j], c.z, acc[j].z);
-                acc[j].w = fmaf(T[j], c.w, acc[j].w);
-                T[j] = fmaf(-T[j], c.w, T[j]);
+                over(c, acc[j], T[j]);
             }
         }
     }
 
-    const size_t o = (size_t)y * (size_t)D.pitch + (size_t)x;
-    if constexpr (!F16) {
-        float4* op = reinterpret_cast<float4*>(D.color) + o;
-        if (D.vec) st_stream(op, acc[0]);
-        else { float* f = reinterpret_cast<float*>(op); f[0] = acc[0].x; f[1] = acc[0].y; f[2] = acc[0].z; f[3] = acc[0].w; }
-    } else {
-        uint2* op = reinterpret_cast<uint2*>(D.color) + o;
-        const uint2 h0 = float4_to_half4(acc[0]), h1 = float4_to_half4(acc[1]);
-        if (D.vec && x + 2 <= D.W) {
-            st_stream(reinterpret_cast<uint4*>(op), make_uint4(h0.x, h0.y, h1.x, h1.y));
-        } else if ((reinterpret_cast<uintptr_t>(op) & 7u) == 0) {      // whole pixels
-            op[0] = h0;
-            if (x + 1 < D.W) op[1] = h1;
-        } else {
-            unsigned short* hp = reinterpret_cast<unsigned short*>(op);
-            hp[0] = (unsigned short)h0.x; hp[1] = (unsigned short)(h0.x >> 16);
-            hp[2] = (unsigned short)h0.y; hp[3] = (unsigned short)(h0.y >> 16);
-            if (x + 1 < D.W) {
-                hp[4] = (unsigned short)h1.x; hp[5] = (unsigned short)(h1.x >> 16);
-                hp[6] = (unsigned short)h1.y; hp[7] = (unsigned short)(h1.y >> 16);
-            }
-        }
-    }
-    if (D.tfinal) {
-        float* t = D.tfinal + (size_t)y * D.W + x;
-#pragma unroll
-        for (int j = 0; j < PX; ++j)
-            if (x + j < D.W) t[j] = T[j];
-    }
+    store_alpha<F16>(D, x, y, acc, T);
 }
 
 }  // namespace ec

@@ -788,6 +788,7 @@ struct ec_batch {
     uint32_t* d_head = nullptr;
     size_t items_cap = 0;
     int n_items = 0;
+    int kind_items[kBatchKinds] = {};     // of them, per kind (the items are grouped by kind)
     BatchShape shape{};
     int grid = 0;
     int ctas_per_sm = 0;
@@ -803,10 +804,11 @@ std::map<std::string, BatchShape> g_tune_cache;
 
 int job_kind(const BatchJob& j) { return j.mode; }
 
-// Work items for one tile shape, sorted by estimated bytes moved, largest first.
-std::vector<BatchItem> make_items(const ec_batch& b, const BatchShape& sh)
+// Work items for one tile shape, grouped by kind (count[k] of kind k), each group
+// sorted by estimated bytes moved, largest first.
+std::vector<BatchItem> make_items(const ec_batch& b, const BatchShape& sh, int* count)
 {
-    struct Costed { double cost; int idx; BatchItem it; };
+    struct Costed { double cost; int kind; BatchItem it; };
     std::vector<Costed> v;
     for (size_t j = 0; j < b.jobs.size(); ++j) {
         const BatchJob& J = b.jobs[j];
@@ -819,20 +821,29 @@ std::vector<BatchItem> make_items(const ec_batch& b, const BatchShape& sh)
                 const int x0 = x * TW, y0 = y * TH;
                 const int x1 = std::min(x0 + TW, J.D.W), y1 = std::min(y0 + TH, J.D.H);
                 double cost = (double)(x1 - x0) * (y1 - y0) * bpp;           // output
+                bool covered = true;
                 for (int i = 0; i < J.n; ++i) {
                     const SrcDesc& s = b.srcs[J.first + i];
                     const int64_t w = std::min(x1, s.x1) - std::max(x0, s.x0);
                     const int64_t h = std::min(y1, s.y1) - std::max(y0, s.y0);
-                    if (w > 0 && h > 0) cost += (double)w * h * bpp;
+                    if (w <= 0 || h <= 0) continue;
+                    cost += (double)w * h * bpp;
+                    covered = covered && w == x1 - x0 && h == y1 - y0 && (s.vec || J.step != 1);
                 }
                 BatchItem it;
                 it.job = (int32_t)j;
                 it.tx = (int16_t)x;
                 it.ty = (int16_t)y;
-                v.push_back({cost, (int)v.size(), it});
+                it.first = J.first;
+                it.n = J.n;
+                v.push_back({cost, batch_kind(J, covered), it});
             }
     }
-    std::stable_sort(v.begin(), v.end(), [](const Costed& a, const Costed& c) { return a.cost > c.cost; });
+    std::stable_sort(v.begin(), v.end(), [](const Costed& a, const Costed& c) {
+        return a.kind != c.kind ? a.kind < c.kind : a.cost > c.cost;
+    });
+    for (int k = 0; k < kBatchKinds; ++k) count[k] = 0;
+    for (const Costed& c : v) ++count[c.kind];
     std::vector<BatchItem> out(v.size());
     for (size_t i = 0; i < v.size(); ++i) out[i] = v[i].it;
     return out;
@@ -840,7 +851,7 @@ std::vector<BatchItem> make_items(const ec_batch& b, const BatchShape& sh)
 
 ec_status upload_items(ec_batch& b, const BatchShape& sh)
 {
-    const std::vector<BatchItem> items = make_items(b, sh);
+    const std::vector<BatchItem> items = make_items(b, sh, b.kind_items);
     if (items.size() > b.items_cap) {
         if (b.d_items) cudaFree(b.d_items);
         b.d_items = nullptr;
@@ -861,7 +872,7 @@ ec_status capture(ec_batch& b)
     if (b.exec) { cudaGraphExecDestroy(b.exec); b.exec = nullptr; }
     if (b.graph) { cudaGraphDestroy(b.graph); b.graph = nullptr; }
     if (cudaStreamBeginCapture(b.stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return EC_ERR_CUDA;
-    const cudaError_t e = launch_batch(b.d_jobs, b.d_srcs, b.d_items, b.n_items, b.d_head, b.shape, b.grid, b.stream);
+    const cudaError_t e = launch_batch(b.d_jobs, b.d_srcs, b.d_items, b.kind_items, b.d_head, b.shape, b.grid, b.stream);
     const cudaError_t e2 = cudaStreamEndCapture(b.stream, &b.graph);
     if (e != cudaSuccess || e2 != cudaSuccess) return EC_ERR_CUDA;
     if (cudaGraphInstantiate(&b.exec, b.graph, 0) != cudaSuccess) return EC_ERR_CUDA;
@@ -878,7 +889,7 @@ float time_shape(ec_batch& b, const BatchShape& sh)
     float best = 1e30f;
     for (int r = 0; r < 4; ++r) {
         cudaEventRecord(e0, b.stream);
-        launch_batch(b.d_jobs, b.d_srcs, b.d_items, b.n_items, b.d_head, b.shape, b.grid, b.stream);
+        launch_batch(b.d_jobs, b.d_srcs, b.d_items, b.kind_items, b.d_head, b.shape, b.grid, b.stream);
         cudaEventRecord(e1, b.stream);
         cudaEventSynchronize(e1);
         float ms = 0.f;
@@ -1015,6 +1026,9 @@ ec_status ec_batch_plan(ec_ctx* ctx, const ec_job* jobs, int32_t njobs, const ec
                 else st = make_desc(job.in[i], out->pvp, 4, true, &d[i]);
             }
             J.mode = out->format == EC_RGBA8 ? 0 : 1;
+            J.step = 1;
+            for (int i = 0; i < job.n && st == EC_OK; ++i)
+                if (!d[i].vec && d[i].x0 < d[i].x1) J.step = 32;
             J.D.vec = aligned16(out->color) && (!out->depth || aligned16(out->depth)) && out->pitch % 4 == 0;
             J.D.winner = job.winner;
             J.D.depth = out->depth;
@@ -1023,6 +1037,7 @@ ec_status ec_batch_plan(ec_ctx* ctx, const ec_job* jobs, int32_t njobs, const ec
             st = alpha_descs(job.in, job.order, job.n, out->format, out->pvp, d);
             const bool f16 = out->format == EC_RGBA16F;
             J.mode = f16 ? 3 : 2;
+            J.step = 1;
             J.D.vec = aligned16(out->color) && (!f16 || out->pitch % 2 == 0);
             J.D.tfinal = job.t_final;
         } else {
@@ -1047,7 +1062,7 @@ ec_status ec_batch_plan(ec_ctx* ctx, const ec_job* jobs, int32_t njobs, const ec
     if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess) return fail(EC_ERR_CUDA);
     if (cudaMalloc(&b->d_jobs, std::max<size_t>(b->jobs.size(), 1) * sizeof(BatchJob)) != cudaSuccess ||
         cudaMalloc(&b->d_srcs, std::max<size_t>(b->srcs.size(), 1) * sizeof(SrcDesc)) != cudaSuccess ||
-        cudaMalloc(&b->d_head, sizeof(uint32_t)) != cudaSuccess)
+        cudaMalloc(&b->d_head, kBatchKinds * sizeof(uint32_t)) != cudaSuccess)
         return fail(EC_ERR_CUDA);
     if ((!b->jobs.empty() && cudaMemcpy(b->d_jobs, b->jobs.data(), b->jobs.size() * sizeof(BatchJob), cudaMemcpyHostToDevice) != cudaSuccess) ||
         (!b->srcs.empty() && cudaMemcpy(b->d_srcs, b->srcs.data(), b->srcs.size() * sizeof(SrcDesc), cudaMemcpyHostToDevice) != cudaSuccess))
@@ -1078,7 +1093,7 @@ ec_status ec_batch_plan(ec_ctx* ctx, const ec_job* jobs, int32_t njobs, const ec
 
 cudaError_t ec::batch_enqueue(const ec_batch* b, cudaStream_t s)
 {
-    return launch_batch(b->d_jobs, b->d_srcs, b->d_items, b->n_items, b->d_head, b->shape, b->grid, s);
+    return launch_batch(b->d_jobs, b->d_srcs, b->d_items, b->kind_items, b->d_head, b->shape, b->grid, s);
 }
 
 extern "C" {

@@ -159,7 +159,7 @@ struct BatchJob {
     int32_t mode;
     int32_t n;
     int32_t first;
-    int32_t pad;
+    int32_t step;           // mode 0: distance of a lane's pixels (1, or 32 if an input must be read pixel by pixel)
     DstDesc D;
 };
 static_assert(sizeof(BatchJob) == 64, "batch job layout");
@@ -167,16 +167,23 @@ static_assert(sizeof(BatchJob) == 64, "batch job layout");
 struct BatchItem {
     int32_t job;
     int16_t tx, ty;
+    int32_t first, n;       // the job's inputs, repeated here (no dependent load)
 };
+static_assert(sizeof(BatchItem) == 16, "batch item layout");
 
 struct BatchShape {
     int32_t tw[4], th[4];   // tile width / height in pixels, per mode
 };
 
+constexpr int kBatchKinds = 10;         // kernels: an item goes to the one of its kind
+// Kind of an item of job j; covered: every input that meets its tile covers it,
+// with 16-byte rows unless j.step says that some have none.
+int batch_kind(const BatchJob& j, bool covered);
 int batch_warp_px(int mode);
 int batch_ctas_per_sm();
+// items are grouped by kind, n_items[k] of kind k; head: a queue head per kind.
 cudaError_t launch_batch(const BatchJob* jobs, const SrcDesc* srcs, const BatchItem* items,
-                         int n_items, uint32_t* head, const BatchShape& shape, int grid,
+                         const int* n_items, uint32_t* head, const BatchShape& shape, int grid,
                          cudaStream_t s);
 
 // ---- launchers (defined in the kernel translation units) -------------------
