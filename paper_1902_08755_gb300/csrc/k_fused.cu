@@ -106,12 +106,11 @@ __device__ __forceinline__ void load_local(const FusedStage& S, Quad& Q)
 
 // Run path of a decode unit: the chunk's elements are constant between the
 // union of its eight planes' run starts.  U: that union (128 words), PU: the
-// segments starting before each word, SC / SD: each segment's colour and depth.
+// segments starting before each word, S: each segment's colour and depth.
 struct Segs {
     const uint32_t* U;
     const uint32_t* PU;
-    const uint32_t* SC;
-    const uint32_t* SD;
+    const uint2* S;
 };
 
 template <bool CODED>
@@ -120,19 +119,20 @@ __device__ __forceinline__ void finish(const FusedStage& S, const Quad& Q, int q
 {
     uint32_t oc[4], od[4];
     if (CODED && G) {
-        const int i0 = Q.qa - q0;
+        // the segment of the quad's first element in the chunk, and the starts
+        // after it; most quads lie inside one segment
+        const int i0 = Q.qa - q0, a = max(i0, 0);
+        const uint32_t u0 = G->U[a >> 5], u1 = G->U[min((a >> 5) + 1, kChunk / 32 - 1)];
+        const uint32_t s0 = G->PU[a >> 5] + __popc(u0 & ((2u << (a & 31)) - 1u)) - 1u;
+        const uint32_t nb = __funnelshift_r(u0, u1, a & 31);   // bit j: element a + j starts one
+        const uint2 first = G->S[s0];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            uint32_t ic = 0u, id = kBgDepth;
-            if (k >= Q.lo && k < Q.hi) {
-                const int i = i0 + k;
-                const uint32_t u = G->U[i >> 5];
-                const uint32_t s = G->PU[i >> 5] + __popc(u & ((2u << (i & 31)) - 1u)) - 1u;
-                ic = G->SC[s];
-                id = G->SD[s];
-            }
-            if (S.front) merge(ic, id, Q.lc[k], Q.ld[k], oc[k], od[k]);
-            else merge(Q.lc[k], Q.ld[k], ic, id, oc[k], od[k]);
+            uint2 v = first;
+            const int j = i0 + k - a;                          // (>= 0 for the quad's pixels in the unit)
+            if ((nb & 0xEu) && k >= Q.lo && k < Q.hi) v = G->S[s0 + __popc(nb & ((2u << j) - 2u))];
+            if (S.front) merge(v.x, v.y, Q.lc[k], Q.ld[k], oc[k], od[k]);
+            else merge(Q.lc[k], Q.ld[k], v.x, v.y, oc[k], od[k]);
         }
     } else if (CODED) {
         // bytes of elements qa - q0 .. +3 of every plane: two words and a funnel shift
@@ -285,8 +285,7 @@ k_fused_depth(const FusedStage* __restrict__ stages, const FusedUnit* __restrict
         uint32_t* U = reinterpret_cast<uint32_t*>(base8 + 6144);
         uint32_t* PU = U + 128;
         uint32_t* wt = PU + 128;                                     // scan scratch
-        uint32_t* SC = reinterpret_cast<uint32_t*>(base8 + 7296);    // <= 8 * 255 segments
-        uint32_t* SD = SC + 2040;
+        uint2* SS = reinterpret_cast<uint2*>(base8 + 7296);          // <= 8 * 255 segments
         const uint8_t* val = base8 + 4096;
         const bool csw = s_mode[0] == 2, dsw = s_mode[1] == 2;
         uint32_t un = 0u, eu = 0u, ec = 0u, ed = 0u, wb[8];
@@ -323,12 +322,11 @@ k_fused_depth(const FusedStage* __restrict__ stages, const FusedUnit* __restrict
                     d |= (uint32_t)val[256 * (4 + q) + rd] << (8 * q);
                 }
                 const uint32_t sidx = eu + __popc(un & (le >> 1));
-                SC[sidx] = csw ? rlec::swizzle(c) : c;
-                SD[sidx] = dsw ? rlec::swizzle(d) : d;
+                SS[sidx] = make_uint2(csw ? rlec::swizzle(c) : c, dsw ? rlec::swizzle(d) : d);
             }
         }
         __syncthreads();
-        const Segs G{U, PU, SC, SD};
+        const Segs G{U, PU, SS};
         compose<true>(S, u, ra, rb - ra + 1, (int)q0, len, planes, false, false, &G);
         return;
     }

@@ -340,8 +340,8 @@ constexpr int kCT = 128;
 
 // Plane stream of a chunk of len elements from its m <= 32 change points, run
 // by run, where every run is at least 3 bytes (so all of it is repeat tokens).
-// Lane i holds change point i: byte v at position q (valid: i < m).  Returns
-// the bytes written, or 0 (nothing written) when a run is shorter.
+// Lane i holds change point i: byte v at position q (valid: i < m); out is even.
+// Returns the bytes written, or 0 (nothing written) when a run is shorter.
 __device__ __forceinline__ uint32_t code_plane_few(bool valid, uint32_t v, int q, int len, uint8_t* out)
 {
     const int lane = threadIdx.x & 31;
@@ -355,13 +355,11 @@ __device__ __forceinline__ uint32_t code_plane_few(bool valid, uint32_t v, int q
     const uint32_t cost = keep ? 2u * (uint32_t)((L + 127) >> 7) : 0u;
     const uint32_t incl = (uint32_t)rlec::warp_incl_sum((int)cost, lane);
     const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-    if (keep) {
-        uint8_t* o = out + (incl - cost);
-        for (int r = L; r > 0; r -= 128) {
-            o[0] = (uint8_t)(127 + min(r, 128));
-            o[1] = (uint8_t)v;
-            o += 2;
-        }
+    if (keep) {                                       // (out and every token's place are even)
+        uint16_t* o = reinterpret_cast<uint16_t*>(out + (incl - cost));
+        int r = L;
+        for (; r > 128; r -= 128) *o++ = (uint16_t)(0xFFu | (v << 8));
+        *o = (uint16_t)((uint32_t)(127 + r) | (v << 8));
     }
     return total;
 }
@@ -536,16 +534,22 @@ k_rle_code(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, uint32_t* rec
         mbar_wait(&full, 0u, status);
     } else {                                          // (also a contiguous image that ends inside a 16-byte group)
         const uint32_t w = (uint32_t)jb.w;
-        uint32_t y = row_of(jb, q0 + (uint32_t)tid), x = q0 + (uint32_t)tid - y * w;
-        for (int i = tid; i < len; i += kCT) {
-            cp_async4(el + i, jb.src + (size_t)y * jb.pitch + x);
-            x += (uint32_t)kCT;
-            if (w >= (uint32_t)kCT) {
-                if (x >= w) { x -= w; ++y; }
-            } else {
-                y = row_of(jb, q0 + (uint32_t)(i + kCT));
-                x = q0 + (uint32_t)(i + kCT) - y * w;
+        const uint32_t y = row_of(jb, q0 + (uint32_t)tid);
+        if (w >= (uint32_t)kCT) {                     // at most one row further per step
+            uint32_t x = q0 + (uint32_t)tid - y * w;
+            const uint32_t* p = jb.src + (size_t)y * jb.pitch + x;
+            const int64_t skip = (int64_t)jb.pitch - jb.w;
+            uint32_t* to = el + tid;
+#pragma unroll 8
+            for (int i = tid; i < len; i += kCT) {
+                cp_async4(to, p);
+                to += kCT;
+                p += kCT;
+                x += (uint32_t)kCT;
+                if (x >= w) { x -= w; p += skip; }
             }
+        } else {
+            for (int i = tid; i < len; i += kCT) cp_async4(el + i, jb.src + elem_off(jb, q0 + (uint32_t)i));
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
