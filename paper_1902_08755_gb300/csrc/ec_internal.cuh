@@ -226,9 +226,9 @@ struct RleJobList {
 };
 static_assert(sizeof(RleJobList<kRleJobsPerLaunch>) < 32764 - 256, "kernel parameter limit");
 
-// Scratch of a compress launch of `units` work units: a ticket, a counter and a
-// pool cursor, a 16-byte record and a 4-byte list entry per unit, then a pool
-// of pool_bytes for the coded chunks.  A chunk that finds the pool full is
+// Scratch of a compress launch of `units` work units: two counters and a pool
+// cursor, a 16-byte record and two 4-byte list entries per unit, a sum per 32
+// units, then a pool of pool_bytes for the coded chunks.  A chunk that finds the pool full is
 // coded a second time when placed, so any pool size gives the same stream.
 size_t rle_compress_scratch_bytes(uint32_t units, size_t pool_bytes);
 

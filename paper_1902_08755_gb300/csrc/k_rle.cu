@@ -137,9 +137,10 @@ __device__ __forceinline__ void copy_out(uint8_t* __restrict__ o, const uint8_t*
 // The coding kernels list each chunk's change points.  A chunk of few of them
 // (sparse) is coded at once from the list, its streams left in a scratch pool;
 // the others (dense) are listed, and a recoding kernel codes them from the
-// image.  A scan over each job's chunk sizes gives every chunk its offset; the
-// placing kernels copy the pooled chunks to their place, and code those that
-// the pool had no room for again.  No kernel waits for another's warps.
+// image.  A chunk's offset is the sum of its image's chunk sizes before it (sums
+// over 32 chunks are taken while they are coded; mode 0 scans them); the placing
+// kernels copy the pooled chunks to their place, and code those that the pool
+// had no room for again.  No kernel waits for another's warps.
 //
 // Four-plane modes: a CTA of four warps per chunk (k_rle_code).  Mode 0: every
 // warp of a persistent kernel works alone, chunk after chunk (k_rle_compress0):
@@ -177,14 +178,26 @@ static_assert((kQ + 4) * 4 % 16 == 0 && sizeof(WarpRing) % 16 == 0, "16-byte ali
 // A coded chunk, as the coding kernels leave it for the placing kernels: its
 // four plane stream sizes, where its streams wait in the pool (a sparse chunk's
 // offset / 4, a dense chunk's offset / 16 with kDense, or kRecode: not kept,
-// coded again from the image when placed), and its offset inside the stream's
-// payload (written by the scan).
+// coded again from the image when placed), and, in mode 0, its offset inside the
+// stream's payload (written by the scan).
 struct ChunkRec {
     uint16_t T[4];
     uint32_t pool;
     uint32_t off;
 };
 static_assert(sizeof(ChunkRec) == 16, "chunk record");
+
+// A launch's scratch.
+constexpr uint32_t kGroup = 32;                // chunks whose sizes are summed up while they are coded
+struct RleScratch {
+    uint32_t* counters;     // [0] mode 0: ticket, else sparse chunks to code again; [1] listed chunks; [2, 3] pool cursor
+    ChunkRec* rec;          // per chunk
+    uint32_t* recode;       // listed chunks: the dense ones, in mode 0 also those that found the pool full
+    uint32_t* again;        // sparse chunks that found the pool full
+    uint32_t* groups;       // bytes coded per kGroup chunks
+    uint8_t* pool;
+    size_t pool_bytes;
+};
 constexpr size_t kCompressSmem = kWPB * sizeof(WarpRing);
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -485,8 +498,7 @@ __device__ __forceinline__ uint32_t code_plane_many(const uint32_t* el, const ui
 
 template <int N>
 __global__ void __launch_bounds__(kCT, 12)
-k_rle_code(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, uint32_t* recode, uint8_t* pool, size_t pool_bytes,
-           uint32_t* ticket, uint32_t* status)
+k_rle_code(const __grid_constant__ RleJobList<N> J, const RleScratch W, uint32_t* status)
 {
     __shared__ __align__(16) uint32_t raw[4 + kChunk];      // the chunk, after a guard
     __shared__ __align__(16) uint8_t stage[4][kStagePlane];
@@ -534,19 +546,26 @@ k_rle_code(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, uint32_t* rec
         mbar_wait(&full, 0u, status);
     } else {                                          // (also a contiguous image that ends inside a 16-byte group)
         const uint32_t w = (uint32_t)jb.w;
-        const uint32_t y = row_of(jb, q0 + (uint32_t)tid);
-        if (w >= (uint32_t)kCT) {                     // at most one row further per step
-            uint32_t x = q0 + (uint32_t)tid - y * w;
-            const uint32_t* p = jb.src + (size_t)y * jb.pitch + x;
-            const int64_t skip = (int64_t)jb.pitch - jb.w;
-            uint32_t* to = el + tid;
-#pragma unroll 8
-            for (int i = tid; i < len; i += kCT) {
-                cp_async4(to, p);
-                to += kCT;
-                p += kCT;
-                x += (uint32_t)kCT;
-                if (x >= w) { x -= w; p += skip; }
+        if (w >= 32u) {                               // a warp takes a quarter of the chunk, a row's part at a time
+            int q = kChunk / 4 * warp;
+            const int qe = min(len, q + kChunk / 4);
+            const uint32_t y = row_of(jb, q0 + (uint32_t)min(q, len - 1));
+            uint32_t x = q0 + (uint32_t)q - y * w;
+            const uint32_t* row = jb.src + (size_t)y * jb.pitch;
+            while (q < qe) {
+                const int n = min((int)(w - x), qe - q);
+                const uint32_t* from = row + x + lane;
+                uint32_t* to = el + q + lane;
+                for (int i = lane; i < n; i += 256) {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        if (i + 32 * k < n) cp_async4(to + 32 * k, from + 32 * k);
+                    from += 256;
+                    to += 256;
+                }
+                q += n;
+                x = 0u;
+                row += jb.pitch;
             }
         } else {
             for (int i = tid; i < len; i += kCT) cp_async4(el + i, jb.src + elem_off(jb, q0 + (uint32_t)i));
@@ -582,8 +601,7 @@ k_rle_code(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, uint32_t* rec
     const int m = (int)(n0 + n1 + n2 + n3);
     if (m > kCap) {                                   // dense: coded by the recoding kernel
         if (tid == 0) {
-            rec[unit] = ChunkRec{{0, 0, 0, 0}, kRecode, 0u};
-            recode[atomicAdd(ticket + 1, 1u)] = unit;
+            W.recode[atomicAdd(W.counters + 1, 1u)] = unit;
         }
         return;
     }
@@ -611,13 +629,13 @@ k_rle_code(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, uint32_t* rec
     const size_t slots = kRlePoolPerUnit * (size_t)J.total_units;
     const uint32_t need = (total + 4u + 31u) & ~31u;
     uint32_t po = kRecode;
-    if (need <= kRlePoolPerUnit && kRlePoolPerUnit * ((size_t)unit + 1) <= pool_bytes)
+    if (need <= kRlePoolPerUnit && kRlePoolPerUnit * ((size_t)unit + 1) <= W.pool_bytes)
         po = unit * (uint32_t)(kRlePoolPerUnit / 4);
     if (po == kRecode) {
         if (tid == 0) {
-            const unsigned long long a = slots + atomicAdd(reinterpret_cast<unsigned long long*>(ticket + 2),
+            const unsigned long long a = slots + atomicAdd(reinterpret_cast<unsigned long long*>(W.counters + 2),
                                                            (unsigned long long)need);
-            s_po = a + need <= pool_bytes ? (uint32_t)(a >> 2) : kRecode;
+            s_po = a + need <= W.pool_bytes ? (uint32_t)(a >> 2) : kRecode;
         }
         __syncthreads();
         po = s_po;
@@ -626,12 +644,13 @@ k_rle_code(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, uint32_t* rec
         uint8_t* flat = reinterpret_cast<uint8_t*>(el) + (warp > 0 ? T0 : 0u) + (warp > 1 ? T1 : 0u) + (warp > 2 ? T2 : 0u);
         for (uint32_t i = lane; i < T; i += 32) flat[i] = stage[warp][i];
         __syncthreads();
-        uint4* o = reinterpret_cast<uint4*>(pool + 4 * (size_t)po);
+        uint4* o = reinterpret_cast<uint4*>(W.pool + 4 * (size_t)po);
         for (uint32_t i = tid; 16u * i < need; i += kCT) o[i] = reinterpret_cast<const uint4*>(el)[i];
     }
     if (tid == 0) {
-        rec[unit] = ChunkRec{{(uint16_t)T0, (uint16_t)T1, (uint16_t)T2, (uint16_t)T3}, po, 0u};
-        if (po == kRecode) recode[atomicAdd(ticket + 1, 1u)] = unit;   // coded again when placed
+        W.rec[unit] = ChunkRec{{(uint16_t)T0, (uint16_t)T1, (uint16_t)T2, (uint16_t)T3}, po, 0u};
+        atomicAdd(W.groups + unit / kGroup, total);
+        if (po == kRecode) W.again[atomicAdd(W.counters, 1u)] = unit;
     }
 }
 
@@ -1250,16 +1269,18 @@ k_rle_compress0(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, uint32_t
     }
 }
 
-// The counters of a launch: ticket, chunks to recode, pool cursor.
-__global__ void k_rle_begin(uint4* counters)
+// Clears the counters and the groups' sums.
+__global__ void k_rle_begin(uint4* counters, uint32_t* groups, uint32_t n)
 {
     chain_wait();
-    if (threadIdx.x == 0) *counters = make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) *counters = make_uint4(0u, 0u, 0u, 0u);
+    if (i < n) groups[i] = 0u;
 }
 
-// Scan kernel: one CTA per job.  The exclusive prefix of the job's chunk sizes
-// gives every chunk its offset in the payload (written to its record); the
-// job's header and stream size are written here too.
+// Mode 0's scan kernel: one CTA per job.  The exclusive prefix of the job's
+// chunk sizes gives every chunk its offset in the payload (written to its
+// record); the job's header and stream size are written here too.
 template <int N>
 __global__ void __launch_bounds__(1024)
 k_rle_scan(const __grid_constant__ RleJobList<N> J, ChunkRec* rec)
@@ -1302,114 +1323,168 @@ k_rle_scan(const __grid_constant__ RleJobList<N> J, ChunkRec* rec)
     }
 }
 
-// Placing: kPlaceLanes lanes (a quarter-warp) per chunk copy its streams from
-// the pool to their place and write its end-table entries (four; one in mode
-// 0), so a warp's four chunks have their loads in flight together.  Listed
-// chunks (dense, or to be coded again) are left to the recoding kernel.
 constexpr int kPlaceLanes = 8;
-template <int N>
-__device__ __forceinline__ void place_chunk(const RleJobList<N>& J, const ChunkRec* rec, const uint8_t* pool,
-                                            uint32_t unit, int lane)
-{
-    if (unit >= J.total_units) return;
-    const ChunkRec r = rec[unit];                     // (in flight during the job search)
-    const RleJobDesc& jb = J.j[find_job(J, unit)];
-    const uint32_t nc = jb.n_chunks;
-    if (nc == 0) return;                              // header written by the scan
-    if (r.pool & kDense) return;                      // (kRecode too: the recoding kernel's)
-    const uint8_t* from = pool + 4ull * r.pool;
-    const uint32_t c = unit - jb.first_unit;
-    const uint32_t T0 = r.T[0], T1 = r.T[1], T2 = r.T[2], T3 = r.T[3];
-    const uint32_t total = T0 + T1 + T2 + T3;
-    uint8_t* dst = reinterpret_cast<uint8_t*>(jb.dst);
-    if (jb.mode == 0) {                               // one stream, one end-table entry
-        copy_out(dst + 32 + 4ull * nc + r.off, from, total, lane, kPlaceLanes);
-        if (lane == 0) put_u32(dst + 32 + 4ull * c, r.off + total);
-        return;
-    }
-    copy_out(dst + 32 + 16ull * nc + r.off, from, total, lane, kPlaceLanes);
-    const uint32_t mine = lane == 0 ? T0 : lane == 1 ? T0 + T1 : lane == 2 ? T0 + T1 + T2 : total;
-    if (lane < 4) put_u32(dst + 32 + 16ull * c + 4u * lane, r.off + mine);
-}
 
-// Mode 0's placing kernel.
+// Mode 0's placing kernel: kPlaceLanes lanes (a quarter-warp) per chunk copy its
+// stream from the pool to its place and write its end-table entry, so a warp's
+// four chunks have their loads in flight together.  Listed chunks are left to
+// the recoding kernel.
 template <int N>
 __global__ void __launch_bounds__(128, 8)
 k_rle_place(const __grid_constant__ RleJobList<N> J, const ChunkRec* rec, const uint8_t* pool)
 {
     chain_wait();
-    place_chunk(J, rec, pool, blockIdx.x * (128u / kPlaceLanes) + threadIdx.x / kPlaceLanes,
-                (int)threadIdx.x % kPlaceLanes);
+    const uint32_t unit = blockIdx.x * (128u / kPlaceLanes) + threadIdx.x / kPlaceLanes;
+    const int lane = (int)threadIdx.x % kPlaceLanes;
+    if (unit >= J.total_units) return;
+    const ChunkRec r = rec[unit];                     // (in flight during the job search)
+    const RleJobDesc& jb = J.j[find_job(J, unit)];
+    const uint32_t nc = jb.n_chunks;
+    if (nc == 0 || r.pool == kRecode) return;         // (an empty image's header is written by the scan)
+    uint8_t* dst = reinterpret_cast<uint8_t*>(jb.dst);
+    copy_out(dst + 32 + 4ull * nc + r.off, pool + 4ull * r.pool, r.T[0], lane, kPlaceLanes);
+    if (lane == 0) put_u32(dst + 32 + 4ull * (unit - jb.first_unit), r.off + r.T[0]);
 }
 
-// Recoding kernels: the listed chunks (dense, or sparse ones that found the
-// pool full), a CTA of 8 warps per listed chunk over a persistent grid.  Before
-// the scan (PLACE false) the dense ones are coded from the image into the
-// stage; their sizes go to their records and, where the pool has room, their
-// streams to the pool with 16-byte stores.  After it (PLACE true) the pooled
-// ones are copied to their place, the others coded (again) from the image and
-// copied from the stage; both write the four end-table entries.  That launch
-// also places the sparse chunks, with the CTAs behind the first `grid`.
+// Bytes of the chunks [f, u), from the groups' sums where they lie inside: the
+// part of one of kRT threads.
+constexpr uint32_t kRT = 256;
+__device__ __forceinline__ uint32_t bytes_between(const RleScratch& W, uint32_t f, uint32_t u, uint32_t tid)
+{
+    auto of = [&](uint32_t c) {
+        const ChunkRec& r = W.rec[c];
+        return (uint32_t)r.T[0] + r.T[1] + r.T[2] + r.T[3];
+    };
+    const uint32_t g0 = (f + kGroup - 1) / kGroup, g1 = u / kGroup;
+    uint32_t sum = 0u;
+    if (g0 >= g1) {                                   // (then fewer than 2 kGroup chunks)
+        if (f + tid < u) sum = of(f + tid);
+        return sum;
+    }
+    if (tid < kGroup) {
+        if (f + tid < kGroup * g0) sum = of(f + tid);
+    } else if (tid < 2 * kGroup) {
+        if (kGroup * g1 + tid - kGroup < u) sum = of(kGroup * g1 + tid - kGroup);
+    }
+    for (uint32_t g = g0 + tid; g < g1; g += kRT) sum += W.groups[g];
+    return sum;
+}
+
+__device__ __forceinline__ uint32_t warp_sum(uint32_t v)
+{
+    return __reduce_add_sync(0xffffffffu, v);
+}
+
+// Placing, a CTA per kGroup chunks.  A chunk's place is the sum of its image's
+// chunks before it: the groups' sums up to the CTA's first chunk and a scan of
+// the CTA's own.  kPlaceLanes lanes copy a sparse chunk, so a warp's four have
+// their loads in flight together (a dense one is another CTA's); the end-table
+// entries, and with an image's last chunk its header and stream size, are
+// written here for all chunks.  (A scan launch of a CTA per image between the
+// coding and the placing launch took 2.9 us more: 8.1 us for both against 5.2 us
+// for the 32 pieces of a 1920x1080 swap's level.)
+template <int N>
+__device__ __forceinline__ void place_group(const RleJobList<N>& J, const RleScratch& W, uint32_t group, uint32_t* sum)
+{
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = kGroup * group;
+    const uint32_t k = tid / kPlaceLanes, sub = tid % kPlaceLanes, unit = b + k;
+    const bool in = unit < J.total_units;
+    const ChunkRec r = in ? W.rec[unit] : ChunkRec{{0, 0, 0, 0}, kRecode, 0u};
+    uint32_t own = 0u;                                // lane i: the size of the group's i-th chunk
+    if (b + lane < J.total_units) {
+        const ChunkRec& o = W.rec[b + lane];
+        own = (uint32_t)o.T[0] + o.T[1] + o.T[2] + o.T[3];
+    }
+    const RleJobDesc& jb = J.j[find_job(J, in ? unit : J.total_units - 1u)];
+    const uint32_t nc = jb.n_chunks, f = jb.first_unit, f0 = J.j[find_job(J, b)].first_unit;
+    const uint32_t part = warp_sum(bytes_between(W, f0, b, tid));
+    if (lane == 0) sum[warp] = part;
+    __syncthreads();
+    uint32_t base = 0u;
+#pragma unroll
+    for (int i = 0; i < (int)kRT / 32; ++i) base += sum[i];
+    const uint32_t ex = (uint32_t)rlec::warp_incl_sum((int)own, (int)lane) - own;
+    const uint32_t pk = __shfl_sync(0xffffffffu, ex, k), pf = __shfl_sync(0xffffffffu, ex, (f - b) & 31u);
+    const uint32_t off = f < b ? base + pk : pk - pf;
+    const uint32_t T0 = r.T[0], T1 = r.T[1], T2 = r.T[2], T3 = r.T[3], total = T0 + T1 + T2 + T3;
+    uint8_t* const dst = reinterpret_cast<uint8_t*>(jb.dst);
+    if (!in) return;
+    if (nc > 0 && !(r.pool & kDense)) copy_out(dst + 32 + 16ull * nc + off, W.pool + 4ull * r.pool, total, sub, kPlaceLanes);
+    if (nc > 0) {
+        const uint32_t mine = sub == 0 ? T0 : sub == 1 ? T0 + T1 : sub == 2 ? T0 + T1 + T2 : total;
+        if (sub < 4) put_u32(dst + 32 + 16ull * (unit - f) + 4u * sub, off + mine);
+    }
+    if (sub == 0 && (nc == 0 || unit - f == nc - 1u)) {
+        write_header(dst, jb);
+        *jb.d_size = 32ull + 16ull * nc + (nc ? off + total : 0u);
+    }
+}
+
+// Recoding kernels, a CTA of 8 warps per listed chunk over a persistent grid.
+// Before placing (PLACE false) the dense chunks are coded from the image into
+// the stage; their sizes go to their records and their groups' sums and, where
+// the pool has room, their streams to the pool with 16-byte stores.  The
+// placing launch (PLACE true) copies the pooled ones to their place; the others,
+// and the sparse ones that found the pool full, are coded (again) from the image
+// and copied from the stage.  Its first CTAs place the sparse chunks.
 constexpr int kDenseStage = 4 * (kChunk + kChunk / 128) + 64;   // all literals, copy_out's read-ahead, whole sectors
 
 template <int N, bool PLACE>
-__global__ void __launch_bounds__(256, 4)
-k_rle_recode(const __grid_constant__ RleJobList<N> J, ChunkRec* rec, const uint32_t* recode, uint32_t* ticket,
-             uint8_t* pool, size_t pool_bytes, uint32_t grid)
+__global__ void __launch_bounds__(kRT, 4)
+k_rle_recode(const __grid_constant__ RleJobList<N> J, const RleScratch W, uint32_t grid)
 {
     __shared__ P4 xw[16];
     __shared__ __align__(16) uint8_t stage[kDenseStage];
-    __shared__ uint32_t s_pool;
+    __shared__ uint32_t s_pool, s_sum[kRT / 32];
     chain_wait();
     const int tid = threadIdx.x;
-    if (PLACE && blockIdx.x >= grid) {
-        place_chunk(J, rec, pool, (blockIdx.x - grid) * (256u / kPlaceLanes) + (uint32_t)tid / kPlaceLanes, tid % kPlaceLanes);
-        return;
+    uint32_t first = blockIdx.x;
+    if (PLACE) {
+        const uint32_t groups = gridDim.x - grid;
+        if (first < groups) {
+            place_group(J, W, first, s_sum);
+            return;
+        }
+        first -= groups;
     }
-    const uint32_t n = ticket[1];
-    for (uint32_t i = blockIdx.x; i < n; i += grid) {
-        const uint32_t unit = recode[i];
+    const uint32_t dense = W.counters[1], n = dense + (PLACE ? W.counters[0] : 0u);
+    for (uint32_t i = first; i < n; i += grid) {
+        const uint32_t unit = i < dense ? W.recode[i] : W.again[i - dense];
         const RleJobDesc& jb = J.j[find_job(J, unit)];
-        const uint32_t nc = jb.n_chunks, c = unit - jb.first_unit;
-        const ChunkRec r = rec[unit];
-        uint32_t T[4] = {r.T[0], r.T[1], r.T[2], r.T[3]};
-        const uint32_t q0 = c * (uint32_t)kChunk;
+        const uint32_t q0 = (unit - jb.first_unit) * (uint32_t)kChunk;
         const int len = (int)min((uint32_t)kChunk, (uint32_t)jb.w * (uint32_t)jb.h - q0);
+        uint32_t T[4];
         if (!PLACE) {
-            if (T[0] != 0u) continue;                         // sized already (a sparse chunk)
             dense_chunk(jb, q0, len, jb.mode == 2, T, stage, xw);
             const uint32_t total = T[0] + T[1] + T[2] + T[3];
             if (tid == 0) {
                 const uint32_t need = (total + 4u + 31u) & ~31u;
                 const unsigned long long a = kRlePoolPerUnit * (unsigned long long)J.total_units +
-                    atomicAdd(reinterpret_cast<unsigned long long*>(ticket + 2), (unsigned long long)need);
-                s_pool = a + need <= pool_bytes ? kDense | (uint32_t)(a >> 4) : kRecode;
-                ChunkRec o;
-                o.T[0] = (uint16_t)T[0]; o.T[1] = (uint16_t)T[1]; o.T[2] = (uint16_t)T[2]; o.T[3] = (uint16_t)T[3];
-                o.pool = s_pool;
-                o.off = 0u;
-                rec[unit] = o;
+                    atomicAdd(reinterpret_cast<unsigned long long*>(W.counters + 2), (unsigned long long)need);
+                s_pool = a + need <= W.pool_bytes ? kDense | (uint32_t)(a >> 4) : kRecode;
+                W.rec[unit] = ChunkRec{{(uint16_t)T[0], (uint16_t)T[1], (uint16_t)T[2], (uint16_t)T[3]}, s_pool, 0u};
+                atomicAdd(W.groups + unit / kGroup, total);
             }
             __syncthreads();                                  // the stage is complete
             if (s_pool != kRecode) {
-                uint4* to = reinterpret_cast<uint4*>(pool + ((size_t)(s_pool & ~kDense) << 4));
-                for (uint32_t j = tid; 32u * (j >> 1) < total + 4u; j += 256u)   // (whole 32-byte sectors)
+                uint4* to = reinterpret_cast<uint4*>(W.pool + ((size_t)(s_pool & ~kDense) << 4));
+                for (uint32_t j = tid; 32u * (j >> 1) < total + 4u; j += kRT)    // (whole 32-byte sectors)
                     to[j] = reinterpret_cast<const uint4*>(stage)[j];
             }
         } else {
-            uint8_t* dst = reinterpret_cast<uint8_t*>(jb.dst);
-            const uint8_t* from = pool + ((size_t)(r.pool & ~kDense) << 4);
-            if (r.pool == kRecode) {
-                dense_chunk(jb, q0, len, jb.mode == 2, T, stage, xw);
-                __syncthreads();
-                from = stage;
-            }
-            const uint32_t total = T[0] + T[1] + T[2] + T[3];
-            copy_out(dst + 32 + 16ull * nc + r.off, from, total, tid, 256);
-            const uint32_t mine = tid == 0 ? T[0] : tid == 1 ? T[0] + T[1] : tid == 2 ? T[0] + T[1] + T[2] : total;
-            if (tid < 4) put_u32(dst + 32 + 16ull * c + 4u * tid, r.off + mine);
+            const ChunkRec r = W.rec[unit];
+            const uint32_t part = warp_sum(bytes_between(W, jb.first_unit, unit, (uint32_t)tid));
+            if ((tid & 31) == 0) s_sum[tid >> 5] = part;
+            if (r.pool == kRecode) dense_chunk(jb, q0, len, jb.mode == 2, T, stage, xw);
+            __syncthreads();                                  // (the stage is complete, too)
+            uint32_t off = 0u;
+#pragma unroll
+            for (int k = 0; k < (int)kRT / 32; ++k) off += s_sum[k];
+            const uint8_t* from = r.pool == kRecode ? stage : W.pool + ((size_t)(r.pool & ~kDense) << 4);
+            copy_out(reinterpret_cast<uint8_t*>(jb.dst) + 32 + 16ull * jb.n_chunks + off, from,
+                     (uint32_t)r.T[0] + r.T[1] + r.T[2] + r.T[3], tid, kRT);
         }
-        __syncthreads();                                      // stage and xw are reused
+        __syncthreads();                                      // stage, xw and s_sum are reused
     }
 }
 
@@ -1779,62 +1854,60 @@ cudaError_t compress_grid(int* grid)
     return cudaSuccess;
 }
 
-// Code (a CTA per chunk; in mode 0 persistent warps), code or size the dense
-// chunks, scan the sizes (a CTA per job), place (a quarter-warp per chunk), place
-// or write the dense chunks.  M0: basic RLE.
-template <int N, bool M0>
-cudaError_t compress_n(const RleJobDesc* jobs, int n, uint32_t total_units, void* scratch, size_t scratch_bytes,
-                       uint32_t* status, cudaStream_t s)
+// Mode 0: code (persistent warps), size the dense chunks, scan the sizes (a CTA
+// per job), place (a quarter-warp per chunk), write the listed chunks.
+template <int N>
+cudaError_t compress0(const RleJobDesc* jobs, int n, uint32_t total_units, const RleScratch& W, int rgrid,
+                      uint32_t* status, cudaStream_t s)
 {
     cudaError_t e;
-    uint32_t* ticket = reinterpret_cast<uint32_t*>(scratch);     // [0] ticket, [1] chunks to recode, [2, 3] pool cursor
-    ChunkRec* rec = reinterpret_cast<ChunkRec*>(reinterpret_cast<char*>(scratch) + 16);
-    uint32_t* recode = reinterpret_cast<uint32_t*>(rec + total_units);
-    const size_t used = rle_compress_scratch_bytes(total_units, 0), pool_bytes = scratch_bytes - used;
-    uint8_t* pool = reinterpret_cast<uint8_t*>(scratch) + used;
     const RleJobList<N> J = make_jobs<N>(jobs, n, total_units);
-    int sms = 0;
-    int dev = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const int rgrid = std::max(1, sms) * 4;
-    if (M0) {
-        int grid = 0;
-        if ((e = compress_grid<N>(&grid)) != cudaSuccess) return e;
-        grid = (int)std::min<uint32_t>((uint32_t)grid, (total_units + kWPB - 1) / kWPB);
-        // pool space is taken in slabs of up to 16 KB per warp where the pool
-        // has room for eight slabs per warp of the grid (their unused tails are
-        // then at most an eighth of it), else chunk by chunk
-        const uint32_t pb = (uint32_t)std::min<size_t>(pool_bytes, 0xFFFFFFF0u);
-        uint32_t slab = std::min<uint32_t>(pb / (8u * (uint32_t)grid * kWPB), 16384u) & ~255u;
-        if (slab < 4u * kStagePlane) slab = 0u;
-        e = launch_chained(k_rle_compress0<N>, grid, 32 * kWPB, kCompressSmem, s, J, rec, recode, pool, pb, slab, ticket,
-                           status);
-        if (e != cudaSuccess) return e;
-        if ((e = launch_chained(k_rle0_recode<N, false>, rgrid, kT, 0, s, J, rec, recode, ticket + 1)) != cudaSuccess) return e;
-    } else {
-        e = launch_chained(k_rle_code<N>, total_units, kCT, 0, s, J, rec, recode, pool, pool_bytes, ticket, status);
-        if (e != cudaSuccess) return e;
-        e = launch_chained(k_rle_recode<N, false>, rgrid, 256, 0, s, J, rec, recode, ticket, pool, pool_bytes, (uint32_t)rgrid);
-        if (e != cudaSuccess) return e;
-    }
-    if ((e = launch_chained(k_rle_scan<N>, n, 1024, 0, s, J, rec)) != cudaSuccess) return e;
-    if (M0) {
-        e = launch_chained(k_rle_place<N>, (total_units + 128 / kPlaceLanes - 1) / (128 / kPlaceLanes), 128, 0, s, J, rec, pool);
-        if (e != cudaSuccess) return e;
-        return launch_chained(k_rle0_recode<N, true>, rgrid, kT, 0, s, J, rec, recode, ticket + 1);
-    }
-    const uint32_t place = (total_units + 256 / kPlaceLanes - 1) / (256 / kPlaceLanes);
-    return launch_chained(k_rle_recode<N, true>, (uint32_t)rgrid + place, 256, 0, s, J, rec, recode, ticket, pool, pool_bytes,
+    int grid = 0;
+    if ((e = compress_grid<N>(&grid)) != cudaSuccess) return e;
+    grid = (int)std::min<uint32_t>((uint32_t)grid, (total_units + kWPB - 1) / kWPB);
+    // pool space is taken in slabs of up to 16 KB per warp where the pool
+    // has room for eight slabs per warp of the grid (their unused tails are
+    // then at most an eighth of it), else chunk by chunk
+    const uint32_t pb = (uint32_t)std::min<size_t>(W.pool_bytes, 0xFFFFFFF0u);
+    uint32_t slab = std::min<uint32_t>(pb / (8u * (uint32_t)grid * kWPB), 16384u) & ~255u;
+    if (slab < 4u * kStagePlane) slab = 0u;
+    e = launch_chained(k_rle_compress0<N>, grid, 32 * kWPB, kCompressSmem, s, J, W.rec, W.recode, W.pool, pb, slab,
+                       W.counters, status);
+    if (e != cudaSuccess) return e;
+    const uint32_t* count = W.counters + 1;
+    if ((e = launch_chained(k_rle0_recode<N, false>, rgrid, kT, 0, s, J, W.rec, W.recode, count)) != cudaSuccess) return e;
+    if ((e = launch_chained(k_rle_scan<N>, n, 1024, 0, s, J, W.rec)) != cudaSuccess) return e;
+    constexpr uint32_t per = 128 / kPlaceLanes;
+    e = launch_chained(k_rle_place<N>, (total_units + per - 1) / per, 128, 0, s, J, W.rec, W.pool);
+    if (e != cudaSuccess) return e;
+    return launch_chained(k_rle0_recode<N, true>, rgrid, kT, 0, s, J, W.rec, W.recode, count);
+}
+
+// The four-plane modes: code (a CTA per chunk), code the dense chunks, place.
+template <int N>
+cudaError_t compress_n(const RleJobDesc* jobs, int n, uint32_t total_units, const RleScratch& W, int rgrid,
+                       uint32_t* status, cudaStream_t s)
+{
+    const RleJobList<N> J = make_jobs<N>(jobs, n, total_units);
+    cudaError_t e = launch_chained(k_rle_code<N>, total_units, kCT, 0, s, J, W, status);
+    if (e != cudaSuccess) return e;
+    if ((e = launch_chained(k_rle_recode<N, false>, rgrid, kRT, 0, s, J, W, (uint32_t)rgrid)) != cudaSuccess) return e;
+    return launch_chained(k_rle_recode<N, true>, (uint32_t)rgrid + (total_units + kGroup - 1) / kGroup, kRT, 0, s, J, W,
                           (uint32_t)rgrid);
+}
+
+// Offsets of the scratch's parts after the counters; the pool starts at a 128-byte line.
+constexpr size_t scratch_groups(uint32_t units) { return 16 + (sizeof(ChunkRec) + 8) * (size_t)units; }
+constexpr size_t scratch_pool(uint32_t units)
+{
+    return (scratch_groups(units) + 4 * (((size_t)units + kGroup - 1) / kGroup) + 127) & ~(size_t)127;
 }
 
 }  // namespace
 
 size_t rle_compress_scratch_bytes(uint32_t units, size_t pool_bytes)
 {
-    const size_t u = std::max<uint32_t>(units, 1);
-    return ((16 + sizeof(ChunkRec) * u + 4 * u + 127) & ~(size_t)127) + pool_bytes;   // the pool starts at a 128-byte line
+    return scratch_pool(std::max<uint32_t>(units, 1)) + pool_bytes;
 }
 
 cudaError_t launch_rle_compress(const RleJobDesc* jobs, int n, uint32_t total_units,
@@ -1842,17 +1915,32 @@ cudaError_t launch_rle_compress(const RleJobDesc* jobs, int n, uint32_t total_un
 {
     if (n <= 0 || total_units == 0) return cudaSuccess;
     if (scratch_bytes < rle_compress_scratch_bytes(total_units, 0)) return cudaErrorInvalidValue;
+    char* base = reinterpret_cast<char*>(scratch);
+    RleScratch W;
+    W.counters = reinterpret_cast<uint32_t*>(base);
+    W.rec = reinterpret_cast<ChunkRec*>(base + 16);
+    W.recode = reinterpret_cast<uint32_t*>(W.rec + total_units);
+    W.again = W.recode + total_units;
+    W.groups = reinterpret_cast<uint32_t*>(base + scratch_groups(total_units));
+    W.pool = reinterpret_cast<uint8_t*>(base + scratch_pool(total_units));
+    W.pool_bytes = scratch_bytes - scratch_pool(total_units);
+    int sms = 0, dev = 0;
+    cudaError_t e;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    const int rgrid = std::max(1, sms) * 4;
     // (a memset between the kernels would end the chain)
-    const cudaError_t e = launch_chained(k_rle_begin, 1, 32, 0, s, reinterpret_cast<uint4*>(scratch));
+    const uint32_t ng = jobs[0].mode == 0 ? 0u : (total_units + kGroup - 1) / kGroup;
+    e = launch_chained(k_rle_begin, std::max(1u, (ng + 255) / 256), 256, 0, s, reinterpret_cast<uint4*>(scratch), W.groups, ng);
     if (e != cudaSuccess) return e;
     if (jobs[0].mode == 0) {                      // (one launch codes one mode family)
-        if (n <= 8) return compress_n<8, true>(jobs, n, total_units, scratch, scratch_bytes, status, s);
-        if (n <= 64) return compress_n<64, true>(jobs, n, total_units, scratch, scratch_bytes, status, s);
-        return compress_n<kRleJobsPerLaunch, true>(jobs, n, total_units, scratch, scratch_bytes, status, s);
+        if (n <= 8) return compress0<8>(jobs, n, total_units, W, rgrid, status, s);
+        if (n <= 64) return compress0<64>(jobs, n, total_units, W, rgrid, status, s);
+        return compress0<kRleJobsPerLaunch>(jobs, n, total_units, W, rgrid, status, s);
     }
-    if (n <= 8) return compress_n<8, false>(jobs, n, total_units, scratch, scratch_bytes, status, s);
-    if (n <= 64) return compress_n<64, false>(jobs, n, total_units, scratch, scratch_bytes, status, s);
-    return compress_n<kRleJobsPerLaunch, false>(jobs, n, total_units, scratch, scratch_bytes, status, s);
+    if (n <= 8) return compress_n<8>(jobs, n, total_units, W, rgrid, status, s);
+    if (n <= 64) return compress_n<64>(jobs, n, total_units, W, rgrid, status, s);
+    return compress_n<kRleJobsPerLaunch>(jobs, n, total_units, W, rgrid, status, s);
 }
 
 cudaError_t launch_selftest_wait(uint32_t* status, cudaStream_t s)
