@@ -33,17 +33,33 @@ constexpr int kFT = 256;
 constexpr int kChunk = rlec::kChunk;
 constexpr uint32_t kBgDepth = 0x3F800000u;   // 1.0f
 constexpr int kStageWords = 1024;             // staged stream bytes per stream: 4 KB
+// The run path's tables: bitmaps, run bytes, their union with its prefix, scan
+// scratch, segments (at most 8 * 255).
+constexpr int kRunArea = 4096 + 2048 + 512 + 512 + 128 + 8 * 2040;
+static_assert(kRunArea % 16 == 0 && kRunArea + 2 * 4 * kStageWords <= 8 * kChunk, "run path in the planes' space");
 
 __device__ __forceinline__ bool below_one(uint32_t d) { return __uint_as_float(d) < 1.0f; }
 __device__ __forceinline__ bool less(uint32_t a, uint32_t b) { return __uint_as_float(a) < __uint_as_float(b); }
 
-// Merge one pixel: front (fc, fd) and back (bc, bd) as raw bits.
-__device__ __forceinline__ void merge(uint32_t fc, uint32_t fd, uint32_t bc, uint32_t bd, uint32_t& oc, uint32_t& od)
+// A front pixel over the cleared background.
+__device__ __forceinline__ void clear_far(uint32_t& c, uint32_t& d)
 {
-    if (!below_one(fd)) { fc = 0u; fd = kBgDepth; }
+    if (!below_one(d)) { c = 0u; d = kBgDepth; }
+}
+
+// A cleared front pixel (fc, fd) and a back one (bc, bd), as raw bits.
+__device__ __forceinline__ void over(uint32_t fc, uint32_t fd, uint32_t bc, uint32_t bd, uint32_t& oc, uint32_t& od)
+{
     const bool b = less(bd, fd);
     oc = b ? bc : fc;
     od = b ? bd : fd;
+}
+
+// Merge one pixel.
+__device__ __forceinline__ void merge(uint32_t fc, uint32_t fd, uint32_t bc, uint32_t bd, uint32_t& oc, uint32_t& od)
+{
+    clear_far(fc, fd);
+    over(fc, fd, bc, bd, oc, od);
 }
 
 // Pixels are handled in quads: four horizontally adjacent pixels whose first
@@ -52,43 +68,42 @@ __device__ __forceinline__ void merge(uint32_t fc, uint32_t fd, uint32_t bc, uin
 // `nrows` rows of its rectangle from row `ra`; a decode unit only the elements
 // [q0, q0 + len) of its chunk (element q = row * w + column).
 struct Quad {
-    int fx, fy, lo, hi, qa;       // frame position, pixels [lo, hi) inside the unit, element of pixel 0
+    int r, x, lo, hi;             // row after the unit's first, column of pixel 0, pixels [lo, hi) inside the unit
     uint32_t lc[4], ld[4];        // the receiver's own image there
 };
 
+// What the quads of a unit share.  Columns are the rectangle's, rows count from
+// the unit's first.
 struct Grid {
-    int qx0, nq, slots;
-    float inv;
+    const uint32_t *lc, *ld;      // the local image at row 0, column 0
+    uint32_t *oc, *od;            // the output there
+    int lpitch, opitch;
+    int rx0, rx1, ry0, ry1;       // the local image's ROI
+    int w, e0, e1;                // columns; element of row 0, column 0 in the chunk; the chunk's length
+    bool lvec, ovec, front;
 };
 
 template <bool CODED>
-__device__ __forceinline__ bool quad_at(const FusedUnit& u, const Grid& g, int s, int ra, int q0, int len, Quad& Q)
+__device__ __forceinline__ bool bounds(const Grid& g, Quad& Q)
 {
-    int r = (int)((float)s * g.inv);
-    if (r * g.nq > s) --r;
-    else if ((r + 1) * g.nq <= s) ++r;
-    const int row = ra + r;
-    Q.fx = g.qx0 + 4 * (s - r * g.nq);
-    Q.fy = u.y + row;
-    const int xs = Q.fx - u.x;
-    Q.lo = max(0, -xs);
-    Q.hi = min(4, u.w - xs);
-    Q.qa = row * u.w + xs;
+    Q.lo = max(0, -Q.x);
+    Q.hi = min(4, g.w - Q.x);
     if (CODED) {
-        Q.lo = max(Q.lo, q0 - Q.qa);
-        Q.hi = min(Q.hi, q0 + len - Q.qa);
+        const int i0 = g.e0 + Q.r * g.w + Q.x;
+        Q.lo = max(Q.lo, -i0);
+        Q.hi = min(Q.hi, g.e1 - i0);
     }
     return Q.lo < Q.hi;
 }
 
 // The receiver's own image at the quad (background outside its ROI).
-__device__ __forceinline__ void load_local(const FusedStage& S, Quad& Q)
+__device__ __forceinline__ void load_local(const Grid& g, Quad& Q)
 {
-    const bool in_y = Q.fy >= S.r0y && Q.fy < S.r1y;
-    const size_t le = (size_t)(Q.fy - S.ly) * S.lpitch + (Q.fx - S.lx);
-    if (in_y && Q.fx >= S.r0x && Q.fx + 3 < S.r1x && S.lvec && (le & 3) == 0) {
-        const uint4 c = __ldcs(reinterpret_cast<const uint4*>(S.lc + le));
-        const uint4 d = __ldcs(reinterpret_cast<const uint4*>(S.ld + le));
+    const bool in_y = Q.r >= g.ry0 && Q.r < g.ry1;
+    const int64_t le = (int64_t)Q.r * g.lpitch + Q.x;
+    if (in_y && Q.x >= g.rx0 && Q.x + 3 < g.rx1 && g.lvec) {
+        const uint4 c = __ldcs(reinterpret_cast<const uint4*>(g.lc + le));
+        const uint4 d = __ldcs(reinterpret_cast<const uint4*>(g.ld + le));
         Q.lc[0] = c.x; Q.lc[1] = c.y; Q.lc[2] = c.z; Q.lc[3] = c.w;
         Q.ld[0] = d.x; Q.ld[1] = d.y; Q.ld[2] = d.z; Q.ld[3] = d.w;
         return;
@@ -97,9 +112,9 @@ __device__ __forceinline__ void load_local(const FusedStage& S, Quad& Q)
     for (int k = 0; k < 4; ++k) {
         Q.lc[k] = 0u;
         Q.ld[k] = kBgDepth;
-        if (k >= Q.lo && k < Q.hi && in_y && Q.fx + k >= S.r0x && Q.fx + k < S.r1x) {
-            Q.lc[k] = __ldcs(S.lc + le + k);
-            Q.ld[k] = __ldcs(reinterpret_cast<const uint32_t*>(S.ld) + le + k);
+        if (k >= Q.lo && k < Q.hi && in_y && Q.x + k >= g.rx0 && Q.x + k < g.rx1) {
+            Q.lc[k] = __ldcs(g.lc + le + k);
+            Q.ld[k] = __ldcs(g.ld + le + k);
         }
     }
 }
@@ -114,29 +129,32 @@ struct Segs {
 };
 
 template <bool CODED>
-__device__ __forceinline__ void finish(const FusedStage& S, const Quad& Q, int q0, const uint8_t (*planes)[kChunk],
-                                       bool csw, bool dsw, const Segs* G = nullptr)
+__device__ __forceinline__ void finish(const Grid& g, const Quad& Q, const uint8_t (*planes)[kChunk], bool csw, bool dsw,
+                                       const Segs* G = nullptr)
 {
     uint32_t oc[4], od[4];
     if (CODED && G) {
         // the segment of the quad's first element in the chunk, and the starts
-        // after it; most quads lie inside one segment
-        const int i0 = Q.qa - q0, a = max(i0, 0);
+        // after it (bit k: pixel k starts one); most quads lie inside one segment
+        const int i0 = g.e0 + Q.r * g.w + Q.x, a = max(i0, 0);
         const uint32_t u0 = G->U[a >> 5], u1 = G->U[min((a >> 5) + 1, kChunk / 32 - 1)];
-        const uint32_t s0 = G->PU[a >> 5] + __popc(u0 & ((2u << (a & 31)) - 1u)) - 1u;
-        const uint32_t nb = __funnelshift_r(u0, u1, a & 31);   // bit j: element a + j starts one
-        const uint2 first = G->S[s0];
+        const uint2* s0 = G->S + (G->PU[a >> 5] + __popc(u0 & ((2u << (a & 31)) - 1u)) - 1u);
+        const uint32_t nb = (__funnelshift_r(u0, u1, a & 31) & 0xEu) << (a - i0);
+        uint2 v[4];
+        v[0] = v[1] = v[2] = v[3] = *s0;
+        if (nb & 0xEu) {
+            v[1] = s0[__popc(nb & 0x2u)];
+            v[2] = s0[__popc(nb & 0x6u)];
+            v[3] = s0[__popc(nb & 0xEu)];
+        }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            uint2 v = first;
-            const int j = i0 + k - a;                          // (>= 0 for the quad's pixels in the unit)
-            if ((nb & 0xEu) && k >= Q.lo && k < Q.hi) v = G->S[s0 + __popc(nb & ((2u << j) - 2u))];
-            if (S.front) merge(v.x, v.y, Q.lc[k], Q.ld[k], oc[k], od[k]);
-            else merge(Q.lc[k], Q.ld[k], v.x, v.y, oc[k], od[k]);
+            if (g.front) over(v[k].x, v[k].y, Q.lc[k], Q.ld[k], oc[k], od[k]);   // (cleared when the segment was made)
+            else merge(Q.lc[k], Q.ld[k], v[k].x, v[k].y, oc[k], od[k]);
         }
     } else if (CODED) {
-        // bytes of elements qa - q0 .. +3 of every plane: two words and a funnel shift
-        const int i0 = Q.qa - q0;
+        // bytes of elements i0 .. i0 + 3 of every plane: two words and a funnel shift
+        const int i0 = g.e0 + Q.r * g.w + Q.x;
         const int wi = i0 >> 2, sh = 8 * (i0 & 3);
         const int w0 = max(wi, 0), w1 = min(wi + 1, kChunk / 4 - 1);
         uint32_t pb[8];
@@ -152,7 +170,7 @@ __device__ __forceinline__ void finish(const FusedStage& S, const Quad& Q, int q
         for (int k = 0; k < 4; ++k) {
             if (csw) ic[k] = rlec::swizzle(ic[k]);
             if (dsw) id[k] = rlec::swizzle(id[k]);
-            if (S.front) merge(ic[k], id[k], Q.lc[k], Q.ld[k], oc[k], od[k]);
+            if (g.front) merge(ic[k], id[k], Q.lc[k], Q.ld[k], oc[k], od[k]);
             else merge(Q.lc[k], Q.ld[k], ic[k], id[k], oc[k], od[k]);
         }
     } else {
@@ -163,53 +181,88 @@ __device__ __forceinline__ void finish(const FusedStage& S, const Quad& Q, int q
             od[k] = keep ? Q.ld[k] : kBgDepth;
         }
     }
-    const size_t oe = (size_t)(Q.fy - S.oy) * S.opitch + (Q.fx - S.ox);
-    if (Q.lo == 0 && Q.hi == 4 && S.ovec) {
-        st_stream(reinterpret_cast<uint4*>(S.oc + oe), make_uint4(oc[0], oc[1], oc[2], oc[3]));
-        st_stream(reinterpret_cast<uint4*>(S.od + oe), make_uint4(od[0], od[1], od[2], od[3]));
+    const int64_t oe = (int64_t)Q.r * g.opitch + Q.x;
+    if (Q.lo == 0 && Q.hi == 4 && g.ovec) {
+        st_stream(reinterpret_cast<uint4*>(g.oc + oe), make_uint4(oc[0], oc[1], oc[2], oc[3]));
+        st_stream(reinterpret_cast<uint4*>(g.od + oe), make_uint4(od[0], od[1], od[2], od[3]));
     } else {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             if (k >= Q.lo && k < Q.hi) {
-                S.oc[oe + k] = oc[k];
-                reinterpret_cast<uint32_t*>(S.od)[oe + k] = od[k];
+                g.oc[oe + k] = oc[k];
+                g.od[oe + k] = od[k];
             }
     }
 }
 
-__device__ __forceinline__ Grid grid_of(const FusedStage& S, const FusedUnit& u, int nrows)
-{
-    Grid g;
-    g.qx0 = u.x - ((u.x - S.ox) & 3);
-    g.nq = (u.x + u.w - g.qx0 + 3) >> 2;
-    g.slots = nrows * g.nq;
-    g.inv = 1.0f / (float)g.nq;
-    return g;
-}
-
-// Two quads per thread at a time: both local loads are in flight together.
+// The unit's quads in row order, from the one of its first element to the one of
+// its last: thread t takes the t-th of every kFT, two at a time, so that both
+// local loads are in flight together.  The step from one quad to the next is the
+// same for all of a thread's quads but for a wrap into the next row.
 template <bool CODED>
 __device__ __forceinline__ void compose(const FusedStage& S, const FusedUnit& u, int ra, int nrows,
                                         int q0, int len, const uint8_t (*planes)[kChunk], bool csw, bool dsw,
                                         const Segs* G = nullptr)
 {
-    const Grid g = grid_of(S, u, nrows);
-    for (int s = threadIdx.x; s < g.slots; s += 2 * kFT) {
-        Quad A, B;
-        const bool a = quad_at<CODED>(u, g, s, ra, q0, len, A);
-        const bool b = s + kFT < g.slots && quad_at<CODED>(u, g, s + kFT, ra, q0, len, B);
-        if (a) load_local(S, A);
-        if (b) load_local(S, B);
-        if (a) finish<CODED>(S, A, q0, planes, csw, dsw, G);
-        if (b) finish<CODED>(S, B, q0, planes, csw, dsw, G);
+    const int head = (u.x - S.ox) & 3;                        // pixels of a row's first quad before the unit
+    const int nq = (u.w + head + 3) >> 2;                     // quads of a row
+    Grid g;
+    const int64_t lo = (int64_t)(u.y + ra - S.ly) * S.lpitch + (u.x - S.lx);
+    const int64_t oo = (int64_t)(u.y + ra - S.oy) * S.opitch + (u.x - S.ox);
+    g.lc = S.lc + lo;
+    g.ld = reinterpret_cast<const uint32_t*>(S.ld) + lo;
+    g.oc = S.oc + oo;
+    g.od = reinterpret_cast<uint32_t*>(S.od) + oo;
+    g.lpitch = S.lpitch;
+    g.opitch = S.opitch;
+    g.rx0 = S.r0x - u.x;
+    g.rx1 = S.r1x - u.x;
+    g.ry0 = S.r0y - u.y - ra;
+    g.ry1 = S.r1y - u.y - ra;
+    g.w = u.w;
+    g.e0 = CODED ? ra * u.w - q0 : 0;
+    g.e1 = len;
+    g.lvec = S.lvec && ((u.x - head - S.lx) & 3) == 0;
+    g.ovec = S.ovec;
+    g.front = S.front;
+    const int s0 = CODED ? (head - g.e0) >> 2 : 0;
+    const int s1 = CODED ? (nrows - 1) * nq + ((head + len - 1 - g.e0 - (nrows - 1) * u.w) >> 2) + 1 : nrows * nq;
+    const int dr = kFT / nq, dx = 4 * (kFT - dr * nq);
+    const int s = s0 + (int)threadIdx.x, r = s / nq;
+    Quad A, B;
+    B.r = r;
+    B.x = 4 * (s - r * nq) - head;
+    const int end = 4 * nq - head;
+    auto step = [&](const Quad& from, Quad& to) {
+        to.r = from.r + dr;
+        to.x = from.x + dx;
+        if (to.x >= end) { to.x -= 4 * nq; ++to.r; }
+    };
+    for (int left = s1 - s; left > 0; left -= 2 * kFT) {
+        A.r = B.r;
+        A.x = B.x;
+        step(A, B);
+        const bool a = bounds<CODED>(g, A), b = left > kFT && bounds<CODED>(g, B);
+        if (a) load_local(g, A);
+        if (b) load_local(g, B);
+        if (a) finish<CODED>(g, A, planes, csw, dsw, G);
+        if (b) finish<CODED>(g, B, planes, csw, dsw, G);
+        step(B, B);
     }
 }
 
-__global__ void __launch_bounds__(kFT, 5)
+// Bound by instruction issue, and in small launches by the chain from a unit's
+// header to its last pixel.  The four fused launches of a binary swap of 16
+// 1920x1080 sources (about 1100 x 1000 pixels each, 30 % covered) take 104 us;
+// with rows walked quad by quad with a division each, every warp checking the
+// headers and 41 KB of shared memory they took 123 us.  Four CTAs per SM: six
+// (40 registers) took 114 us, five (48) 105 us.
+__global__ void __launch_bounds__(kFT, 4)
 k_fused_depth(const FusedStage* __restrict__ stages, const FusedUnit* __restrict__ units, uint32_t* status)
 {
+    // the decoded planes; before them, the run path's tables and staged streams
     __shared__ __align__(16) uint8_t planes[8][kChunk];
-    __shared__ __align__(16) uint32_t staged[2][kStageWords];
+    uint32_t (*staged)[kStageWords] = reinterpret_cast<uint32_t (*)[kStageWords]>(&planes[0][0] + kRunArea);
     __shared__ uint32_t s_beg[2][5];
     __shared__ int s_mode[2];
     __shared__ int s_fail, s_over;
@@ -234,17 +287,19 @@ k_fused_depth(const FusedStage* __restrict__ stages, const FusedUnit* __restrict
     const uint64_t csz = *u.csize, dsz = *u.dsize;
     // the run bitmaps (aliased with the planes) start empty
     uint32_t* bm = reinterpret_cast<uint32_t*>(&planes[0][0]);       // [8][128] run starts per plane
-    for (int i = tid; i < 8 * 128; i += kFT) bm[i] = 0u;
-    // warps 0-3 check the colour stream, 4-7 the depth stream
-    const rlec::ChunkEnds E = warp < 4
-        ? rlec::check_chunk(u.cs, u.cap, csz, (uint32_t)u.w, (uint32_t)u.h, nc, u.chunk, false)
-        : rlec::check_chunk(u.ds, u.cap, dsz, (uint32_t)u.w, (uint32_t)u.h, nc, u.chunk, false);
+    reinterpret_cast<uint4*>(bm)[tid] = make_uint4(0u, 0u, 0u, 0u);
+    // a warp checks the colour stream, another the depth stream
+    bool bad = false;
     if ((warp & 3) == 0) {
+        const rlec::ChunkEnds E = warp == 0
+            ? rlec::check_chunk(u.cs, u.cap, csz, (uint32_t)u.w, (uint32_t)u.h, nc, u.chunk, false)
+            : rlec::check_chunk(u.ds, u.cap, dsz, (uint32_t)u.w, (uint32_t)u.h, nc, u.chunk, false);
         if (lane >= 8 && lane < 13) s_beg[warp >> 2][lane - 8] = E.v;
         if (lane == 0) s_mode[warp >> 2] = E.mode;
+        bad = E.bad;
     }
     if (tid == 0) { s_fail = 0; s_over = 0; }
-    if (__syncthreads_or(E.bad)) {
+    if (__syncthreads_or(bad)) {
         if (tid == 0) set_status(status, EC_ERR_CORRUPT);
         return;
     }
@@ -255,10 +310,12 @@ k_fused_depth(const FusedStage* __restrict__ stages, const FusedUnit* __restrict
     const uint8_t* dpay = u.ds + 32 + 16ull * nc;
     const int cw0 = (int)(s_beg[0][0] >> 2), cnw = (int)((s_beg[0][4] + 3u) >> 2) - cw0;
     const int dw0 = (int)(s_beg[1][0] >> 2), dnw = (int)((s_beg[1][4] + 3u) >> 2) - dw0;
-    if (cnw <= kStageWords)
-        for (int i = tid; i < cnw; i += kFT) staged[0][i] = __ldg(reinterpret_cast<const uint32_t*>(cpay) + cw0 + i);
-    if (dnw <= kStageWords)
-        for (int i = tid; i < dnw; i += kFT) staged[1][i] = __ldg(reinterpret_cast<const uint32_t*>(dpay) + dw0 + i);
+    {
+        const int k = warp >> 2, w0 = k ? dw0 : cw0, nw = k ? dnw : cnw;
+        const uint32_t* from = reinterpret_cast<const uint32_t*>(k ? dpay : cpay) + w0;
+        if (nw <= kStageWords)
+            for (int i = tid & 127; i < nw; i += 128) staged[k][i] = __ldg(from + i);
+    }
     __syncthreads();
     // run path: warp k*4+p walks stream k's plane p, recording its runs
     uint8_t* const base8 = &planes[0][0];
@@ -322,7 +379,10 @@ k_fused_depth(const FusedStage* __restrict__ stages, const FusedUnit* __restrict
                     d |= (uint32_t)val[256 * (4 + q) + rd] << (8 * q);
                 }
                 const uint32_t sidx = eu + __popc(un & (le >> 1));
-                SS[sidx] = make_uint2(csw ? rlec::swizzle(c) : c, dsw ? rlec::swizzle(d) : d);
+                if (csw) c = rlec::swizzle(c);
+                if (dsw) d = rlec::swizzle(d);
+                if (S.front) clear_far(c, d);
+                SS[sidx] = make_uint2(c, d);
             }
         }
         __syncthreads();
