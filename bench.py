@@ -273,7 +273,7 @@ class DepthPipeline:
             ev[3].record()
 
     def launches_per_step(self):
-        return 7                             # compress: five kernels; decompress; merge
+        return 6                             # compress: four kernels; decompress; merge
 
     def compressed_bytes(self):
         return sum(int(s.item()) for s in self.sizes)
@@ -442,7 +442,7 @@ class CodecPipeline:
             ev[k + 1].record()
 
     def launches_per_step(self):
-        return 9 if self.yuv else 7          # compress: five kernels
+        return 8                             # compress: four kernels (and YUV's two), in mode 0 six; decompress; merge
 
     def compressed_bytes(self):
         return sum(int(s.item()) for s in self.sizes)
@@ -824,7 +824,7 @@ class Schedules:
         self.sch.run()
 
     def launches_per_step(self):
-        return len(self.launch_list)
+        return sum(4 if kind == "rle_compress" else 1 for kind in self.kind_of)    # compress: four kernels
 
     def compressed_bytes(self):
         if self.variant == "raw":
@@ -890,7 +890,7 @@ class Schedules:
 class BatchedTiles:
     """cfg4: 1000 uneven tiles (w, h log-uniform in [16, 1024], 2..64 layers, half
     depth RGBA8+Z32 at 30% box coverage, half alpha FP32 with a <= 0.3), all in
-    one persistent graph-captured launch (autotuned tile shapes)."""
+    a graph of persistent launches, one per kind of work item (autotuned tile shapes)."""
 
     def __init__(self, device, n_tiles=1000):
         import ctypes as C
@@ -901,8 +901,8 @@ class BatchedTiles:
         import synthetic as S
         self.ec = ec
         self.desc = (f"{n_tiles} tiles, w,h log-uniform [16,1024], layers U{{2..64}}, half depth "
-                     f"RGBA8+Z32 (30% coverage), half alpha FP32 (a<=0.3); one persistent "
-                     f"graph-captured launch vs one launch per tile")
+                     f"RGBA8+Z32 (30% coverage), half alpha FP32 (a<=0.3); a graph of persistent "
+                     f"launches, one per kind of work item, vs one launch per tile")
         self.tiles = S.uneven_tiles(4, n_tiles, device=device)
         self.units = sum(t.w * t.h * t.L for t in self.tiles)
         self.bytes = sum(t.w * t.h * (t.L * (8 if t.mode == "depth" else 16) + (8 if t.mode == "depth" else 16))
@@ -1251,7 +1251,7 @@ def depth_secondary(name, device, flush, peak, steps=50, warmup=5):
 
 
 def batched_extra(device, flush, peak, reps=20):
-    """The 1000 uneven tiles: one persistent graph-captured launch against one
+    """The 1000 uneven tiles: a graph of persistent launches against one
     plain launch per tile (median times)."""
     wl = BatchedTiles(device)
     wl.step()

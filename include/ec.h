@@ -546,7 +546,7 @@ ec_status ec_yuv_decode_batch(ec_ctx* ctx, const ec_yuv_job* jobs, int32_t njobs
  * refused with EC_ERR_UNSUPPORTED.  The first call on a device looks up the
  * array's device address with that device current; make that first call
  * before any stream capture.  All calls share the one array and it keeps the
- * last call's contents (each call clears what it needs with a memset on s), so
+ * last call's contents (each call clears what it needs on s), so
  * calls that overlap on the GPU -- on different streams or from several host
  * threads -- race; serialise them.
  *
@@ -556,7 +556,7 @@ ec_status ec_yuv_decode_batch(ec_ctx* ctx, const ec_yuv_job* jobs, int32_t njobs
  * up), since there is no context status word.  The stream written is byte for
  * byte the one ec_rle_compress writes. */
 #define EC_RLE_NOALLOC_MAX_CHUNKS 8192
-#define EC_RLE_NOALLOC_SCRATCH_BYTES (16 + 532 * EC_RLE_NOALLOC_MAX_CHUNKS)
+#define EC_RLE_NOALLOC_SCRATCH_BYTES (256 + 537 * EC_RLE_NOALLOC_MAX_CHUNKS)
 ec_status ec_rle_compress_noalloc(const void* src, int32_t w, int32_t h, int32_t pitch,
                                   uint32_t mode, void* dst, size_t dst_capacity,
                                   uint64_t* d_size, uint32_t* d_status, ec_stream_t s);

@@ -25,8 +25,11 @@
 
 namespace {
 
-constexpr size_t kScratchBytes = 16 + (16 + 4 + ec::kRlePoolPerUnit) * EC_RLE_NOALLOC_MAX_CHUNKS;
-static_assert(kScratchBytes == EC_RLE_NOALLOC_SCRATCH_BYTES, "documented scratch size");
+// counters; a record, two list entries and the pool's slot per chunk; a sum per
+// 32 chunks; the pool's alignment
+constexpr size_t kScratchBytes = EC_RLE_NOALLOC_SCRATCH_BYTES;
+static_assert(kScratchBytes >= 16 + (16 + 8 + ec::kRlePoolPerUnit) * EC_RLE_NOALLOC_MAX_CHUNKS +
+                                   4 * (EC_RLE_NOALLOC_MAX_CHUNKS / 32) + 127, "every chunk of the largest image has a slot");
 
 // Counters, chunk records and pool shared by every call of the entry point.
 static __device__ __align__(256) unsigned char g_rle_scratch[kScratchBytes];
