@@ -186,9 +186,11 @@ __device__ __forceinline__ int warp_incl_sum(int v, int lane)
 // from stream to plane position comes from the lane of the last token start),
 // and a window inside one literal token is copied without any parsing.
 //
-// (Windows of 32 bytes, each with a dependent load and five levels of shuffles,
-// and a loop per literal token: the decoder launch over 8 shaded 1920x1080
-// sources, RGBA8 + depth, took 265 us; this: 131 us.)
+// Bound by instruction issue (21 K warp instructions per chunk, 67 % of the issue
+// slots: the planes of a chunk are of uneven length, and its warps wait for the
+// longest).  Windows of 32 bytes, each with a dependent load and five levels of
+// shuffles, and a loop per literal token: the decoder launch over 8 shaded
+// 1920x1080 sources, RGBA8 + depth, took 265 us; this: 127 us.
 struct GlobalWords {      // payload bytes; reads stay below `end`
     const uint8_t* __restrict__ p;
     __device__ __forceinline__ uint32_t operator()(int off, int end) const
@@ -228,22 +230,22 @@ __device__ __forceinline__ int decode_plane_dense(const Words& words, int beg, i
             uint32_t nx = __shfl_down_sync(0xffffffffu, pair, 1);
             const uint32_t wn = __shfl_sync(0xffffffffu, odd ? L1 : L0, odd ? 0 : 16);   // the next window's first
             if (lane == 31) nx = wn;
-            const uint32_t R0 = __ballot_sync(0xffffffffu, b0 >= 128u), R1 = __ballot_sync(0xffffffffu, b1 >= 128u);
+            // lanes whose first / second byte would be a literal control (bytes past lim read as 0)
+            const uint32_t N0 = __ballot_sync(0xffffffffu, b0 < 128u), N1 = __ballot_sync(0xffffffffu, b1 < 128u);
             uint32_t T0 = 0u, T1 = 0u;                // lanes whose first / second byte starts a token
-            while (p < lim) {
-                const int l = p >> 1;
+            while (p < lim) {                         // repeats in a row and the literal (if any) behind them
                 const bool s = p & 1;
-                const uint32_t r = ~((s ? R1 : R0) >> l);
-                const int m = r ? __ffs(r) - 1 : 32;  // repeats in a row (none past lim: those bytes read as 0)
-                const uint32_t reps = (m == 32 ? 0xFFFFFFFFu : (1u << m) - 1u) << l;
-                p += 2 * m;
-                uint32_t lit = 0u;
-                if (p < lim) {
-                    lit = 1u << (p >> 1);
-                    p += 2 + (int)__shfl_sync(0xffffffffu, s ? b1 : b0, p >> 1);
-                }
-                if (s) T1 |= reps | lit;
-                else T0 |= reps | lit;
+                const uint32_t from = 0xFFFFFFFFu << (p >> 1), t = (s ? N1 : N0) & from, low = t & (0u - t);
+                const uint32_t starts = (2u * low - 1u) & from;
+                if (s) T1 |= starts;
+                else T0 |= starts;
+                const int k = low ? 31 - __clz(low) : 32;
+                p = 2 * k + (s ? 1 : 0);
+                if (p < lim) p += 2 + (int)__shfl_sync(0xffffffffu, s ? b1 : b0, k);
+            }
+            if (lim < 64) {                           // the stream's last bytes: no token starts past them
+                T0 &= 0xFFFFFFFFu >> (31 - ((lim - 1) >> 1));
+                T1 &= (1u << (lim >> 1)) - 1u;
             }
             const bool st0 = (T0 >> lane) & 1u, st1 = (T1 >> lane) & 1u, has = st0 || st1;
             const uint32_t ctl = st1 ? b1 : b0;
