@@ -949,7 +949,7 @@ class BatchedTiles:
             fn(*args, s)
 
     def launches_per_step(self):
-        return 1
+        return 3                             # alpha FP32, depth with and without 16-byte aligned rows
 
     def algorithmic_bytes(self):
         return {"batch": self.bytes}

@@ -342,12 +342,12 @@ __device__ void issue_quarter(const RleJobDesc& jb, uint32_t unit, int qi, int s
 // kernel.
 //
 // Bound by instruction issue up to a few thousand chunks per launch, by HBM and
-// issue alike beyond (2280 warp instructions per chunk, issue 68% active, DRAM
-// 74%).  16 flat sources, colour and depth: 1920x1080 54 -> 34.5 us, 7680x4320
-// (1.87 GB) 357 -> 322 us, against persistent warps that each streamed a chunk
+// issue alike beyond (2110 warp instructions per chunk, issue 65% active, DRAM
+// 75%).  16 flat sources, colour and depth: 1920x1080 54 -> 34.5 us, 7680x4320
+// (1.87 GB) 357 -> 314 us, against persistent warps that each streamed a chunk
 // through two 2 KB buffers (2930 instructions per chunk, and a chunk's whole
 // latency on one warp: the pieces of a binary-swap stage took 34 us whatever
-// their number, 18 here).  Holding the chunk in registers (eight 16-byte groups
+// their number, 10 to 24 here).  Holding the chunk in registers (eight 16-byte groups
 // per lane, eight CTAs per SM) took 3220 instructions per chunk and 465 us.
 constexpr int kCT = 128;
 
@@ -727,7 +727,7 @@ __device__ __forceinline__ uint32_t bit_range(int lo, int hi)
 // so the lanes of a warp stay together whatever their tokens.  xw: 16 P4 of
 // shared memory.  The caller synchronises before it reads the stage.
 // Bound by instruction issue: the dense chunks of 8 shaded 1920x1080 sources
-// (colour and depth, 68 MB) take 99 us, and 12 us to be copied to their place;
+// (colour and depth, 68 MB) take 95 us, and 16 us to be placed;
 // sizing them (45 us) and coding them again to their place with scattered
 // byte stores (134 us) came before.
 __device__ __forceinline__ void dense_chunk(const RleJobDesc& jb, uint32_t q0, int len, bool sw, uint32_t* T,
