@@ -41,3 +41,31 @@ def test_places_match_the_oracle(counts):
         want = oracle.rle_compress(a, m)
         assert int(size.item()) == len(want)
         assert dst[: len(want)].cpu().numpy().tobytes() == want
+
+
+@pytest.mark.parametrize("mode", [1, 2])
+@pytest.mark.parametrize("m", [33, 64, 97, 128])
+@pytest.mark.parametrize("w,h", [(CHUNK, 2), (1001, 9)])
+def test_chunks_of_many_runs_without_short_ones(m, w, h, mode):
+    """Chunks of 33 to 128 change points (the list's whole range above the
+    few-run case) whose runs all have three or more elements, so every plane is
+    repeat tokens only: runs of 3, of whole tokens, of one more, and long ones."""
+    require_gpu()
+    r = np.random.default_rng([m, w, mode])
+    n = w * h
+    flat = np.zeros(n, np.uint32)
+    for c0 in range(0, n, CHUNK):
+        left = min(CHUNK, n - c0)
+        k = min(m, left // 3)
+        L = np.full(k, 3)
+        for j, want in zip(r.permutation(k), [125, 126, 253, 0, 1, 254, 60]):     # 128, 129, 256, 3, 4, 257, 63
+            if L.sum() + want <= left:
+                L[j] += want
+        L[int(r.integers(0, k))] += left - L.sum()
+        e = r.integers(0, 1 << 32, size=k, dtype=np.uint64).astype(np.uint32)
+        flat[c0:c0 + left] = np.repeat(e, L)
+    img = flat.reshape(h, w)
+    want = oracle.rle_compress(img, mode)
+    buf, size = ec.rle_compress(torch.from_numpy(img.view(np.int32)).cuda().view(torch.uint32), mode)
+    ec.default_context().check_status()
+    assert buf[: int(size.item())].cpu().numpy().tobytes() == want
