@@ -343,13 +343,22 @@ __device__ void issue_quarter(const RleJobDesc& jb, uint32_t unit, int qi, int s
 //
 // Bound by instruction issue up to a few thousand chunks per launch, by HBM and
 // issue alike beyond (2110 warp instructions per chunk, issue 65% active, DRAM
-// 75%).  16 flat sources, colour and depth: 1920x1080 54 -> 33.8 us, 7680x4320
-// (1.87 GB) 357 -> 313 us, against persistent warps that each streamed a chunk
+// 75%).  16 flat sources, colour and depth: 1920x1080 54 -> 33.4 us, 7680x4320
+// (1.87 GB) 357 -> 307 us, against persistent warps that each streamed a chunk
 // through two 2 KB buffers (2930 instructions per chunk, and a chunk's whole
 // latency on one warp: the pieces of a binary-swap stage took 34 us whatever
 // their number, 10 to 24 here).  Holding the chunk in registers (eight 16-byte groups
 // per lane, eight CTAs per SM) took 3220 instructions per chunk and 465 us.
 constexpr int kCT = 128;
+
+// Bytes that a plane of at most kCap runs codes to: r repeat runs to 2 r +
+// kChunk / 64 (2 ceil(L / 128) <= 2 + L / 64 for a run of L), k short ones, of
+// at most two bytes, in s literal spans to 2 k + s + k / 64.  A repeat run lies
+// between two spans, so s <= kCap / 2.  (With the tables, 18.3 KB per CTA: twelve
+// fit on an SM.  With 3 kCap + kChunk / 64 eleven did: 313 -> 307 us for 16 flat
+// 7680x4320 sources.)
+constexpr int kStagePlane4 = 2 * kCap + kCap / 2 + kCap / 64 + kChunk / 64 + 6;
+static_assert(kStagePlane4 % 8 == 0, "planes' stages are aligned");
 
 // Plane stream of a chunk of len elements from its m <= 32 change points, run
 // by run, where every run is at least 3 bytes (so all of it is repeat tokens).
@@ -388,7 +397,7 @@ __device__ __forceinline__ uint32_t code_plane_few(bool valid, uint32_t v, int q
 // of those of flat-shaded sources) needs no spans, and its tokens are whole
 // 16-bit stores (out is even): a binary swap of 16 1920x1080 sources 199.5 us
 // without that path, 197.0 with it.  Returns the bytes written (at most
-// kStagePlane).
+// kStagePlane4).
 __device__ __forceinline__ uint32_t code_plane_many(const uint32_t* el, const uint16_t* cq, int m, int shift, bool sw,
                                                     int len, uint8_t* out)
 {
@@ -520,7 +529,7 @@ __global__ void __launch_bounds__(kCT, 12)
 k_rle_code(const __grid_constant__ RleJobList<N> J, const RleScratch W, uint32_t* status)
 {
     __shared__ __align__(16) uint32_t raw[4 + kChunk];      // the chunk, after a guard
-    __shared__ __align__(16) uint8_t stage[4][kStagePlane];
+    __shared__ __align__(16) uint8_t stage[4][kStagePlane4];
     __shared__ uint16_t cq[kCap];                            // the change points' positions
     __shared__ uint64_t full;
     __shared__ uint32_t s_cnt[4], s_T[4], s_po;
