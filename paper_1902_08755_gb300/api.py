@@ -158,8 +158,9 @@ def _target(color: torch.Tensor, depth: Optional[torch.Tensor], pvp, dev: int) -
     dptr = None
     if depth is not None:
         _on_device(depth, dev, "output depth")
-        if depth.dtype != torch.float32 or depth.stride(0) != pitch or depth.stride(1) != 1:
-            raise ValueError("output depth must be float32 with the colour's pitch")
+        if depth.dtype != torch.float32 or depth.dim() != 2 or depth.stride(1) != 1 or depth.stride(0) != pitch \
+                or depth.shape[0] < pvp[3] or depth.shape[1] < pvp[2]:
+            raise ValueError("output depth must be float32 [h][pitch] with the colour's pitch")
         dptr = depth.data_ptr()
     return ec_target(_rect(pvp), pitch, fmt, color.data_ptr(), dptr)
 

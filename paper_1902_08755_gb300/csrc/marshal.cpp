@@ -206,7 +206,7 @@ PyObject* target(PyObject*, PyObject* args)
         out->color = t->data_ptr();
         out->depth = nullptr;
         if (depth != Py_None) {
-            const at::Tensor* d = depth_of(depth, dev, l, 0, 0);
+            const at::Tensor* d = depth_of(depth, dev, l, out->pvp.w, out->pvp.h);
             if (!d) Py_RETURN_FALSE;
             out->depth = static_cast<float*>(d->data_ptr());
         }
