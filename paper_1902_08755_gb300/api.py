@@ -361,7 +361,10 @@ def composite_depth_backward(winner: torch.Tensor, out_pvp: Rect, grad_out: torc
         if gf != A.EC_RGBA32F or gpitch != pitch:
             raise ValueError("depth gradients are float32 [h][pitch][4] with the input's pitch")
         _on_device(g, dev, "gradient")
-        pvps.append(_rect(im.pvp if im.pvp is not None else (0, 0, w, h)))
+        pvp = _rect(im.pvp if im.pvp is not None else (0, 0, w, h))
+        if g.shape[0] < pvp.h or g.shape[1] < pvp.w:
+            raise ValueError("depth gradients cover their input's pvp")
+        pvps.append(pvp)
         pitches.append(pitch)
     rp = (ec_rect * max(1, n))(*pvps)
     pp = (C.c_int32 * max(1, n))(*pitches)
