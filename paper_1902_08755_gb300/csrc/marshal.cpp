@@ -33,6 +33,16 @@ struct Ref {
     Ref& operator=(const Ref&) = delete;
 };
 
+// Item i of a list or tuple (nullptr past its end), held: reading an attribute
+// may run Python code, which may take the item out of the list.
+PyObject* item_of(PyObject* seq, Py_ssize_t i)
+{
+    if (i >= PySequence_Fast_GET_SIZE(seq)) return nullptr;
+    PyObject* o = PySequence_Fast_GET_ITEM(seq, i);
+    Py_INCREF(o);
+    return o;
+}
+
 const at::Tensor* tensor_of(PyObject* o)
 {
     if (!o || !THPVariable_CheckExact(o)) return nullptr;
@@ -148,8 +158,8 @@ PyObject* images(PyObject*, PyObject* args)
         const Py_ssize_t n = PySequence_Fast_GET_SIZE(seq);
         Layout l;
         for (Py_ssize_t i = 0; i < n; ++i) {
-            if (i >= PySequence_Fast_GET_SIZE(seq)) Py_RETURN_FALSE;      // (an attribute's code changed the list)
-            if (!image_of(PySequence_Fast_GET_ITEM(seq, i), dev, need, &out[i], &l)) Py_RETURN_FALSE;
+            const Ref im(item_of(seq, i));
+            if (!im.p || !image_of(im.p, dev, need, &out[i], &l)) Py_RETURN_FALSE;
         }
         Py_RETURN_TRUE;
     });
@@ -172,9 +182,10 @@ PyObject* gradients(PyObject*, PyObject* args)
         if (n == 0 || n != PySequence_Fast_GET_SIZE(imgs)) Py_RETURN_FALSE;
         int fmt = -1;
         for (Py_ssize_t i = 0; i < n; ++i) {
-            if (i >= PySequence_Fast_GET_SIZE(seq) || i >= PySequence_Fast_GET_SIZE(imgs)) Py_RETURN_FALSE;
-            const at::Tensor* g = tensor_of(PySequence_Fast_GET_ITEM(seq, i));
-            const Ref color(PyObject_GetAttr(PySequence_Fast_GET_ITEM(imgs, i), s_color));
+            const Ref grad(item_of(seq, i)), im(item_of(imgs, i));
+            if (!grad.p || !im.p) Py_RETURN_FALSE;
+            const at::Tensor* g = tensor_of(grad.p);
+            const Ref color(PyObject_GetAttr(im.p, s_color));
             const at::Tensor* c = tensor_of(color.p);
             Layout lg, lc;
             if (!g || !c || !on_device(*g, dev) || !layout_of(*g, &lg) || !layout_of(*c, &lc)) Py_RETURN_FALSE;

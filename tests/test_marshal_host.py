@@ -1,5 +1,8 @@
 """Host checks of the binding's argument marshalling that need no GPU: what its
 Python path refuses."""
+import os
+import subprocess
+import sys
 import types
 
 import pytest
@@ -7,6 +10,8 @@ import torch
 
 import paper_1902_08755_gb300 as ec
 from paper_1902_08755_gb300 import api
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def _shapes(h, w, pitch):
@@ -80,3 +85,44 @@ def test_depth_gradients_cover_their_input(calls, pvp):
         with pytest.raises(ValueError):
             run(bad)
     assert len(calls) == 2
+
+
+_CHANGING_LISTS = r"""
+import ctypes as C, gc, sys
+import torch
+from paper_1902_08755_gb300 import _abi as A
+
+t = torch.zeros((4, 4), dtype=torch.int32)
+
+class Clears:                                   # reading one of its attributes empties the lists
+    def __init__(self, lists, attr):
+        self.lists, self.attr, self.load = lists, attr, [bytearray(4096) for _ in range(8)]
+    def __getattribute__(self, name):
+        get = object.__getattribute__
+        if name in ("color", "depth", "pvp", "roi"):
+            if name == get(self, "attr"):
+                for l in get(self, "lists"):
+                    l.clear()
+                gc.collect()
+                junk = [bytearray(64) for _ in range(4096)]
+            return t if name == "color" else None
+        return get(self, name)
+
+arr = (C.c_uint64 * 64)()
+for attr in ("color", "pvp", "roi"):
+    for _ in range(50):
+        images = []
+        images.append(Clears([images], attr))
+        assert A.marshal().images(images, 0, 0, C.addressof(arr)) is False and not images
+        images, grads = [], [torch.zeros((4, 4, 4))]
+        images.append(Clears([images, grads], "color"))
+        assert A.marshal().gradients(grads, images, 0, C.addressof(arr)) is False and not images and not grads
+print("fine")
+"""
+
+
+def test_attributes_may_change_the_lists():
+    """The images' attributes may be properties: code that takes the image (and
+    its gradient) out of the lists while they are read."""
+    r = subprocess.run([sys.executable, "-X", "dev", "-c", _CHANGING_LISTS], cwd=ROOT, capture_output=True, text=True)
+    assert r.returncode == 0 and r.stdout.strip() == "fine", (r.returncode, r.stdout, r.stderr[-2000:])
