@@ -122,7 +122,11 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t s
     c.attrs = at;
     c.numAttrs = 1;
     void* pargs[] = {const_cast<void*>(static_cast<const void*>(&args))...};
-    return cudaLaunchKernelExC(&c, reinterpret_cast<const void*>(kernel), pargs);
+    const cudaError_t e = cudaLaunchKernelExC(&c, reinterpret_cast<const void*>(kernel), pargs);
+    // a refused launch is reported here; the runtime's last error is not left
+    // set, where the next call that reads it would take it for its own
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
 }
 
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
