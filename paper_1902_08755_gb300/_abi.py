@@ -6,8 +6,10 @@ raises.  Struct layouts must match include/ec.h field for field.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 import threading
+import warnings
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 
@@ -167,12 +169,28 @@ def load(build_if_missing: bool = True):
         return _lib
 
 
+class _PythonChecks:
+    """In the place of the native marshalling where it cannot be loaded: takes no
+    arguments, so that the binding's own checks do."""
+
+    images = gradients = target = order = staticmethod(lambda *args: False)
+
+
 def marshal():
     """The native argument marshalling (csrc/marshal.cpp), built with libec.so."""
     global _marshal
     if _marshal is None:
         load()
-        from . import _marshal as m
+        from . import build as _build
+        try:
+            if _build.marshal_stale():
+                raise ImportError("not built from the current source for this Python and torch")
+            spec = importlib.util.spec_from_file_location(__package__ + "._marshal", _build.marshal_path())
+            m = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(m)
+        except ImportError as e:
+            warnings.warn(f"the native argument marshalling is not used (arguments are checked in Python): {e}")
+            m = _PythonChecks
         _marshal = m
     return _marshal
 
