@@ -107,17 +107,33 @@ ec_status cuda_status(cudaError_t e) { return e == cudaSuccess ? EC_OK : EC_ERR_
 
 uint32_t rle_units(uint64_t n) { return (uint32_t)std::max<uint64_t>(1, (n + EC_RLE_CHUNK - 1) / EC_RLE_CHUNK); }
 
-ec_status ensure_scratch(ec_ctx* ctx, size_t bytes)
+// Codec scratch for a compress launch of `units` chunks.  Growing it
+// synchronises with the device (cudaFree); contexts start with room for
+// kScratchUnits chunks (4 Mi elements).
+constexpr uint32_t kScratchUnits = 1024;
+
+ec_status ensure_scratch(ec_ctx* ctx, uint32_t units)
 {
-    if (ctx->scratch_bytes >= bytes) return EC_OK;
-    // growing synchronises with the device (cudaFree); contexts start with
-    // room for 65536 chunks (256 Mi elements), so this is rare
+    if (ctx->scratch_units >= units) return EC_OK;
     if (ctx->scratch) cudaFree(ctx->scratch);
     ctx->scratch = nullptr;
     ctx->scratch_bytes = 0;
-    if (cudaMalloc(&ctx->scratch, bytes) != cudaSuccess) return EC_ERR_CUDA;
-    ctx->scratch_bytes = bytes;
-    return EC_OK;
+    ctx->scratch_units = 0;
+    // on a device that is nearly full, the smaller pool: dense chunks are then
+    // coded a second time when placed
+    for (const size_t pool : {rle_pool_bytes(units), kRlePoolPerUnit * (size_t)units}) {
+        const size_t bytes = rle_compress_scratch_bytes(units, pool);
+        const cudaError_t e = cudaMalloc(&ctx->scratch, bytes);
+        if (e == cudaSuccess) {
+            ctx->scratch_bytes = bytes;
+            ctx->scratch_units = units;
+            return EC_OK;
+        }
+        ctx->scratch = nullptr;
+        (void)cudaGetLastError();
+        if (e != cudaErrorMemoryAllocation) break;
+    }
+    return EC_ERR_CUDA;
 }
 
 ec_status ensure_roi_scratch(ec_ctx* ctx, size_t bytes)
@@ -165,7 +181,7 @@ ec_status ec_create(ec_ctx** out, int device)
     cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, device);
     if (cudaMalloc(&ctx->d_status, sizeof(uint32_t)) != cudaSuccess ||
         cudaMemset(ctx->d_status, 0, sizeof(uint32_t)) != cudaSuccess ||
-        ensure_scratch(ctx, rle_compress_scratch_bytes(1024, rle_pool_bytes(1024))) != EC_OK) {
+        ensure_scratch(ctx, kScratchUnits) != EC_OK) {
         ec_destroy(ctx);
         return EC_ERR_CUDA;
     }
@@ -573,7 +589,7 @@ static ec_status rle_batch(ec_ctx* ctx, const ec_rle_job* jobs, int32_t njobs, b
         }
         cudaError_t e;
         if (compress) {
-            const ec_status st = ensure_scratch(ctx, rle_compress_scratch_bytes(units, rle_pool_bytes(units)));
+            const ec_status st = ensure_scratch(ctx, units);
             if (st != EC_OK) return st;
             e = launch_rle_compress(&d[b], cnt, units, ctx->scratch, ctx->scratch_bytes, ctx->d_status,
                                     (cudaStream_t)s);

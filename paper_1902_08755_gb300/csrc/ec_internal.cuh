@@ -35,6 +35,7 @@ struct ec_ctx {
     uint32_t* d_status = nullptr;   // first device-side error (0 = none)
     void* scratch = nullptr;        // codec scratch: counters, chunk records, pool
     size_t scratch_bytes = 0;
+    uint32_t scratch_units = 0;     // chunks of the largest launch that it is for
     void* roi_scratch = nullptr;    // ROI detection: per-image box accumulators + done counter
     size_t roi_scratch_bytes = 0;
     int sm_count = 0;
@@ -238,7 +239,8 @@ size_t rle_compress_scratch_bytes(uint32_t units, size_t pool_bytes);
 
 // The pool a launch is given: 512 bytes per unit, which few-run chunks stay
 // below on average, and 8 KB more per unit (half of a chunk's size) for chunks
-// of many tokens, up to 256 MB in all.
+// of many tokens, up to 256 MB in all.  Where the device has no room for that,
+// the 512 bytes alone.
 constexpr size_t kRlePoolPerUnit = 512;
 constexpr size_t kRleDensePoolPerUnit = 8192, kRleDensePoolMax = 256u << 20;
 inline size_t rle_pool_bytes(uint32_t units)

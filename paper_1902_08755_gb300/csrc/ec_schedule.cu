@@ -575,13 +575,29 @@ ec_status ec_schedule_plan(ec_ctx* ctx, int32_t mode, int32_t algorithm, const e
         lr.fun_off = A.take(std::max<size_t>(nu, 1) * sizeof(FusedUnit));
     }
     const uint32_t scratch_units = (uint32_t)std::max<uint64_t>(max_units, 1);
-    const size_t scratch_bytes = ec::rle_compress_scratch_bytes(scratch_units, ec::rle_pool_bytes(scratch_units));
+    // (the arena's last part: where the device has no room for the whole pool,
+    // the least one is tried)
+    const size_t least_pool = ec::kRlePoolPerUnit * (size_t)scratch_units;
+    const size_t more_pool = ec::rle_pool_bytes(scratch_units) - least_pool;
+    size_t scratch_bytes = ec::rle_compress_scratch_bytes(scratch_units, least_pool);
     const size_t scratch_off = A.take(scratch_bytes);
 
     DeviceGuard g(ctx->device);
     if (!g.ok) return fail(EC_ERR_CUDA);
-    S->arena_bytes = std::max<size_t>(A.top, 256);
-    if (cudaMalloc(&S->arena, S->arena_bytes) != cudaSuccess) return fail(EC_ERR_CUDA);
+    S->arena_bytes = std::max<size_t>(A.top + more_pool, 256);
+    cudaError_t me = cudaMalloc(&S->arena, S->arena_bytes);
+    if (me == cudaSuccess) {
+        scratch_bytes += more_pool;
+    } else {
+        (void)cudaGetLastError();
+        S->arena_bytes = std::max<size_t>(A.top, 256);
+        if (me == cudaErrorMemoryAllocation) me = cudaMalloc(&S->arena, S->arena_bytes);
+        if (me != cudaSuccess) {
+            S->arena = nullptr;
+            (void)cudaGetLastError();
+            return fail(EC_ERR_CUDA);
+        }
+    }
     char* base = S->arena;
     if (cudaStreamCreateWithFlags(&S->stream, cudaStreamNonBlocking) != cudaSuccess) return fail(EC_ERR_CUDA);
 
