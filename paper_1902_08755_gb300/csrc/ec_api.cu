@@ -917,18 +917,25 @@ float time_shape(ec_batch& b, const BatchShape& sh)
     return best;
 }
 
+// Key of a batch's tile shape in the tune cache: all that the choice of its
+// items' kernels and their cost follows from -- the kernels themselves (a stored
+// shape outlives the library that timed it), sizes, where the inputs lie (which
+// tiles they cover) and whether their rows are 16-byte groups.
+constexpr int64_t kTuneVersion = 2;     // to be raised with the batch kernels (1: one kernel for all kinds)
+
 std::string signature(const ec_batch& b, int device)
 {
     cudaDeviceProp prop{};
     cudaGetDeviceProperties(&prop, device);
     uint64_t h = 1469598103934665603ull;
     auto mix = [&](int64_t v) { h ^= (uint64_t)v; h *= 1099511628211ull; };
+    mix(kTuneVersion);
     mix(b.ctas_per_sm);
     for (const BatchJob& J : b.jobs) {
-        mix(J.mode); mix(J.n); mix(J.D.W); mix(J.D.H);
+        mix(J.mode); mix(J.n); mix(J.step); mix(J.D.W); mix(J.D.H);
         for (int i = 0; i < J.n; ++i) {
             const SrcDesc& s = b.srcs[J.first + i];
-            mix(s.x1 - s.x0); mix(s.y1 - s.y0);
+            mix(s.x0); mix(s.y0); mix(s.x1); mix(s.y1); mix(s.vec);
         }
     }
     char buf[64];
