@@ -47,9 +47,23 @@ template <> struct ColorT<16> { using T = float4; };
 __device__ __forceinline__ void zero(uint32_t& c) { c = 0u; }
 __device__ __forceinline__ void zero(float4& c) { c = make_float4(0.f, 0.f, 0.f, 0.f); }
 
+// An RGBA32F pixel a word at a time (WORDS: a colour buffer of the call does not
+// start at a multiple of 16 bytes, and a whole pixel's access would fault).
+__device__ __forceinline__ float4 load_words(const float4* p)
+{
+    const float* f = reinterpret_cast<const float*>(p);
+    return make_float4(__ldcs(f), __ldcs(f + 1), __ldcs(f + 2), __ldcs(f + 3));
+}
+
+__device__ __forceinline__ void store_words(float4* p, const float4& c)
+{
+    float* f = reinterpret_cast<float*>(p);
+    f[0] = c.x; f[1] = c.y; f[2] = c.z; f[3] = c.w;
+}
+
 // The pixels x + j STEP, j = 0..3, of one source: 16-byte loads (vec, STEP 1) or
 // per-pixel loads.
-template <int CB, int STEP>
+template <int CB, int STEP, bool WORDS>
 __device__ __forceinline__ void load4(const SrcDesc& s, int x, int y, float (&d)[4],
                                       typename ColorT<CB>::T (&c)[4])
 {
@@ -74,6 +88,7 @@ __device__ __forceinline__ void load4(const SrcDesc& s, int x, int y, float (&d)
             if (xj >= s.x0 && xj < s.x1) {
                 d[j] = __ldcs(dp + j * STEP);
                 if constexpr (CB == 4) c[j] = __ldcs(reinterpret_cast<const unsigned int*>(cp + j * STEP));
+                else if constexpr (WORDS) c[j] = load_words(cp + j * STEP);
                 else c[j] = __ldcs(cp + j * STEP);
             } else {
                 d[j] = 1.0f;
@@ -84,7 +99,7 @@ __device__ __forceinline__ void load4(const SrcDesc& s, int x, int y, float (&d)
 }
 
 // Write the merged pixels x + j STEP of row y: depth, colour, winner.
-template <int CB, int STEP>
+template <int CB, int STEP, bool WORDS = false>
 __device__ __forceinline__ void store_depth4(const DstDesc& D, int x, int y, const float (&bd)[4],
                                              const typename ColorT<CB>::T (&bc)[4], const int (&bi)[4])
 {
@@ -102,7 +117,8 @@ __device__ __forceinline__ void store_depth4(const DstDesc& D, int x, int y, con
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             if (x + j * STEP < D.W) {
-                oc[j * STEP] = bc[j];
+                if constexpr (CB == 16 && WORDS) store_words(oc + j * STEP, bc[j]);
+                else oc[j * STEP] = bc[j];
                 if (D.depth) D.depth[o + j * STEP] = bd[j];
             }
         }
@@ -121,7 +137,7 @@ __device__ __forceinline__ void store_depth4(const DstDesc& D, int x, int y, con
 // warp's lanes own adjacent pixels, for calls with inputs that must be read
 // pixel by pixel: every load of the warp then covers 128 contiguous bytes, where
 // adjacent pixels per lane would spread it over 512 (four times the sectors).
-template <int CB, int STEP, class At, int U = 4>
+template <int CB, int STEP, bool WORDS = false, class At, int U = 4>
 __device__ __forceinline__ void depth_px4(At at, const int16_t* act, int nact, int x, int y,
                                           const DstDesc& D)
 {
@@ -144,7 +160,7 @@ __device__ __forceinline__ void depth_px4(At at, const int16_t* act, int nact, i
             if (idx[u] >= 0) {
                 const SrcDesc& s = at(a + u, idx[u]);
                 live[u] = y >= s.y0 && y < s.y1 && x + 3 * STEP >= s.x0 && x < s.x1;
-                if (live[u]) load4<CB, STEP>(s, x, y, d[u], c[u]);
+                if (live[u]) load4<CB, STEP, WORDS>(s, x, y, d[u], c[u]);
             }
         }
 #pragma unroll
@@ -165,7 +181,7 @@ __device__ __forceinline__ void depth_px4(At at, const int16_t* act, int nact, i
         }
     }
 
-    store_depth4<CB, STEP>(D, x, y, bd, bc, bi);
+    store_depth4<CB, STEP, WORDS>(D, x, y, bd, bc, bi);
 }
 
 // ----------------------------------------------------------------- alpha ---

@@ -24,12 +24,17 @@ template <> struct Grp<4> { static constexpr int PX = 4; };
 template <> struct Grp<8> { static constexpr int PX = 2; };
 template <> struct Grp<16> { static constexpr int PX = 1; };
 
-// Pixel j of a 16-byte group as raw 32-bit words (BPP / 4 of them).
-template <int BPP>
+// Pixel j of a 16-byte group as raw 32-bit words (BPP / 4 of them).  WORDS: a
+// buffer of the call does not start at a multiple of its pixel size, so pixels
+// are read and written a word at a time (the kernels' other instances move whole
+// pixels, which such an address faults).
+template <int BPP, bool WORDS>
 __device__ __forceinline__ void load_px(const uint8_t* p, uint32_t* w)
 {
-    if constexpr (BPP == 4) w[0] = __ldcs(reinterpret_cast<const uint32_t*>(p));
-    else if constexpr (BPP == 8) {
+    if constexpr (BPP == 4 || WORDS) {
+#pragma unroll
+        for (int k = 0; k < BPP / 4; ++k) w[k] = __ldcs(reinterpret_cast<const uint32_t*>(p) + k);
+    } else if constexpr (BPP == 8) {
         const uint2 v = __ldcs(reinterpret_cast<const uint2*>(p));
         w[0] = v.x; w[1] = v.y;
     } else {
@@ -38,11 +43,13 @@ __device__ __forceinline__ void load_px(const uint8_t* p, uint32_t* w)
     }
 }
 
-template <int BPP>
+template <int BPP, bool WORDS>
 __device__ __forceinline__ void store_px(uint8_t* p, const uint32_t* w)
 {
-    if constexpr (BPP == 4) *reinterpret_cast<uint32_t*>(p) = w[0];
-    else if constexpr (BPP == 8) *reinterpret_cast<uint2*>(p) = make_uint2(w[0], w[1]);
+    if constexpr (BPP == 4 || WORDS) {
+#pragma unroll
+        for (int k = 0; k < BPP / 4; ++k) reinterpret_cast<uint32_t*>(p)[k] = w[k];
+    } else if constexpr (BPP == 8) *reinterpret_cast<uint2*>(p) = make_uint2(w[0], w[1]);
     else *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
@@ -73,7 +80,7 @@ struct TileMasks {
 // MASK: the sources come from the tile masks (n <= 64), else each CTA lists
 // them (build_active).  Every pixel walks them from last to first and stops
 // once its 16-byte group is complete.
-template <int N, int BPP, bool MASK>
+template <int N, int BPP, bool MASK, bool WORDS>
 __global__ void __launch_bounds__(kAT, 8)
 k_assemble_tiles(const __grid_constant__ SrcList<N> L, const __grid_constant__ DstDesc D,
                  const __grid_constant__ TileMasks M)
@@ -130,7 +137,7 @@ k_assemble_tiles(const __grid_constant__ SrcList<N> L, const __grid_constant__ D
             } else if ((fast >> pass) & 1u) {
                 uint32_t w[PX][WPP];
 #pragma unroll
-                for (int j = 0; j < PX; ++j) load_px<BPP>(fp[pass] + j * BPP, w[j]);
+                for (int j = 0; j < PX; ++j) load_px<BPP, WORDS>(fp[pass] + j * BPP, w[j]);
                 const uint32_t* f = &w[0][0];
                 v[pass] = make_uint4(f[0], f[1], f[2], f[3]);
             }
@@ -176,7 +183,7 @@ k_assemble_tiles(const __grid_constant__ SrcList<N> L, const __grid_constant__ D
         } else {
 #pragma unroll
             for (int j = 0; j < PX; ++j)
-                if ((m >> j) & 1u) load_px<BPP>(p + j * BPP, w[j]);
+                if ((m >> j) & 1u) load_px<BPP, WORDS>(p + j * BPP, w[j]);
         }
         have |= m;
     }
@@ -192,7 +199,7 @@ k_assemble_tiles(const __grid_constant__ SrcList<N> L, const __grid_constant__ D
     } else {
 #pragma unroll
         for (int j = 0; j < PX; ++j)
-            if ((have >> j) & 1u) store_px<BPP>(o + j * BPP, w[j]);
+            if ((have >> j) & 1u) store_px<BPP, WORDS>(o + j * BPP, w[j]);
     }
     }
 }
@@ -202,7 +209,7 @@ k_assemble_tiles(const __grid_constant__ SrcList<N> L, const __grid_constant__ D
 // FMT: 0 RGBA8 (integer sums, (sum + count/2) / count), 1 RGBA32F, 2 RGBA16F
 // (FP32 sums in input order, divided by the count).  Sources are read four
 // at a time, all four groups in flight before any is added.
-template <int N, int FMT>
+template <int N, int FMT, bool WORDS>
 __global__ void __launch_bounds__(kAT)
 k_average(const __grid_constant__ SrcList<N> L, const __grid_constant__ DstDesc D)
 {
@@ -271,7 +278,7 @@ k_average(const __grid_constant__ SrcList<N> L, const __grid_constant__ DstDesc 
                 } else {
 #pragma unroll
                     for (int j = 0; j < PX; ++j)
-                        if ((m[b] >> j) & 1u) load_px<BPP>(p + j * BPP, w[b][j]);
+                        if ((m[b] >> j) & 1u) load_px<BPP, WORDS>(p + j * BPP, w[b][j]);
                 }
             }
 #pragma unroll
@@ -341,14 +348,14 @@ k_average(const __grid_constant__ SrcList<N> L, const __grid_constant__ DstDesc 
         } else {
 #pragma unroll
             for (int j = 0; j < PX; ++j)
-                if (x + j < D.W) store_px<BPP>(o + j * BPP, out[j]);
+                if (x + j < D.W) store_px<BPP, WORDS>(o + j * BPP, out[j]);
         }
     }
 }
 
 // ---- pixel compound --------------------------------------------------------
 
-template <int N, int BPP>
+template <int N, int BPP, bool WORDS>
 __global__ void __launch_bounds__(kAT)
 k_assemble_pixels(const __grid_constant__ PixList<N> P, const __grid_constant__ DstDesc D)
 {
@@ -375,7 +382,7 @@ k_assemble_pixels(const __grid_constant__ PixList<N> P, const __grid_constant__ 
             if (k >= 0) {
                 const PixSrc& s = P.s[k];
                 const size_t e = (size_t)j0 * (size_t)s.pitch + (size_t)i0;
-                load_px<BPP>(reinterpret_cast<const uint8_t*>(s.color) + e * BPP, w[pass][j]);
+                load_px<BPP, WORDS>(reinterpret_cast<const uint8_t*>(s.color) + e * BPP, w[pass][j]);
                 have[pass] |= 1u << j;
             }
             if (++rx == P.nx) { rx = 0; ++i0; }
@@ -396,7 +403,7 @@ k_assemble_pixels(const __grid_constant__ PixList<N> P, const __grid_constant__ 
         } else {
 #pragma unroll
             for (int j = 0; j < PX; ++j)
-                if ((have[pass] >> j) & 1u) store_px<BPP>(o + j * BPP, w[pass][j]);
+                if ((have[pass] >> j) & 1u) store_px<BPP, WORDS>(o + j * BPP, w[pass][j]);
         }
     }
 }
@@ -414,9 +421,27 @@ SrcList<N> make_src_list(const SrcDesc* src, int n)
 template <int N, bool MASK>
 cudaError_t tiles_bpp(const SrcList<N>& L, int bpp, const DstDesc& D, const TileMasks& M, dim3 grid, cudaStream_t s)
 {
-    if (bpp == 4) return launch_chained(k_assemble_tiles<N, 4, MASK>, grid, kAT, 0, s, L, D, M);
-    if (bpp == 8) return launch_chained(k_assemble_tiles<N, 8, MASK>, grid, kAT, 0, s, L, D, M);
-    return launch_chained(k_assemble_tiles<N, 16, MASK>, grid, kAT, 0, s, L, D, M);
+    if (bpp == 4) return launch_chained(k_assemble_tiles<N, 4, MASK, false>, grid, kAT, 0, s, L, D, M);
+    if (bpp == 8) return launch_chained(k_assemble_tiles<N, 8, MASK, false>, grid, kAT, 0, s, L, D, M);
+    return launch_chained(k_assemble_tiles<N, 16, MASK, false>, grid, kAT, 0, s, L, D, M);
+}
+
+// Whether every buffer of a call starts at a multiple of the pixel size (offsets
+// inside a buffer are whole pixels).
+bool whole_pixels(const void* p, int bpp) { return (reinterpret_cast<uintptr_t>(p) & (uintptr_t)(bpp - 1)) == 0; }
+
+bool whole_pixels(const SrcDesc* src, int n, int bpp, const DstDesc& D)
+{
+    bool ok = whole_pixels(D.color, bpp);
+    for (int i = 0; i < n; ++i) ok = ok && (src[i].x0 >= src[i].x1 || whole_pixels(src[i].color, bpp));
+    return ok;
+}
+
+bool whole_pixels(const PixSrc* src, int n, int bpp, const DstDesc& D)
+{
+    bool ok = whole_pixels(D.color, bpp);
+    for (int i = 0; i < n; ++i) ok = ok && whole_pixels(src[i].color, bpp);
+    return ok;
 }
 
 template <int N>
@@ -426,6 +451,12 @@ cudaError_t tiles_n(const SrcDesc* src, int n, int bpp, const DstDesc& D, cudaSt
     const int tw = 32 * (16 / bpp), th = kARows * kTPasses;
     const dim3 grid(ceil_div(D.W, tw), ceil_div(D.H, th));
     static thread_local TileMasks M;
+    if constexpr (N == EC_MAX_SOURCES) {
+        if (!whole_pixels(src, n, bpp, D)) {
+            if (bpp == 8) return launch_chained(k_assemble_tiles<N, 8, false, true>, grid, kAT, 0, s, L, D, M);
+            return launch_chained(k_assemble_tiles<N, 16, false, true>, grid, kAT, 0, s, L, D, M);
+        }
+    }
     if (N <= 64 && grid.x <= (unsigned)kMaskCols && grid.y <= (unsigned)kMaskRows) {
         for (unsigned c = 0; c < grid.x; ++c) M.col[c] = 0;
         for (unsigned r = 0; r < grid.y; ++r) M.row[r] = 0;
@@ -448,9 +479,15 @@ cudaError_t average_n(const SrcDesc* src, int n, int fmt, const DstDesc& D, cuda
     const SrcList<N> L = make_src_list<N>(src, n);
     const int px = fmt == 0 ? 4 : fmt == 1 ? 1 : 2;
     const dim3 grid(ceil_div(D.W, 32 * px), ceil_div(D.H, kARows * kAPasses));
-    if (fmt == 0) return launch_chained(k_average<N, 0>, grid, kAT, 0, s, L, D);
-    if (fmt == 1) return launch_chained(k_average<N, 1>, grid, kAT, 0, s, L, D);
-    return launch_chained(k_average<N, 2>, grid, kAT, 0, s, L, D);
+    if constexpr (N == EC_MAX_SOURCES) {
+        if (!whole_pixels(src, n, 16 / px, D)) {
+            if (fmt == 1) return launch_chained(k_average<N, 1, true>, grid, kAT, 0, s, L, D);
+            return launch_chained(k_average<N, 2, true>, grid, kAT, 0, s, L, D);
+        }
+    }
+    if (fmt == 0) return launch_chained(k_average<N, 0, false>, grid, kAT, 0, s, L, D);
+    if (fmt == 1) return launch_chained(k_average<N, 1, false>, grid, kAT, 0, s, L, D);
+    return launch_chained(k_average<N, 2, false>, grid, kAT, 0, s, L, D);
 }
 
 template <int N>
@@ -466,9 +503,15 @@ cudaError_t pixels_n(const PixSrc* src, const int16_t* owner, int n, int nx, int
     for (int i = 0; i < nx * ny; ++i) P.owner[i] = owner[i];
     const int px = 16 / bpp;
     const dim3 grid(ceil_div(D.W, 32 * px), ceil_div(D.H, kARows * kAPasses));
-    if (bpp == 4) return launch_chained(k_assemble_pixels<N, 4>, grid, kAT, 0, s, P, D);
-    if (bpp == 8) return launch_chained(k_assemble_pixels<N, 8>, grid, kAT, 0, s, P, D);
-    return launch_chained(k_assemble_pixels<N, 16>, grid, kAT, 0, s, P, D);
+    if constexpr (N == kPixMaxSources) {
+        if (!whole_pixels(src, n, bpp, D)) {
+            if (bpp == 8) return launch_chained(k_assemble_pixels<N, 8, true>, grid, kAT, 0, s, P, D);
+            return launch_chained(k_assemble_pixels<N, 16, true>, grid, kAT, 0, s, P, D);
+        }
+    }
+    if (bpp == 4) return launch_chained(k_assemble_pixels<N, 4, false>, grid, kAT, 0, s, P, D);
+    if (bpp == 8) return launch_chained(k_assemble_pixels<N, 8, false>, grid, kAT, 0, s, P, D);
+    return launch_chained(k_assemble_pixels<N, 16, false>, grid, kAT, 0, s, P, D);
 }
 
 }  // namespace
@@ -476,6 +519,7 @@ cudaError_t pixels_n(const PixSrc* src, const int16_t* owner, int n, int nx, int
 cudaError_t launch_assemble_tiles(const SrcDesc* src, int n, int bpp, const DstDesc& D, cudaStream_t s)
 {
     if (D.W <= 0 || D.H <= 0 || n <= 0) return cudaSuccess;
+    if (!whole_pixels(src, n, bpp, D)) return tiles_n<EC_MAX_SOURCES>(src, n, bpp, D, s);
     if (n <= 16) return tiles_n<16>(src, n, bpp, D, s);
     if (n <= 64) return tiles_n<64>(src, n, bpp, D, s);
     return tiles_n<EC_MAX_SOURCES>(src, n, bpp, D, s);
@@ -484,6 +528,7 @@ cudaError_t launch_assemble_tiles(const SrcDesc* src, int n, int bpp, const DstD
 cudaError_t launch_average(const SrcDesc* src, int n, int fmt, const DstDesc& D, cudaStream_t s)
 {
     if (D.W <= 0 || D.H <= 0) return cudaSuccess;
+    if (!whole_pixels(src, n, fmt == 0 ? 4 : fmt == 1 ? 16 : 8, D)) return average_n<EC_MAX_SOURCES>(src, n, fmt, D, s);
     if (n <= 16) return average_n<16>(src, n, fmt, D, s);
     if (n <= 64) return average_n<64>(src, n, fmt, D, s);
     return average_n<EC_MAX_SOURCES>(src, n, fmt, D, s);
@@ -493,6 +538,7 @@ cudaError_t launch_assemble_pixels(const PixSrc* src, const int16_t* owner, int 
                                    const DstDesc& D, cudaStream_t s)
 {
     if (D.W <= 0 || D.H <= 0 || n <= 0) return cudaSuccess;
+    if (!whole_pixels(src, n, bpp, D)) return pixels_n<kPixMaxSources>(src, owner, n, nx, ny, bpp, D, s);
     if (n <= 16) return pixels_n<16>(src, owner, n, nx, ny, bpp, D, s);
     return pixels_n<kPixMaxSources>(src, owner, n, nx, ny, bpp, D, s);
 }

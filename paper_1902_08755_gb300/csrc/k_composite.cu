@@ -27,7 +27,7 @@ constexpr int kDThreads = 128;
 constexpr int kDRows = kDThreads / 32;
 
 // STEP 32: a lane's pixels lie 32 apart (see depth_px4).
-template <int N, int CB, int STEP>
+template <int N, int CB, int STEP, bool WORDS = false>
 __global__ void __launch_bounds__(kDThreads)
 k_depth(const __grid_constant__ SrcList<N> L, const __grid_constant__ DstDesc D)
 {
@@ -43,7 +43,7 @@ k_depth(const __grid_constant__ SrcList<N> L, const __grid_constant__ DstDesc D)
     chain_wait();
     const int x = tx0 + lane * (STEP == 1 ? 4 : 1), y = ty0 + row;
     if (x >= D.W || y >= D.H) return;
-    depth_px4<CB, STEP>(at, act, nact_s, x, y, D);
+    depth_px4<CB, STEP, WORDS>(at, act, nact_s, x, y, D);
 }
 
 template <int N, bool F16>
@@ -89,6 +89,15 @@ SrcList<N> make_list(const SrcDesc* src, int n)
     return L;
 }
 
+// Whether every RGBA32F buffer of a call starts at a multiple of 16 bytes.
+bool whole_pixels(const SrcDesc* src, int n, int cb, const DstDesc& D)
+{
+    auto whole = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
+    bool ok = cb == 4 || whole(D.color);
+    for (int i = 0; i < n; ++i) ok = ok && (cb == 4 || src[i].x0 >= src[i].x1 || whole(src[i].color));
+    return ok;
+}
+
 template <int N>
 cudaError_t depth_n(const SrcDesc* src, int n, int cb, const DstDesc& D, cudaStream_t s)
 {
@@ -96,6 +105,9 @@ cudaError_t depth_n(const SrcDesc* src, int n, int cb, const DstDesc& D, cudaStr
     const SrcList<N> L = make_list<N>(src, n);
     bool vec = true;
     for (int i = 0; i < n; ++i) vec = vec && (src[i].vec || src[i].x0 >= src[i].x1);
+    if constexpr (N == EC_MAX_SOURCES) {
+        if (!whole_pixels(src, n, cb, D)) return launch_chained(k_depth<N, 16, 1, true>, grid, kDThreads, 0, s, L, D);
+    }
     if (cb != 4) return launch_chained(k_depth<N, 16, 1>, grid, kDThreads, 0, s, L, D);
     if (vec) return launch_chained(k_depth<N, 4, 1>, grid, kDThreads, 0, s, L, D);
     return launch_chained(k_depth<N, 4, 32>, grid, kDThreads, 0, s, L, D);
@@ -120,6 +132,7 @@ cudaError_t launch_depth(const SrcDesc* src, int n, int color_bytes, const DstDe
                          cudaStream_t s)
 {
     if (D.W <= 0 || D.H <= 0) return cudaSuccess;
+    if (!whole_pixels(src, n, color_bytes, D)) return depth_n<EC_MAX_SOURCES>(src, n, color_bytes, D, s);
     if (n <= 16) return depth_n<16>(src, n, color_bytes, D, s);
     if (n <= 64) return depth_n<64>(src, n, color_bytes, D, s);
     return depth_n<EC_MAX_SOURCES>(src, n, color_bytes, D, s);
