@@ -204,9 +204,13 @@ __device__ __forceinline__ uint2 float4_to_half4(float4 f)
     return v;
 }
 
+// How the pixels of an FP16 layer whose rows are not 16-byte groups are read:
+// whole (8-byte aligned layers), by halves, or as each layer's address says.
+enum { kWhole, kHalves, kEither };
+
 // Raw 16 bytes of one premultiplied layer at the thread's pixels (1 RGBA32F or
 // 2 RGBA16F pixels), zero outside the layer's ROI on the per-pixel path.
-template <bool F16>
+template <bool F16, int READ>
 __device__ __forceinline__ uint4 load_raw(const SrcDesc& s, int x, int y)
 {
     const size_t e = (size_t)(y - s.oy) * (size_t)s.pitch + (size_t)(x - s.ox);
@@ -218,20 +222,21 @@ __device__ __forceinline__ uint4 load_raw(const SrcDesc& s, int x, int y)
     } else {
         const uint2* p = reinterpret_cast<const uint2*>(s.color) + e;
         if (s.vec) return ld_stream(reinterpret_cast<const uint4*>(p));
+        const bool whole = READ == kWhole || (READ == kEither && (reinterpret_cast<uintptr_t>(p) & 7u) == 0);
         uint32_t w[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const int xj = x + j;
             if (xj >= s.x0 && xj < s.x1) {
-                const unsigned short* h = reinterpret_cast<const unsigned short*>(p + j);
-                if ((reinterpret_cast<uintptr_t>(p) & 7u) == 0) {      // whole pixels
+                if (whole) {
                     const uint2 v = __ldcs(p + j);
                     w[2 * j] = v.x;
                     w[2 * j + 1] = v.y;
-                    continue;
+                } else {
+                    const unsigned short* h = reinterpret_cast<const unsigned short*>(p + j);
+                    w[2 * j] = (uint32_t)__ldcs(h) | ((uint32_t)__ldcs(h + 1) << 16);
+                    w[2 * j + 1] = (uint32_t)__ldcs(h + 2) | ((uint32_t)__ldcs(h + 3) << 16);
                 }
-                w[2 * j] = (uint32_t)__ldcs(h) | ((uint32_t)__ldcs(h + 1) << 16);
-                w[2 * j + 1] = (uint32_t)__ldcs(h + 2) | ((uint32_t)__ldcs(h + 3) << 16);
             }
         }
         return make_uint4(w[0], w[1], w[2], w[3]);
@@ -303,7 +308,7 @@ __device__ __forceinline__ void store_alpha(const DstDesc& D, int x, int y, cons
 // active layer's ROI covers the CTA's whole tile, so the per-layer and
 // per-pixel range tests are skipped (pixels past the frame's right edge are
 // computed but never stored).
-template <bool F16, class At, int U = 8>
+template <bool F16, int READ = kEither, class At, int U = 8>
 __device__ __forceinline__ void alpha_px(At at, const int16_t* act, int nact, int x, int y,
                                          const DstDesc& D, bool full = false)
 {
@@ -324,7 +329,7 @@ __device__ __forceinline__ void alpha_px(At at, const int16_t* act, int nact, in
             if (idx[u] >= 0) {
                 const SrcDesc& s = at(a + u, idx[u]);
                 live[u] = full || (y >= s.y0 && y < s.y1 && x + PX > s.x0 && x < s.x1);
-                if (live[u]) raw[u] = load_raw<F16>(s, x, y);
+                if (live[u]) raw[u] = load_raw<F16, READ>(s, x, y);
             }
         }
 #pragma unroll
