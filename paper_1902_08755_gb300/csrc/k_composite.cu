@@ -103,14 +103,27 @@ cudaError_t depth_n(const SrcDesc* src, int n, int cb, const DstDesc& D, cudaStr
 {
     const dim3 grid(ceil_div(D.W, 128), ceil_div(D.H, kDRows));
     const SrcList<N> L = make_list<N>(src, n);
-    bool vec = true;
-    for (int i = 0; i < n; ++i) vec = vec && (src[i].vec || src[i].x0 >= src[i].x1);
     if constexpr (N == EC_MAX_SOURCES) {
         if (!whole_pixels(src, n, cb, D)) return launch_chained(k_depth<N, 16, 1, true>, grid, kDThreads, 0, s, L, D);
     }
     if (cb != 4) return launch_chained(k_depth<N, 16, 1>, grid, kDThreads, 0, s, L, D);
-    if (vec) return launch_chained(k_depth<N, 4, 1>, grid, kDThreads, 0, s, L, D);
-    return launch_chained(k_depth<N, 4, 32>, grid, kDThreads, 0, s, L, D);
+    // STEP 32 where most inputs must be read pixel by pixel, and the frame is not
+    // larger than kFarPixels.  Device time of STEP 32 against STEP 1 (whose aligned
+    // inputs keep their 16-byte loads): all inputs unaligned, 640x480 0.89 to 0.95,
+    // 1920x1080 0.94 to 0.97, crops of 1920x1080 0.86 to 0.97; from 3840x2160 on,
+    // where DRAM bounds both, 0.98 to 1.04 (crops of 3840x2160, 8 inputs: 40.5 us
+    // against 38.8).  One unaligned input of 1920x1080: 1.03 to 1.04, of 3840x2160
+    // 1.01 to 1.07; half of them: 1.00 and 1.01 to 1.04.
+    constexpr int64_t kFarPixels = 1 << 22;
+    int live = 0, single = 0;
+    for (int i = 0; i < n; ++i) {
+        if (src[i].x0 >= src[i].x1) continue;
+        ++live;
+        single += !src[i].vec;
+    }
+    if (2 * single > live && (int64_t)D.W * D.H <= kFarPixels)
+        return launch_chained(k_depth<N, 4, 32>, grid, kDThreads, 0, s, L, D);
+    return launch_chained(k_depth<N, 4, 1>, grid, kDThreads, 0, s, L, D);
 }
 
 template <int N>
