@@ -107,21 +107,21 @@ cudaError_t depth_n(const SrcDesc* src, int n, int cb, const DstDesc& D, cudaStr
         if (!whole_pixels(src, n, cb, D)) return launch_chained(k_depth<N, 16, 1, true>, grid, kDThreads, 0, s, L, D);
     }
     if (cb != 4) return launch_chained(k_depth<N, 16, 1>, grid, kDThreads, 0, s, L, D);
-    // STEP 32 where most inputs must be read pixel by pixel, and the frame is not
-    // larger than kFarPixels.  Device time of STEP 32 against STEP 1 (whose aligned
-    // inputs keep their 16-byte loads): all inputs unaligned, 640x480 0.89 to 0.95,
-    // 1920x1080 0.94 to 0.97, crops of 1920x1080 0.86 to 0.97; from 3840x2160 on,
-    // where DRAM bounds both, 0.98 to 1.04 (crops of 3840x2160, 8 inputs: 40.5 us
-    // against 38.8).  One unaligned input of 1920x1080: 1.03 to 1.04, of 3840x2160
-    // 1.01 to 1.07; half of them: 1.00 and 1.01 to 1.04.
-    constexpr int64_t kFarPixels = 1 << 22;
+    // STEP 32 where more than half of the inputs must be read pixel by pixel: the
+    // others' 16-byte loads are given up for them.  Time of STEP 32 against STEP 1,
+    // calls back to back and alone: all inputs unaligned, 640x480 0.97 to 1.00 and
+    // 0.97 to 1.03 (the kernel alone 0.89 to 0.95), 1920x1080 0.95 to 0.97 and 0.98 to
+    // 1.00, 3840x2160 0.95 to 1.02 and 0.98 to 1.00, 7680x4320 1.02 to 1.05 and 0.96 to
+    // 0.98; half of them, 1920x1080 0.99 to 1.00 and 1.00, 3840x2160 1.03 to 1.04 and
+    // 1.00 to 1.01; one, 1920x1080 1.02 to 1.03 and 1.00 to 1.01, 3840x2160 1.02 to 1.04
+    // and 1.01, 7680x4320 1.06 to 1.09 and 1.01 to 1.02.
     int live = 0, single = 0;
     for (int i = 0; i < n; ++i) {
         if (src[i].x0 >= src[i].x1) continue;
         ++live;
         single += !src[i].vec;
     }
-    if (2 * single > live && (int64_t)D.W * D.H <= kFarPixels)
+    if (2 * single > live)
         return launch_chained(k_depth<N, 4, 32>, grid, kDThreads, 0, s, L, D);
     return launch_chained(k_depth<N, 4, 1>, grid, kDThreads, 0, s, L, D);
 }

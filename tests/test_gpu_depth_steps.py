@@ -1,6 +1,5 @@
 """The depth merge gives the same bits whichever way its lanes take their pixels:
-with any number of unaligned inputs among aligned ones, and on both sides of the
-largest frame whose lanes' pixels lie apart."""
+with any number of unaligned inputs among aligned ones."""
 import pytest
 import torch
 
@@ -49,12 +48,3 @@ def test_any_share_of_unaligned_inputs(w, h, rect, n):
     for single in sorted({0, 1, n // 2, n // 2 + 1, n} & set(range(n + 1))):
         a, b = _inputs(n, single, w, h, rect, g)
         assert all(torch.equal(p, q) for p, q in zip(_merge(a, w, h), _merge(b, w, h))), single
-
-
-@pytest.mark.parametrize("w,h", [(2048, 2048), (2049, 2048), (1, 40000)])
-def test_frames_around_the_largest(w, h):
-    require_gpu()
-    g = torch.Generator(device="cuda")
-    g.manual_seed(w)
-    a, b = _inputs(3, 3, w, h, (0, 0, w, h), g)
-    assert all(torch.equal(p, q) for p, q in zip(_merge(a, w, h), _merge(b, w, h)))
