@@ -197,6 +197,7 @@ struct RleScratch {
     uint32_t* groups;       // bytes coded per kGroup chunks
     uint8_t* pool;
     size_t pool_bytes;
+    size_t slots;           // of them the first: a slot of kRlePoolPerUnit bytes per chunk, or none
 };
 constexpr size_t kCompressSmem = kWPB * sizeof(WarpRing);
 
@@ -359,6 +360,23 @@ constexpr int kCT = 128;
 // 7680x4320 sources.)
 constexpr int kStagePlane4 = 2 * kCap + kCap / 2 + kCap / 64 + kChunk / 64 + 6;
 static_assert(kStagePlane4 % 8 == 0, "planes' stages are aligned");
+
+// Pool space of a chunk of `total` bytes: the copy to its place reads up to one
+// word past them, and the last 32-byte sector is filled up (a sector written in
+// part would be fetched from memory when it is read).
+__host__ __device__ constexpr uint32_t pool_need(uint32_t total) { return (total + 4u + 31u) & ~31u; }
+
+// The pool of a launch.  Where it has room behind them for every few-run chunk,
+// chunks of up to kRlePoolPerUnit bytes have slots of their own, and only the
+// others take space with an atomic (2025 flat chunks: 8.2 us, 8.7 with an atomic
+// for each).  Otherwise (the least pool, the allocation-free entry point's,
+// launches of more than 167 thousand chunks) all take what they need: the slots
+// would leave the others no room, and those would be coded twice (8192 few-run
+// chunks of 512 to 770 bytes: 188 us, 75 to 98 so).
+constexpr size_t pool_slots(size_t units, size_t pool_bytes)
+{
+    return pool_bytes >= (kRlePoolPerUnit + pool_need(4 * kStagePlane4)) * units ? kRlePoolPerUnit * units : 0;
+}
 
 // Plane stream of a chunk of len elements from its m <= 32 change points, run
 // by run, where every run is at least 3 bytes (so all of it is repeat tokens).
@@ -650,19 +668,13 @@ k_rle_code(const __grid_constant__ RleJobList<N> J, const RleScratch W, uint32_t
     if (lane == 0) s_T[warp] = T;
     __syncthreads();
     const uint32_t T0 = s_T[0], T1 = s_T[1], T2 = s_T[2], T3 = s_T[3], total = T0 + T1 + T2 + T3;
-    // The unit's own slot, or space behind the slots (+ 4: the copy to its place
-    // reads up to one word past a chunk's bytes).  The last 32-byte sector is
-    // filled up: a sector written in part would be fetched from memory when it
-    // is read.
-    const size_t slots = kRlePoolPerUnit * (size_t)J.total_units;
-    const uint32_t need = (total + 4u + 31u) & ~31u;
-    uint32_t po = kRecode;
-    if (need <= kRlePoolPerUnit && kRlePoolPerUnit * ((size_t)unit + 1) <= W.pool_bytes)
-        po = unit * (uint32_t)(kRlePoolPerUnit / 4);
-    if (po == kRecode) {
+    // the unit's own slot, or space behind the slots
+    const uint32_t need = pool_need(total);
+    uint32_t po = unit * (uint32_t)(kRlePoolPerUnit / 4);
+    if (W.slots == 0 || need > kRlePoolPerUnit) {
         if (tid == 0) {
-            const unsigned long long a = slots + atomicAdd(reinterpret_cast<unsigned long long*>(W.counters + 2),
-                                                           (unsigned long long)need);
+            const unsigned long long a = W.slots + atomicAdd(reinterpret_cast<unsigned long long*>(W.counters + 2),
+                                                             (unsigned long long)need);
             s_po = a + need <= W.pool_bytes ? (uint32_t)(a >> 2) : kRecode;
         }
         __syncthreads();
@@ -1486,9 +1498,8 @@ k_rle_recode(const __grid_constant__ RleJobList<N> J, const RleScratch W, uint32
             dense_chunk(jb, q0, len, jb.mode == 2, T, stage, xw);
             const uint32_t total = T[0] + T[1] + T[2] + T[3];
             if (tid == 0) {
-                const uint32_t need = (total + 4u + 31u) & ~31u;
-                const unsigned long long a = kRlePoolPerUnit * (unsigned long long)J.total_units +
-                    atomicAdd(reinterpret_cast<unsigned long long*>(W.counters + 2), (unsigned long long)need);
+                const uint32_t need = pool_need(total);
+                const unsigned long long a = W.slots + atomicAdd(reinterpret_cast<unsigned long long*>(W.counters + 2), (unsigned long long)need);
                 s_pool = a + need <= W.pool_bytes ? kDense | (uint32_t)(a >> 4) : kRecode;
                 W.rec[unit] = ChunkRec{{(uint16_t)T[0], (uint16_t)T[1], (uint16_t)T[2], (uint16_t)T[3]}, s_pool, 0u};
                 atomicAdd(W.groups + unit / kGroup, total);
@@ -1952,6 +1963,7 @@ cudaError_t launch_rle_compress(const RleJobDesc* jobs, int n, uint32_t total_un
     W.groups = reinterpret_cast<uint32_t*>(base + scratch_groups(total_units));
     W.pool = reinterpret_cast<uint8_t*>(base + scratch_pool(total_units));
     W.pool_bytes = scratch_bytes - scratch_pool(total_units);
+    W.slots = pool_slots(total_units, W.pool_bytes);
     int sms = 0, dev = 0;
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

@@ -25,11 +25,11 @@
 
 namespace {
 
-// counters; a record, two list entries and the pool's slot per chunk; a sum per
+// counters; a record, two list entries and 512 bytes of pool per chunk; a sum per
 // 32 chunks; the pool's alignment
 constexpr size_t kScratchBytes = EC_RLE_NOALLOC_SCRATCH_BYTES;
 static_assert(kScratchBytes >= 16 + (16 + 8 + ec::kRlePoolPerUnit) * EC_RLE_NOALLOC_MAX_CHUNKS +
-                                   4 * (EC_RLE_NOALLOC_MAX_CHUNKS / 32) + 127, "every chunk of the largest image has a slot");
+                                   4 * (EC_RLE_NOALLOC_MAX_CHUNKS / 32) + 127, "512 bytes of pool per chunk of the largest image");
 
 // Counters, chunk records and pool shared by every call of the entry point.
 static __device__ __align__(256) unsigned char g_rle_scratch[kScratchBytes];
