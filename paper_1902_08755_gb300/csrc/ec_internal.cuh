@@ -94,11 +94,16 @@ __device__ __forceinline__ void st_stream(float4* p, float4 v) { __stcs(p, v); }
 // launch_chained is put on the SMs as soon as the last CTAs of the kernel before
 // it on the stream end, without waiting for that kernel's memory flush and the
 // launch's own latency: about 1.7 us less per launch (4 x 640x480 merges back
-// to back 6.2 -> 3.0 us, a compress, decompress and merge of 16 1920x1080
-// sources, nine launches, 117 -> 105 us).  Every thread calls chain_wait before
-// it touches memory that other kernels write: it returns once all earlier
-// kernels of the stream are complete and their writes visible.  Every CTA of a
-// chained kernel calls it, so that its completion implies its predecessors'.
+// to back 6.2 -> 3.0 us; a compress, decompress and merge of 16 1920x1080
+// sources 117 -> 98 us, a memset and a launch fewer among them).  Every thread
+// calls chain_wait before it touches memory that other kernels write: it
+// returns once all earlier kernels of the stream are complete and their writes
+// visible.  Every CTA of a chained kernel calls it, so that its completion
+// implies its predecessors'.  The one exception are a batch's kernels after its
+// first: they read inputs and write outputs before they wait, at their end.
+// That is safe because the first is launched without the attribute (it starts
+// after everything before the batch, and the others once its CTAs have) and
+// because the jobs of a batch do not feed one another.
 // chain_next lets the next chained kernel be put on the SMs once all of this
 // kernel's CTAs have started.  Only the kernels of a batch call it, which share
 // the device by intent: elsewhere the CTAs put there early took the room of

@@ -13,11 +13,11 @@
 // every kind's loop to what they share of its registers, and spilled with more.
 // The kernels of a batch run side by side (a later one's CTAs take the place
 // of an earlier one's as its queue runs out).  HBM-bound: 128 uneven
-// composites, half depth and half alpha, 3.77 GB: 627 us, 0.89 of the measured
+// composites, half depth and half alpha, 3.77 GB: 642 us, 0.87 of the measured
 // copy rate; one kernel with one shared loop body 852 us (640 M warp
 // instructions, four inputs' loads in flight whatever the kind); a kernel per
 // kind 783, with items fetched ahead and the kernels overlapped 756, and with
-// the lean items below 627.
+// the lean items below 642.
 //
 // Every item runs exactly the per-pixel arithmetic of the one-frame kernels
 // (composite_body.cuh), so results are bit-identical to per-job launches and
@@ -191,7 +191,9 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src)
 // kernels' bodies from the staged descriptors.
 //
 // The kernels of a batch are chained but do not wait for one another until
-// they end, so the last items of one overlap the first of the next.
+// they end, so the last items of one overlap the first of the next: no job may
+// read what another one writes, and the first kernel is launched plainly, so
+// that it and all of them start after whatever came before the batch.
 template <int KIND, bool LEAN>
 __global__ void __launch_bounds__(kThreads, 4)
 k_batch(const BatchJob* __restrict__ jobs, const SrcDesc* __restrict__ srcs,

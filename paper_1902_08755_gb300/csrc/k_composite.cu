@@ -109,12 +109,13 @@ cudaError_t depth_n(const SrcDesc* src, int n, int cb, const DstDesc& D, cudaStr
     if (cb != 4) return launch_chained(k_depth<N, 16, 1>, grid, kDThreads, 0, s, L, D);
     // STEP 32 where more than half of the inputs must be read pixel by pixel: the
     // others' 16-byte loads are given up for them.  Time of STEP 32 against STEP 1,
-    // calls back to back and alone: all inputs unaligned, 640x480 0.97 to 1.00 and
-    // 0.97 to 1.03 (the kernel alone 0.89 to 0.95), 1920x1080 0.95 to 0.97 and 0.98 to
-    // 1.00, 3840x2160 0.95 to 1.02 and 0.98 to 1.00, 7680x4320 1.02 to 1.05 and 0.96 to
-    // 0.98; half of them, 1920x1080 0.99 to 1.00 and 1.00, 3840x2160 1.03 to 1.04 and
-    // 1.00 to 1.01; one, 1920x1080 1.02 to 1.03 and 1.00 to 1.01, 3840x2160 1.02 to 1.04
-    // and 1.01, 7680x4320 1.06 to 1.09 and 1.01 to 1.02.
+    // calls back to back and alone: all inputs unaligned, 640x480 0.97 to 1.02 and
+    // 0.97 to 1.03 (the kernel alone 0.89 to 0.95), 1920x1080 0.95 to 0.99 and 0.98 to
+    // 1.01, 3840x2160 0.95 to 1.02 and 0.98 to 1.00, 7680x4320 1.02 to 1.05 and 0.96 to
+    // 0.98; half of them, 1920x1080 0.99 to 1.00 and 0.99 to 1.01, 3840x2160 (4 to 64
+    // inputs) 1.03 to 1.04 and 1.00 to 1.01, 7680x4320 1.06 to 1.09 and 1.00 to 1.01;
+    // one of 8 or more, 1920x1080 1.02 to 1.03 and 1.00 to 1.02, 3840x2160 1.03 to 1.04
+    // and 1.01, 7680x4320 1.06 and 1.02.
     int live = 0, single = 0;
     for (int i = 0; i < n; ++i) {
         if (src[i].x0 >= src[i].x1) continue;

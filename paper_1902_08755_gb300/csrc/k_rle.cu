@@ -15,11 +15,11 @@
 //      three windows of 3 around it is constant), max- and sum-scans over the
 //      CTA, and the streams to the pool where it has room; in mode 0 a CTA per
 //      chunk with block scans, which sizes them.
-//   3. A scan of each job's chunk sizes: the chunks' offsets, the header and
-//      the stream size.
-//   4. Placing: the pooled chunks copied to their place with their end-table
-//      entries; dense chunks that are not in the pool coded again, straight to
-//      their place.
+//   3. Placing: a chunk's offset is the sum of its image's chunks before it
+//      (taken from sums over 32 chunks; in mode 0 a scan launch computes the
+//      offsets); the pooled chunks are copied to their place with their end-table
+//      entries, the header and the stream size are written, and chunks that are
+//      not in the pool are coded again.
 // Every wait (for copies into shared memory) is bounded (EC_ERR_TIMEOUT).
 //
 // Decompress: one CTA of four warps per chunk.  Every warp fetches the header
@@ -163,7 +163,7 @@ constexpr uint32_t kRecode = 0xFFFFFFFFu;      // record: coded again when place
 constexpr uint32_t kDense = 0x80000000u;       // record: a pooled dense chunk (offset / 16 in the low bits)
 
 // One warp's shared memory.  Quarter s of the warp's sequence of quarters
-// (4 per chunk) goes to buf[s % kSlots].
+// (kQPC per chunk) goes to buf[s % kSlots].
 struct WarpRing {
     uint32_t buf[kSlots][kQ + 4];   // + 16 guard bytes before each quarter
     uint64_t full[kSlots];
@@ -585,7 +585,7 @@ k_rle_code(const __grid_constant__ RleJobList<N> J, const RleScratch W, uint32_t
     chain_wait();
     __syncthreads();
     const RleJobDesc& jb = J.j[s_ji];
-    if (jb.n_chunks == 0) return;                     // an empty image: its header is the scan's
+    if (jb.n_chunks == 0) return;                     // an empty image: placing writes its header
     const uint32_t q0 = (unit - jb.first_unit) * (uint32_t)kChunk;
     const int len = (int)min((uint32_t)kChunk, (uint32_t)jb.w * (uint32_t)jb.h - q0);
     if (jb.vec && !(len & 3)) {

@@ -89,8 +89,7 @@ extern "C" ec_status ec_rle_compress_noalloc(const void* src, int32_t w, int32_t
     d.first_unit = 0;
     d.vec = (reinterpret_cast<uintptr_t>(src) & 15u) == 0 && ((w % 4 == 0 && pitch % 4 == 0) || pitch == w);
     const uint32_t units = nchunks > 0 ? (uint32_t)nchunks : 1u;
-    // the launcher clears the counters this call uses (a memset, no
-    // allocation) before the kernels run
+    // the launcher's first kernel clears the counters and sums this call uses
     return ec::launch_rle_compress(&d, 1, units, scratch, kScratchBytes, d_status, (cudaStream_t)s) == cudaSuccess
                ? EC_OK : EC_ERR_CUDA;
 }
