@@ -5,10 +5,8 @@
 //   dL/dc_k^{RGB} = g^{RGB} T_k,   dL/da_k = T_k (g^A - R_k),
 //   R_{n-1} = 0,  R_{k-1} = g.c_k + (1 - a_k) R_k      (reverse "behind" scan).
 // Nothing per layer is kept from the forward.  A CTA owns a tile of 32 lanes
-// by 2 to 64 rows, one pixel per lane (the kernel also takes two adjacent pixels
-// per lane, read and written as one 16-byte word, with segments of at most 4
-// layers); its warps split the tile's layer stack into contiguous segments of
-// at most 8 layers.  A warp loads its layers'
+// by 2 to 64 rows, one pixel per lane; its warps split the tile's layer stack
+// into contiguous segments of at most 8 layers.  A warp loads its layers'
 // pixels straight into registers (zero outside a layer's ROI, which is
 // exactly a transparent layer), runs its segment's forward, and keeps per
 // layer only T', g.c and a.  Both recurrences split exactly across segments:
@@ -42,7 +40,9 @@ namespace {
 
 constexpr int kMaxRows = 64;      // rows per alpha-backward CTA, at most
 constexpr int kMaxWarps = 32;     // segments (warps) per CTA
-static_assert(8 * kMaxWarps >= kMaxBwdLayers, "every stack fits one CTA");
+constexpr int kMS = 8;            // layers per segment, at most
+constexpr int kTW = 32;           // columns of a tile: one per lane
+static_assert(kMS * kMaxWarps >= kMaxBwdLayers, "every stack fits one CTA");
 
 __device__ __forceinline__ float4 h4_to_f4(uint2 v)
 {
@@ -60,24 +60,23 @@ __device__ __forceinline__ uint2 f4_to_h4(float4 f)
     return v;
 }
 
-// What a CTA needs of one layer for its tile (TW columns by `rows` rows),
+// What a CTA needs of one layer for its tile (kTW columns by `rows` rows),
 // built once per CTA: addresses of pixel (tx0, ty0) in the colour and
 // gradient buffers (offset only by rows and columns that lie inside the ROI /
 // pvp before use), the pitch, the ROI and gradient ranges (columns relative
-// to tx0), the colour alignment class, and whether pixel pairs starting at an
-// even column may be read (wide) or their gradients written (gwide) as one
-// 16-byte word.
+// to tx0), the colour alignment class, and whether gradients may be written a
+// pixel at a time.
 struct BandTile {
     uintptr_t src;
     uintptr_t grad;
     int32_t pitch;
     int32_t ry0, ry1, gy0, gy1;
     int16_t rx0, rx1, gx0, gx1;
-    int8_t cls, gvec, wide, gwide;
+    int8_t cls, gvec, pad[2];
 };
 static_assert(sizeof(BandTile) == 48, "tile record");
 
-template <bool F16, bool G16, int TW>
+template <bool F16, bool G16>
 __device__ __forceinline__ BandTile make_band_tile(const BwdDesc& d, int tx0, int ty0)
 {
     constexpr int S = F16 ? 8 : 16, GS = G16 ? 8 : 16;
@@ -88,15 +87,13 @@ __device__ __forceinline__ BandTile make_band_tile(const BwdDesc& d, int tx0, in
     t.pitch = d.pitch;
     t.ry0 = d.y0; t.ry1 = d.y1;
     t.gy0 = d.gy0; t.gy1 = d.gy1;
-    t.rx0 = (int16_t)max(min(d.x0 - tx0, TW), 0);
-    t.rx1 = (int16_t)max(min(d.x1 - tx0, TW), 0);
-    t.gx0 = (int16_t)max(min(d.gx0 - tx0, TW), 0);
-    t.gx1 = (int16_t)max(min(d.gx1 - tx0, TW), 0);
+    t.rx0 = (int16_t)max(min(d.x0 - tx0, kTW), 0);
+    t.rx1 = (int16_t)max(min(d.x1 - tx0, kTW), 0);
+    t.gx0 = (int16_t)max(min(d.gx0 - tx0, kTW), 0);
+    t.gx1 = (int16_t)max(min(d.gx1 - tx0, kTW), 0);
     t.cls = (int8_t)d.cls;
     t.gvec = (int8_t)d.gvec;
-    const bool even = (d.pitch & 1) == 0;
-    t.wide = (int8_t)(F16 && even && d.cls >= 8 && (t.src & 15u) == 0);
-    t.gwide = (int8_t)(G16 && even && d.gvec && (t.grad & 15u) == 0);
+    t.pad[0] = t.pad[1] = 0;
     return t;
 }
 
@@ -152,40 +149,40 @@ __device__ __forceinline__ void store_grad(const BwdDesc& d, int x, int y, float
     store_grad_at<G16>(a, d.gvec != 0, v);
 }
 
-// Alpha backward (and fused forward + backward) for one tile of 32 * PX
-// pixels (PX per lane, adjacent) by `rows` rows.  blockDim.x = 32 * NS: warp s
-// owns segment s of the tile's active layers, at most MS of them.  Tiles that
+// Alpha backward (and fused forward + backward) for one tile of 32 columns by
+// `rows` rows.  blockDim.x = 32 * NS: warp s
+// owns segment s of the tile's active layers, at most kMS of them.  Tiles that
 // every active layer covers entirely (ROI and gradient rectangle) skip the
 // per-row range checks; lean tiles (also aligned, one pitch, inside the
 // frame) take the row passes without any tests.
-template <int N, bool F16, bool G16, bool FUSED, int PX, int MS>
+template <int N, bool F16, bool G16, bool FUSED>
 __global__ void __launch_bounds__(32 * kMaxWarps, 1)
 k_alpha_bwd(const __grid_constant__ BwdList<N> L, const __grid_constant__ DstDesc D,
             const float4* __restrict__ g, int cap, int rows)
 {
-    constexpr int S = F16 ? 8 : 16, GS = G16 ? 8 : 16, TW = 32 * PX;
+    constexpr int S = F16 ? 8 : 16, GS = G16 ? 8 : 16;
     using RawPx = typename Px<F16>::T;
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ int16_t act[N];
     __shared__ int nact_s;
     BandTile* tiles = reinterpret_cast<BandTile*>(smem);                    // [cap]
     const int NS = (int)(blockDim.x / 32);
-    // per row parity, segment and pixel: [2][NS][PX][32], pixel (lane, q) at
-    // q * 32 + lane.  Rows alternate between the two copies, so a row's writes
-    // never meet the previous row's reads and one barrier per row suffices.
+    // per row parity, segment and lane: [2][NS][32].  Rows alternate between the
+    // two copies, so a row's writes never meet the previous row's reads and one
+    // barrier per row suffices.
     float* const Ps0 = reinterpret_cast<float*>(smem + (size_t)cap * sizeof(BandTile));
-    float* const As0 = Ps0 + 2 * NS * TW;
-    float4* const Cs0 = reinterpret_cast<float4*>(As0 + 2 * NS * TW);       // (fused)
-    // FP16 lean tiles: each warp's per-layer state of its row, [MS][32] per
+    float* const As0 = Ps0 + 2 * NS * kTW;
+    float4* const Cs0 = reinterpret_cast<float4*>(As0 + 2 * NS * kTW);       // (fused)
+    // FP16 lean tiles: each warp's per-layer state of its row, [kMS][32] per
     // warp -- (T', g.c) as floats and a as the half it was read as (exact) --
     // so that the registers can hold the next row's loads
-    float2* const St0 = reinterpret_cast<float2*>(Cs0 + (FUSED ? 2 * NS * TW : 0));
-    float2* const St = St0 + (threadIdx.x / 32) * MS * 32;
-    unsigned short* const Sa = reinterpret_cast<unsigned short*>(St0 + NS * MS * 32) + (threadIdx.x / 32) * MS * 32;
+    float2* const St0 = reinterpret_cast<float2*>(Cs0 + (FUSED ? 2 * NS * kTW : 0));
+    float2* const St = St0 + (threadIdx.x / 32) * kMS * 32;
+    unsigned short* const Sa = reinterpret_cast<unsigned short*>(St0 + NS * kMS * 32) + (threadIdx.x / 32) * kMS * 32;
 
     const int lane = threadIdx.x & 31, sg = threadIdx.x / 32;
-    const int tx0 = blockIdx.x * TW, ty0 = blockIdx.y * rows;
-    const int tx1 = min(tx0 + TW, D.W), ty1 = min(ty0 + rows, D.H);
+    const int tx0 = blockIdx.x * kTW, ty0 = blockIdx.y * rows;
+    const int tx1 = min(tx0 + kTW, D.W), ty1 = min(ty0 + rows, D.H);
 
     // layers whose gradient rectangle meets the tile, in compositing order
     if (threadIdx.x < 32) {
@@ -209,7 +206,7 @@ k_alpha_bwd(const __grid_constant__ BwdList<N> L, const __grid_constant__ DstDes
     bool covers = true, lean = true;
     for (int k = threadIdx.x; k < nact; k += blockDim.x) {
         const BwdDesc& dk = L.d[act[k]];
-        const BandTile t = make_band_tile<F16, G16, TW>(dk, tx0, ty0);
+        const BandTile t = make_band_tile<F16, G16>(dk, tx0, ty0);
         tiles[k] = t;
         covers = covers && t.rx0 == 0 && t.rx1 >= tx1 - tx0 && t.ry0 <= ty0 && t.ry1 >= ty1 &&
                  t.gx0 == 0 && t.gx1 >= tx1 - tx0 && t.gy0 <= ty0 && t.gy1 >= ty1;
@@ -220,28 +217,25 @@ k_alpha_bwd(const __grid_constant__ BwdList<N> L, const __grid_constant__ DstDes
     // the frame, with whole-pixel vector loads and stores and one pitch, so a
     // row's addresses are one offset from the tile records
     const bool lean_all = __syncthreads_and(covers && lean);
-    const bool fast = PX == 1 && tx0 + TW <= D.W && lean_all;
+    const bool fast = tx0 + kTW <= D.W && lean_all;
 
-    const int k0 = (sg * nact) / NS, cnt = ((sg + 1) * nact) / NS - k0;   // cnt <= MS
-    const int c0 = PX * lane;                                              // first column of this lane
-    bool valid[PX];
-#pragma unroll
-    for (int q = 0; q < PX; ++q) valid[q] = tx0 + c0 + q < D.W;
+    const int k0 = (sg * nact) / NS, cnt = ((sg + 1) * nact) / NS - k0;   // cnt <= kMS
+    const bool valid = tx0 + lane < D.W;
 
     // Fused output of row y: out = sum over segments u of Tstart(u) C_u,
     // evaluated front to back.  Lane (pixel, channel) of the first warps takes
-    // one channel of one pixel (TW * 4 of them), so no single warp carries the
+    // one channel of one pixel (kTW * 4 of them), so no single warp carries the
     // whole composite; T_final is the running product after the last segment.
     auto composite_row = [&](int y, const float* Ps, const float4* Cs) {
-        for (int i = threadIdx.x; i < 4 * TW; i += blockDim.x) {
+        for (int i = threadIdx.x; i < 4 * kTW; i += blockDim.x) {
             const int idx = i >> 2, ch = i & 3;
-            const int x = tx0 + PX * (idx & 31) + (idx >> 5);
+            const int x = tx0 + idx;
             if (x >= D.W) continue;
             float Tacc = 1.0f, o = 0.0f;
 #pragma unroll 4
             for (int u = 0; u < NS; ++u) {
-                o = fmaf(Tacc, reinterpret_cast<const float*>(Cs + u * TW + idx)[ch], o);
-                Tacc *= Ps[u * TW + idx];
+                o = fmaf(Tacc, reinterpret_cast<const float*>(Cs + u * kTW + idx)[ch], o);
+                Tacc *= Ps[u * kTW + idx];
             }
             const size_t e = ((size_t)y * (size_t)D.pitch + (size_t)x) * 4 + ch;
             if constexpr (F16) reinterpret_cast<__half*>(D.color)[e] = __float2half_rn(o);
@@ -250,17 +244,17 @@ k_alpha_bwd(const __grid_constant__ BwdList<N> L, const __grid_constant__ DstDes
         }
     };
 
-    // Row pass of a lean tile (one pixel per lane): no range or alignment
+    // Row pass of a lean tile: no range or alignment
     // tests, one row offset for every layer's load and gradient store.
     auto row_fast = [&](int y) {
-        float* const Ps = Ps0 + (y & 1) * NS * TW;
-        float* const As = As0 + (y & 1) * NS * TW;
-        float4* const Cs = Cs0 + (y & 1) * NS * TW;
+        float* const Ps = Ps0 + (y & 1) * NS * kTW;
+        float* const As = As0 + (y & 1) * NS * kTW;
+        float4* const Cs = Cs0 + (y & 1) * NS * kTW;
         const float4 gp = __ldcs(g + (size_t)y * D.W + tx0 + lane);
         const int64_t r = (int64_t)(y - ty0) * pitch0 + lane;
-        RawPx raw[MS];
+        RawPx raw[kMS];
 #pragma unroll
-        for (int j = 0; j < MS; ++j) {
+        for (int j = 0; j < kMS; ++j) {
             if constexpr (F16) raw[j] = make_uint2(0u, 0u);
             else raw[j] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (j < cnt) {
@@ -269,11 +263,11 @@ k_alpha_bwd(const __grid_constant__ BwdList<N> L, const __grid_constant__ DstDes
                 else raw[j] = __ldcs(reinterpret_cast<const float4*>(a));
             }
         }
-        float Tl[MS], gcl[MS], al[MS];
+        float Tl[kMS], gcl[kMS], al[kMS];
         float Tp = 1.0f, A = 0.0f;
         float4 Cl = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int j = 0; j < MS; ++j) {
+        for (int j = 0; j < kMS; ++j) {
             float4 c;
             if constexpr (F16) c = h4_to_f4(raw[j]);
             else c = raw[j];
@@ -292,18 +286,18 @@ k_alpha_bwd(const __grid_constant__ BwdList<N> L, const __grid_constant__ DstDes
                 Tp = fmaf(-Tp, c.w, Tp);
             }
         }
-        Ps[sg * TW + lane] = Tp;
-        As[sg * TW + lane] = A;
-        if (FUSED) Cs[sg * TW + lane] = Cl;
+        Ps[sg * kTW + lane] = Tp;
+        As[sg * kTW + lane] = A;
+        if (FUSED) Cs[sg * kTW + lane] = Cl;
         __syncthreads();
 
         float Tstart = 1.0f, R = 0.0f;
-        for (int u = 0; u < sg; ++u) Tstart *= Ps[u * TW + lane];
-        for (int u = NS - 1; u > sg; --u) R = fmaf(Ps[u * TW + lane], R, As[u * TW + lane]);
+        for (int u = 0; u < sg; ++u) Tstart *= Ps[u * kTW + lane];
+        for (int u = NS - 1; u > sg; --u) R = fmaf(Ps[u * kTW + lane], R, As[u * kTW + lane]);
         if (FUSED) composite_row(y, Ps, Cs);
 
 #pragma unroll
-        for (int j = MS - 1; j >= 0; --j) {
+        for (int j = kMS - 1; j >= 0; --j) {
             if (j < cnt) {
                 const float Tk = Tstart * Tl[j];
                 const float4 gr = make_float4(gp.x * Tk, gp.y * Tk, gp.z * Tk, Tk * (gp.w - R));
@@ -318,13 +312,13 @@ k_alpha_bwd(const __grid_constant__ BwdList<N> L, const __grid_constant__ DstDes
     // gradient are loaded while this row's exchange and reverse scan run.
     // The per-layer state lives in shared memory (St) meanwhile.
     auto rows_fast16 = [&]() {
-        RawPx raw[MS];
+        RawPx raw[kMS];
         float4 gn;
         auto load_row = [&](int y) {
             const int64_t r = (int64_t)(y - ty0) * pitch0 + lane;
             gn = __ldcs(g + (size_t)y * D.W + tx0 + lane);
 #pragma unroll
-            for (int j = 0; j < MS; ++j) {
+            for (int j = 0; j < kMS; ++j) {
                 if constexpr (F16) raw[j] = make_uint2(0u, 0u);
                 else raw[j] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (j < cnt) {
@@ -336,14 +330,14 @@ k_alpha_bwd(const __grid_constant__ BwdList<N> L, const __grid_constant__ DstDes
         };
         load_row(ty0);
         for (int y = ty0; y < ty1; ++y) {
-            float* const Ps = Ps0 + (y & 1) * NS * TW;
-            float* const As = As0 + (y & 1) * NS * TW;
-            float4* const Cs = Cs0 + (y & 1) * NS * TW;
+            float* const Ps = Ps0 + (y & 1) * NS * kTW;
+            float* const As = As0 + (y & 1) * NS * kTW;
+            float4* const Cs = Cs0 + (y & 1) * NS * kTW;
             const float4 gp = gn;
             float Tp = 1.0f, A = 0.0f;
             float4 Cl = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int j = 0; j < MS; ++j) {
+            for (int j = 0; j < kMS; ++j) {
                 float4 c;
                 if constexpr (F16) c = h4_to_f4(raw[j]);
                 else c = raw[j];
@@ -361,20 +355,20 @@ k_alpha_bwd(const __grid_constant__ BwdList<N> L, const __grid_constant__ DstDes
                     Tp = fmaf(-Tp, c.w, Tp);
                 }
             }
-            Ps[sg * TW + lane] = Tp;
-            As[sg * TW + lane] = A;
-            if (FUSED) Cs[sg * TW + lane] = Cl;
+            Ps[sg * kTW + lane] = Tp;
+            As[sg * kTW + lane] = A;
+            if (FUSED) Cs[sg * kTW + lane] = Cl;
             __syncthreads();
             if (y + 1 < ty1) load_row(y + 1);
 
             float Tstart = 1.0f, R = 0.0f;
-            for (int u = 0; u < sg; ++u) Tstart *= Ps[u * TW + lane];
-            for (int u = NS - 1; u > sg; --u) R = fmaf(Ps[u * TW + lane], R, As[u * TW + lane]);
+            for (int u = 0; u < sg; ++u) Tstart *= Ps[u * kTW + lane];
+            for (int u = NS - 1; u > sg; --u) R = fmaf(Ps[u * kTW + lane], R, As[u * kTW + lane]);
             if (FUSED) composite_row(y, Ps, Cs);
 
             const int64_t r = (int64_t)(y - ty0) * pitch0 + lane;
 #pragma unroll
-            for (int j = MS - 1; j >= 0; --j) {
+            for (int j = kMS - 1; j >= 0; --j) {
                 if (j < cnt) {
                     const float2 st = St[j * 32 + lane];
                     const float a = __half2float(__ushort_as_half(Sa[j * 32 + lane]));
@@ -390,133 +384,74 @@ k_alpha_bwd(const __grid_constant__ BwdList<N> L, const __grid_constant__ DstDes
 
     auto row_pass = [&](auto full_c, int y) {
         constexpr bool FULL = decltype(full_c)::value;
-        float* const Ps = Ps0 + (y & 1) * NS * TW;
-        float* const As = As0 + (y & 1) * NS * TW;
-        float4* const Cs = Cs0 + (y & 1) * NS * TW;
-        float4 gp[PX];
-#pragma unroll
-        for (int q = 0; q < PX; ++q)
-            gp[q] = valid[q] ? __ldcs(g + (size_t)y * D.W + tx0 + c0 + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+        float* const Ps = Ps0 + (y & 1) * NS * kTW;
+        float* const As = As0 + (y & 1) * NS * kTW;
+        float4* const Cs = Cs0 + (y & 1) * NS * kTW;
+        const float4 gp = valid ? __ldcs(g + (size_t)y * D.W + tx0 + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
         // this segment's pixels, all loads in flight before any is used
-        RawPx raw[MS][PX];
+        RawPx raw[kMS];
 #pragma unroll
-        for (int j = 0; j < MS; ++j) {
-#pragma unroll
-            for (int q = 0; q < PX; ++q) {
-                if constexpr (F16) raw[j][q] = make_uint2(0u, 0u);
-                else raw[j][q] = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
+        for (int j = 0; j < kMS; ++j) {
+            if constexpr (F16) raw[j] = make_uint2(0u, 0u);
+            else raw[j] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (j < cnt) {
                 const BandTile& t = tiles[k0 + j];
-                if (FULL || (y >= t.ry0 && y < t.ry1)) {
-                    const uintptr_t a = t.src + (uintptr_t)(((int64_t)(y - ty0) * t.pitch + c0) * S);
-                    bool in[PX];
-#pragma unroll
-                    for (int q = 0; q < PX; ++q)
-                        in[q] = valid[q] && (FULL || (c0 + q >= t.rx0 && c0 + q < t.rx1));
-                    bool done = false;
-                    if constexpr (PX == 2) {
-                        if (t.wide && in[0] && in[1]) {
-                            const uint4 v = __ldcs(reinterpret_cast<const uint4*>(a));
-                            raw[j][0] = make_uint2(v.x, v.y);
-                            raw[j][1] = make_uint2(v.z, v.w);
-                            done = true;
-                        }
-                    }
-                    if (!done) {
-#pragma unroll
-                        for (int q = 0; q < PX; ++q) {
-                            if (!in[q]) continue;
-                            if constexpr (F16) raw[j][q] = load_px16(a + q * S, t.cls);
-                            else raw[j][q] = load_px32(a + q * S, t.cls);
-                        }
-                    }
+                if ((FULL || (y >= t.ry0 && y < t.ry1)) && valid && (FULL || (lane >= t.rx0 && lane < t.rx1))) {
+                    const uintptr_t a = t.src + (uintptr_t)(((int64_t)(y - ty0) * t.pitch + lane) * S);
+                    if constexpr (F16) raw[j] = load_px16(a, t.cls);
+                    else raw[j] = load_px32(a, t.cls);
                 }
             }
         }
-        // local forward; keep T', g.c and a per layer and pixel
-        float Tl[MS][PX], gcl[MS][PX], al[MS][PX];
-        float Tp[PX], A[PX];
-        float4 Cl[PX];
+        // local forward; keep T', g.c and a per layer
+        float Tl[kMS], gcl[kMS], al[kMS];
+        float Tp = 1.0f, A = 0.0f;
+        float4 Cl = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int q = 0; q < PX; ++q) { Tp[q] = 1.0f; A[q] = 0.0f; Cl[q] = make_float4(0.f, 0.f, 0.f, 0.f); }
-#pragma unroll
-        for (int j = 0; j < MS; ++j) {
-#pragma unroll
-            for (int q = 0; q < PX; ++q) {
-                float4 c;
-                if constexpr (F16) c = h4_to_f4(raw[j][q]);
-                else c = raw[j][q];
-                const float gc = fmaf(gp[q].x, c.x, fmaf(gp[q].y, c.y, fmaf(gp[q].z, c.z, gp[q].w * c.w)));
-                Tl[j][q] = Tp[q];
-                gcl[j][q] = gc;
-                al[j][q] = c.w;
-                if (j < cnt) {
-                    if (FUSED) {
-                        Cl[q].x = fmaf(Tp[q], c.x, Cl[q].x);
-                        Cl[q].y = fmaf(Tp[q], c.y, Cl[q].y);
-                        Cl[q].z = fmaf(Tp[q], c.z, Cl[q].z);
-                        Cl[q].w = fmaf(Tp[q], c.w, Cl[q].w);
-                    }
-                    A[q] = fmaf(Tp[q], gc, A[q]);
-                    Tp[q] = fmaf(-Tp[q], c.w, Tp[q]);
+        for (int j = 0; j < kMS; ++j) {
+            float4 c;
+            if constexpr (F16) c = h4_to_f4(raw[j]);
+            else c = raw[j];
+            const float gc = fmaf(gp.x, c.x, fmaf(gp.y, c.y, fmaf(gp.z, c.z, gp.w * c.w)));
+            Tl[j] = Tp;
+            gcl[j] = gc;
+            al[j] = c.w;
+            if (j < cnt) {
+                if (FUSED) {
+                    Cl.x = fmaf(Tp, c.x, Cl.x);
+                    Cl.y = fmaf(Tp, c.y, Cl.y);
+                    Cl.z = fmaf(Tp, c.z, Cl.z);
+                    Cl.w = fmaf(Tp, c.w, Cl.w);
                 }
+                A = fmaf(Tp, gc, A);
+                Tp = fmaf(-Tp, c.w, Tp);
             }
         }
-#pragma unroll
-        for (int q = 0; q < PX; ++q) {
-            Ps[sg * TW + q * 32 + lane] = Tp[q];
-            As[sg * TW + q * 32 + lane] = A[q];
-            if (FUSED) Cs[sg * TW + q * 32 + lane] = Cl[q];
-        }
+        Ps[sg * kTW + lane] = Tp;
+        As[sg * kTW + lane] = A;
+        if (FUSED) Cs[sg * kTW + lane] = Cl;
         __syncthreads();
 
-        float Tstart[PX], R[PX];
-#pragma unroll
-        for (int q = 0; q < PX; ++q) {
-            Tstart[q] = 1.0f;
-            for (int u = 0; u < sg; ++u) Tstart[q] *= Ps[u * TW + q * 32 + lane];
-            R[q] = 0.0f;
-            for (int u = NS - 1; u > sg; --u) R[q] = fmaf(Ps[u * TW + q * 32 + lane], R[q], As[u * TW + q * 32 + lane]);
-        }
+        float Tstart = 1.0f, R = 0.0f;
+        for (int u = 0; u < sg; ++u) Tstart *= Ps[u * kTW + lane];
+        for (int u = NS - 1; u > sg; --u) R = fmaf(Ps[u * kTW + lane], R, As[u * kTW + lane]);
 
         if (FUSED) composite_row(y, Ps, Cs);
 
         // reverse over this segment, entering with the R of the layers behind it
 #pragma unroll
-        for (int j = MS - 1; j >= 0; --j) {
+        for (int j = kMS - 1; j >= 0; --j) {
             if (j < cnt) {
                 const BandTile& t = tiles[k0 + j];
-                if (FULL || (y >= t.gy0 && y < t.gy1)) {
-                    const bool rrow = FULL || (y >= t.ry0 && y < t.ry1);
-                    float4 gr[PX];
-                    bool gin[PX];
-#pragma unroll
-                    for (int q = 0; q < PX; ++q) {
-                        const int c = c0 + q;
-                        gin[q] = valid[q] && (FULL || (c >= t.gx0 && c < t.gx1));
-                        const float Tk = Tstart[q] * Tl[j][q];
-                        const bool in = FULL || (rrow && c >= t.rx0 && c < t.rx1);
-                        gr[q] = in ? make_float4(gp[q].x * Tk, gp[q].y * Tk, gp[q].z * Tk, Tk * (gp[q].w - R[q]))
-                                   : make_float4(0.f, 0.f, 0.f, 0.f);
-                    }
-                    const uintptr_t ga = t.grad + (uintptr_t)(((int64_t)(y - ty0) * t.pitch + c0) * GS);
-                    bool done = false;
-                    if constexpr (PX == 2 && G16) {
-                        if (t.gwide && gin[0] && gin[1]) {
-                            const uint2 h0 = f4_to_h4(gr[0]), h1 = f4_to_h4(gr[1]);
-                            __stcs(reinterpret_cast<uint4*>(ga), make_uint4(h0.x, h0.y, h1.x, h1.y));
-                            done = true;
-                        }
-                    }
-                    if (!done) {
-#pragma unroll
-                        for (int q = 0; q < PX; ++q)
-                            if (gin[q]) store_grad_at<G16>(ga + q * GS, t.gvec != 0, gr[q]);
-                    }
+                if ((FULL || (y >= t.gy0 && y < t.gy1)) && valid && (FULL || (lane >= t.gx0 && lane < t.gx1))) {
+                    const float Tk = Tstart * Tl[j];
+                    const bool in = FULL || (y >= t.ry0 && y < t.ry1 && lane >= t.rx0 && lane < t.rx1);
+                    const float4 gr = in ? make_float4(gp.x * Tk, gp.y * Tk, gp.z * Tk, Tk * (gp.w - R))
+                                         : make_float4(0.f, 0.f, 0.f, 0.f);
+                    const uintptr_t ga = t.grad + (uintptr_t)(((int64_t)(y - ty0) * t.pitch + lane) * GS);
+                    store_grad_at<G16>(ga, t.gvec != 0, gr);
                 }
-#pragma unroll
-                for (int q = 0; q < PX; ++q) R[q] = fmaf(1.0f - al[j][q], R[q], gcl[j][q]);
+                R = fmaf(1.0f - al[j], R, gcl[j]);
             }
         }
     };
@@ -596,11 +531,11 @@ BwdList<N> make_bwd(const BwdDesc* d, int n)
 }
 
 // Warps (segments) per alpha-backward CTA for a stack of n layers: enough for
-// ms layers each, and at least four (or n) so that short stacks still split
+// kMS layers each, and at least four (or n) so that short stacks still split
 // their scans.
-int alpha_bwd_warps(int n, int ms)
+int alpha_bwd_warps(int n)
 {
-    const int need = (n + ms - 1) / ms;
+    const int need = (n + kMS - 1) / kMS;
     return std::max(1, std::min(kMaxWarps, std::max(need, std::min(n, 4))));
 }
 
@@ -615,10 +550,10 @@ int alpha_bwd_warps(int n, int ms)
 // the shared memory 227 KB.
 // Measured, fused: 12 FP32 layers over 333 x 257, 16 -> 3 rows, 37.9 -> 11.8 us;
 // 128 FP16 layers over 1920 x 1080, 32 -> 54 rows, 785 -> 740 us.
-int alpha_bwd_rows(int n, int W, int H, int tw, int ns, size_t smem, int sms)
+int alpha_bwd_rows(int n, int W, int H, int ns, size_t smem, int sms)
 {
     const int slots = sms * std::max(1, std::min(32 / ns, (int)(232448 / (smem + 1024))));
-    const int64_t tx = ceil_div(W, tw);
+    const int64_t tx = ceil_div(W, kTW);
     const int most = n > 64 ? kMaxRows : 16;
     int best = most;
     int64_t best_cost = INT64_MAX;
@@ -630,30 +565,23 @@ int alpha_bwd_rows(int n, int W, int H, int tw, int ns, size_t smem, int sms)
     return best;
 }
 
-template <int N, bool F16, bool G16, bool FUSED, int PX, int MS>
+// Eight layers per warp, FP32 and FP16 alike.  (Two FP16 pixels per lane with four
+// layers per warp was 1.5 % slower on 32 x 2048^2.)
+template <int N, bool F16, bool G16, bool FUSED>
 cudaError_t alpha_bwd_n(const BwdDesc* d, int n, const DstDesc& D, const float4* g, cudaStream_t s)
 {
-    const int ns = alpha_bwd_warps(n, MS), cap = std::max(n, 1), tw = 32 * PX;
-    const size_t smem = (size_t)cap * sizeof(BandTile) + 2 * (size_t)ns * tw * (8 + (FUSED ? 16 : 0)) +
-                        (F16 ? (size_t)ns * MS * 32 * (sizeof(float2) + sizeof(unsigned short)) : 0);
-    auto kern = k_alpha_bwd<N, F16, G16, FUSED, PX, MS>;
+    const int ns = alpha_bwd_warps(n), cap = std::max(n, 1);
+    const size_t smem = (size_t)cap * sizeof(BandTile) + 2 * (size_t)ns * kTW * (8 + (FUSED ? 16 : 0)) +
+                        (F16 ? (size_t)ns * kMS * 32 * (sizeof(float2) + sizeof(unsigned short)) : 0);
+    auto kern = k_alpha_bwd<N, F16, G16, FUSED>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const int rows = alpha_bwd_rows(n, D.W, D.H, tw, ns, smem, sms);
-    const dim3 grid(ceil_div(D.W, tw), ceil_div(D.H, rows));
+    const int rows = alpha_bwd_rows(n, D.W, D.H, ns, smem, sms);
+    const dim3 grid(ceil_div(D.W, kTW), ceil_div(D.H, rows));
     return launch_chained(kern, grid, 32 * ns, smem, s, make_bwd<N>(d, n), D, g, cap, rows);
-}
-
-// One pixel per lane and eight layers per warp, FP32 and FP16 alike (two FP16
-// pixels per lane with four layers per warp was 1.5% slower on 32 x 2048^2; the
-// kernel keeps the two-pixel form for other tile choices).
-template <int N, bool F16, bool G16, bool FUSED>
-cudaError_t alpha_bwd_px(const BwdDesc* d, int n, const DstDesc& D, const float4* g, cudaStream_t s)
-{
-    return alpha_bwd_n<N, F16, G16, FUSED, 1, 8>(d, n, D, g, s);
 }
 
 template <int N>
@@ -661,15 +589,15 @@ cudaError_t alpha_bwd_dispatch(const BwdDesc* d, int n, bool f16, bool g16, bool
                                const DstDesc& D, const float4* g, cudaStream_t s)
 {
     if (f16) {
-        if (g16) return fused ? alpha_bwd_px<N, true, true, true>(d, n, D, g, s)
-                              : alpha_bwd_px<N, true, true, false>(d, n, D, g, s);
-        return fused ? alpha_bwd_px<N, true, false, true>(d, n, D, g, s)
-                     : alpha_bwd_px<N, true, false, false>(d, n, D, g, s);
+        if (g16) return fused ? alpha_bwd_n<N, true, true, true>(d, n, D, g, s)
+                              : alpha_bwd_n<N, true, true, false>(d, n, D, g, s);
+        return fused ? alpha_bwd_n<N, true, false, true>(d, n, D, g, s)
+                     : alpha_bwd_n<N, true, false, false>(d, n, D, g, s);
     }
-    if (g16) return fused ? alpha_bwd_px<N, false, true, true>(d, n, D, g, s)
-                          : alpha_bwd_px<N, false, true, false>(d, n, D, g, s);
-    return fused ? alpha_bwd_px<N, false, false, true>(d, n, D, g, s)
-                 : alpha_bwd_px<N, false, false, false>(d, n, D, g, s);
+    if (g16) return fused ? alpha_bwd_n<N, false, true, true>(d, n, D, g, s)
+                          : alpha_bwd_n<N, false, true, false>(d, n, D, g, s);
+    return fused ? alpha_bwd_n<N, false, false, true>(d, n, D, g, s)
+                 : alpha_bwd_n<N, false, false, false>(d, n, D, g, s);
 }
 
 }  // namespace
