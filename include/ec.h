@@ -193,9 +193,10 @@ ec_status ec_composite_depth_backward(ec_ctx* ctx, const int16_t* winner,
  * into tiles (work items), sorts them by estimated cost (largest first),
  * uploads all descriptors once and captures the launches -- a reset of the
  * queue heads and, per kind of item, a grid of resident CTAs that pull items
- * with an atomic counter -- in a CUDA graph; ec_batch_run replays that graph.  Results are bit-identical to
- * calling ec_composite_depth / ec_composite_alpha per job, whatever the tile
- * shapes. */
+ * with an atomic counter -- in a CUDA graph; ec_batch_run replays that graph.
+ * The jobs run in no order: none may read or write another one's destination.
+ * Results are bit-identical to calling ec_composite_depth / ec_composite_alpha
+ * per job, whatever the tile shapes. */
 enum { EC_JOB_DEPTH = 0, EC_JOB_ALPHA = 1 };
 #define EC_MAX_BATCH_INPUTS 128     /* inputs per job of a batch              */
 
